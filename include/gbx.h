@@ -98,7 +98,7 @@ typedef struct {
     int algorithm;          /* GBX_ALG_*                                              */
     int levels;             /* dependent kernel phases per start (1 or 3)             */
     int launches;           /* kernels per start                                      */
-    int use_graph;          /* 1 if start replays a captured CUDA graph               */
+    int use_graph;          /* the graph= setting (see gbx_neighbor_alltoallv_init)    */
     int vec_bytes;          /* vector width of the dominant move kernel               */
     int block;              /* threads per block of the dominant move kernel          */
     int unroll;             /* chunks per thread per tile of the dominant kernel      */
@@ -195,7 +195,11 @@ int gbx_graph_free(gbx_graph_t *graph);
  *   info: "key=value;..." with
  *       algorithm=standard|locality|auto   (default standard; auto times both and keeps
  *                                          the faster)
- *       graph=0|1          capture the start sequence in a CUDA graph (default 1)
+ *       graph=0|1          1 (default): a start of several launches replays a CUDA graph
+ *                          captured at init (until a rebind; then, and for a single launch,
+ *                          the kernels are launched with their descriptors as arguments);
+ *                          such a start cannot be captured by the caller (GBX_ERR_CUDA).
+ *                          0: plain launches that read descriptors in device memory
  *       autotune=0|1       time candidate kernel shapes at init (default 1)
  *       vec=V block=B      force the move kernel's vector width / block size
  *       min_run=N          gathered runs of >= N consecutive source elements are copied as
@@ -455,9 +459,11 @@ int gbx_waitall(int count, gbx_request_t *requests);
  * ones; one aligned below the vector width a move program of the request was tuned to
  * gives GBX_ERR_ARG (the old binding stays).  Batches of gbx_startall that hold their own
  * wider copies of the request's programs move them to the new buffers, and a batch whose
- * copies the new buffers no longer align is rebuilt at its next gbx_startall.  The new
- * descriptors are uploaded on the request's stream; a request that belongs to a cached
- * batch (which may run on another request's stream) synchronises that stream first. */
+ * copies the new buffers no longer align is rebuilt at its next gbx_startall.  The next
+ * start takes the new buffers as launch arguments; only where launches read descriptors in
+ * device memory (graph=0, cached batches, several ops pooled in one launch) are those
+ * rewritten, on the request's stream, and a request that belongs to a cached batch (which may
+ * run on another request's stream) synchronises that stream. */
 int gbx_request_bind(gbx_request_t request, const void *src, void *dst);
 
 /* One exchange on HOST buffers: copies host_src (the whole bound source buffer, pinned

@@ -39,7 +39,7 @@ class DistributedHalo:
         self.dp = DevicePattern(p, device)
         self.fwd = Exchange(p, x, h, algorithm=algorithm, info=info, dp=self.dp)
         gh = torch.zeros(self.n_recv, dtype=self.dtype, device=device)
-        gx = torch.zeros(self.n_send, dtype=self.dtype, device=device)
+        self._gx0 = gx = torch.zeros(self.n_send, dtype=self.dtype, device=device)
         self.bwd = backward_init(self.fwd.request, gh, gx, accumulate=False, info=info)
         assert DTYPE_CODES[p.dtype] in (1, 2)
         # Outputs are fresh tensors every call (autograd may hold several at once), but only
@@ -64,6 +64,9 @@ class DistributedHalo:
         self.bwd.bind(g, gx)
         self.bwd.start()
         self.bwd.wait_stream()
+        # the request lets go of the gradient (bound to its own buffer again, whose bytes nobody
+        # reads): autograd then takes gx as it is where it would copy a tensor held elsewhere
+        self.bwd.bind(None, self._gx0)
         return gx
 
     def __call__(self, x: torch.Tensor) -> torch.Tensor:

@@ -20,7 +20,10 @@ struct Batch {
     std::vector<HostOp> widened;   // batch-owned copies of ops re-cut to their widest vector
     std::vector<std::pair<gbx_request_s *, size_t>> widened_of;   // (request, op index) of each
     cudaGraphExec_t exec = nullptr;
-    cudaEvent_t done = nullptr;
+    cudaEvent_t done = nullptr;   // end of the last start, recorded on `on`
+    cudaStream_t on = nullptr;
+    int done_timed = 0, other_streams = 0;   // see done_event_for_other_streams
+    int finished = 0;             // the last start's end has been seen: its members need not ask again
 };
 
 extern "C" const char *gbx_error_string(int code) {
@@ -250,8 +253,6 @@ int gbx_make_copy_op(gbx_request_s *req, int level, const char *src, int src_rol
     GBX_TRY(req->mem.get(&op.d_tile_seg, max_tiles + 1));
     GBX_TRY(req->mem.get(&op.d_tile_e0, max_tiles + 1));
     GBX_TRY(req->mem.alloc(&op.d_desc, sizeof(CopyDesc)));
-    GBX_TRY(req->mem.get(&op.d_self, 1));
-    GBX_TRY(req->mem.get(&op.d_self_prefix, 2));
     d.tile_seg = op.d_tile_seg;
     d.tile_e0 = op.d_tile_e0;
     if (req->allow_flat) {
@@ -302,8 +303,6 @@ int gbx_make_flat_op(gbx_request_s *req, int level, const char *src, int src_rol
     GBX_TRY(req->mem.get(&op.d_tile_e0, max_tiles + 1));
     d.tile_e0 = op.d_tile_e0;
     GBX_TRY(req->mem.alloc(&op.d_desc, sizeof(CopyDesc)));
-    GBX_TRY(req->mem.get(&op.d_self, 1));
-    GBX_TRY(req->mem.get(&op.d_self_prefix, 2));
     req->ops.push_back(op);
     return GBX_SUCCESS;
 }
@@ -395,8 +394,6 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
         }
     }
     GBX_TRY(req->mem.alloc(&op.d_desc, sizeof(FoldDesc)));
-    GBX_TRY(req->mem.get(&op.d_self, 1));
-    GBX_TRY(req->mem.get(&op.d_self_prefix, 2));
     req->ops.push_back(op);
     return GBX_SUCCESS;
 }
@@ -441,10 +438,6 @@ static int set_vec(gbx_request_s *req, HostOp &op, int vec) {
         GBX_TRY(gbx_build_tile_meta(nullptr, 0, cpe, d.ntiles, nullptr, op.d_tile_e0, req->stream));
     }
     GBX_TRY(upload_desc(req, op));
-    void *self = op.d_desc;
-    int64_t pre[2] = {0, op_tiles(op)};
-    GBX_CUDA_TRY(cudaMemcpyAsync(op.d_self, &self, sizeof(void *), cudaMemcpyHostToDevice, req->stream));
-    GBX_CUDA_TRY(cudaMemcpyAsync(op.d_self_prefix, pre, sizeof(pre), cudaMemcpyHostToDevice, req->stream));
     GBX_CUDA_TRY(cudaStreamSynchronize(req->stream));
     return GBX_SUCCESS;
 }
@@ -463,25 +456,33 @@ static int grid_for(int kind, int dtype, int vec, int flat, int block, int persi
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, tiles));
 }
 
-// one: every op of the launch has one chunk per element (the stream forms then run their
-// specialised kernel, launch codes 12 / 13)
-static cudaError_t launch_list(int kind, int dtype, int vec, int flat, void **d_ops, int64_t *d_prefix, int nops,
-                               int64_t tiles, int block, int grid, cudaStream_t st, int one = 0) {
-    if (kind == 0)
-        return gbx_launch_copy((const CopyDesc *const *)d_ops, d_prefix, nops, tiles, vec,
-                               (flat == 10 || flat == 11) && one ? flat + 2 : flat, block, grid, st);
-    return gbx_launch_fold((const FoldDesc *const *)d_ops, d_prefix, nops, tiles, dtype, vec, block, grid, st, flat);
-}
-
 // a copy's form, or a fold's (0 the fold kernel, 1 its stream form)
 static int op_flat(const HostOp &op) { return op.kind == 0 ? op.cd.flat : op.fold_form; }
 
+// Launch code of a copy form: the stream forms run their specialised kernel (codes 12 / 13) when
+// every op of the launch has one chunk per element (one).
+static int launch_code(int flat, int one) { return (flat == 10 || flat == 11) && one ? flat + 2 : flat; }
+
 static cudaError_t launch_op_alone(gbx_request_s *req, HostOp &op, int block, int persistent) {
-    int64_t tiles = op_tiles(op);
+    const int64_t tiles = op_tiles(op);
     const int vec = op_vec(op), flat = op_flat(op);
-    return launch_list(op.kind, req->dtype, vec, flat, op.d_self, op.d_self_prefix, 1, tiles, block,
-                       grid_for(op.kind, req->dtype, vec, flat, block, persistent, tiles, req->max_ctas), req->stream,
-                       op.kind == 0 && op.cd.cpe == 1);
+    const int grid = grid_for(op.kind, req->dtype, vec, flat, block, persistent, tiles, req->max_ctas);
+    if (op.kind == 0)
+        return gbx_launch_copy({&op.cd, nullptr, nullptr, 1, tiles}, vec, launch_code(flat, op.cd.cpe == 1), block, grid,
+                               req->stream, false);
+    return gbx_launch_fold({&op.fd, nullptr, nullptr, 1, tiles}, req->dtype, vec, block, grid, req->stream, flat, false);
+}
+
+// A level's launch in form `flat`, `block` and `grid`; ops: the request's ops, for launches of one
+// op passed by value (null: every launch reads its device descriptor list).
+static cudaError_t launch_level(const LevelLaunch &L, const std::vector<HostOp> *ops, int flat, int block, int grid,
+                                cudaStream_t st, bool dep) {
+    const HostOp *op = ops && L.one_op >= 0 ? &(*ops)[L.one_op] : nullptr;
+    if (L.kind == 0)
+        return gbx_launch_copy({op ? &op->cd : nullptr, (const CopyDesc *const *)L.d_ops, L.d_prefix, L.nops, L.total_tiles},
+                               L.vec, launch_code(flat, L.one), block, grid, st, dep);
+    return gbx_launch_fold({op ? &op->fd : nullptr, (const FoldDesc *const *)L.d_ops, L.d_prefix, L.nops, L.total_tiles},
+                           L.dtype, L.vec, block, grid, st, flat, dep);
 }
 
 // ------------------------------------------------------------------ autotuner
@@ -649,7 +650,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
 // One launch per (level, kind, class): a class is (form, vector width) for copies and
 // (payload type, vector width) for folds, so every launch runs a specialised kernel.  For a
 // batch the ops of all its requests are pooled, so each launch covers every pattern of its
-// class (the generic width-dispatching kernels stay available but are not needed).
+// class.
 // Times a pooled launch in every block size and grid mode with CUDA events and keeps the
 // fastest (the moved bytes do not depend on the shape).
 static int tune_launch(LevelLaunch &L, cudaStream_t st) {
@@ -667,15 +668,13 @@ static int tune_launch(LevelLaunch &L, cudaStream_t st) {
         const bool strm = fl >= 10;
         for (int bi = strm ? (L.one && L.vec <= 8 ? 0 : 1) : 0; bi < (strm ? 3 : 4) && e == cudaSuccess; bi++)
             for (int pers = 1; pers >= (strm ? 1 : 0) && e == cudaSuccess; pers--) {
-                const int blk = gbx_effective_block(L.vec, blocks[bi]);
+                const int blk = blocks[bi];
                 const int grid = grid_for(L.kind, L.dtype, L.vec, fl, blk, pers, L.total_tiles, L.max_ctas);
-                e = launch_list(L.kind, L.dtype, L.vec, fl, L.d_ops, L.d_prefix, L.nops, L.total_tiles, blk, grid, st,
-                                L.one);
+                e = launch_level(L, nullptr, fl, blk, grid, st, false);
                 float t = 1e30f;
                 for (int r = 0; r < 3 && e == cudaSuccess; r++) {
                     cudaEventRecord(a, st);
-                    e = launch_list(L.kind, L.dtype, L.vec, fl, L.d_ops, L.d_prefix, L.nops, L.total_tiles, blk,
-                                    grid, st, L.one);
+                    e = launch_level(L, nullptr, fl, blk, grid, st, false);
                     cudaEventRecord(b, st);
                     if (e == cudaSuccess) e = cudaEventSynchronize(b);
                     float x = 0;
@@ -754,20 +753,13 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
                 LevelLaunch L;
                 L.kind = kind;
                 L.nops = (int)groups[g].size();
-                // common payload type, vector width and form, or 0 / 2 (= mixed)
-                int dt = dtypes[groups[g][0]], vec = op_vec(*ops[groups[g][0]]);
+                // (folds: the payload type is part of the class, copies do not read it)
+                L.dtype = dtypes[groups[g][0]];
+                L.vec = op_vec(*ops[groups[g][0]]);
                 // (a pooled class of one op keeps the form it was tuned to, pipelined included)
-                int fl = kind ? ops[groups[g][0]]->fold_form
+                L.flat = kind ? ops[groups[g][0]]->fold_form
                               : (groups[g].size() == 1 ? op_flat(*ops[groups[g][0]]) : keys[g].first & 15);
-                for (size_t i : groups[g]) {
-                    if (dtypes[i] != dt) dt = -1;
-                    if (op_vec(*ops[i]) != vec) vec = 0;
-                    if (!batch && op_flat(*ops[i]) != fl) fl = 2;
-                }
-                if (dt < 0 && kind == 1) vec = 0;
-                L.dtype = dt < 0 ? GBX_F32 : dt;
-                L.vec = vec;
-                L.flat = vec == 0 ? 2 : fl;
+                L.one_op = !batch && groups[g].size() == 1 ? (int)groups[g][0] : -1;
                 L.one = 1;
                 for (size_t i : groups[g])
                     if (kind != 0 || ops[i]->cd.cpe != 1) L.one = 0;
@@ -782,7 +774,7 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
                 L.total_tiles = pre.back();
                 L.phase = phase_name(batch ? 3 : what, lv, kind);
                 // the launch takes the tuned shape of its largest op
-                L.block = gbx_effective_block(L.vec, big->block);
+                L.block = big->block;
                 L.max_ctas = max_ctas;
                 L.grid = grid_for(kind, L.dtype, L.vec, L.flat, L.block, big->persistent, L.total_tiles, max_ctas);
                 GBX_TRY(mem.get(&L.d_ops, L.nops));
@@ -801,23 +793,25 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
     return GBX_SUCCESS;
 }
 
-static cudaError_t enqueue_levels(const std::vector<LevelLaunch> &levels, cudaStream_t st) {
+static cudaError_t enqueue_levels(const std::vector<LevelLaunch> &levels, const std::vector<HostOp> *ops,
+                                  cudaStream_t st) {
+    bool dep = false;   // the first launch follows the stream's earlier work, the others their predecessor
     for (const LevelLaunch &L : levels) {
         GbxRange r(L.phase);
-        cudaError_t e = launch_list(L.kind, L.dtype, L.vec, L.flat, L.d_ops, L.d_prefix, L.nops, L.total_tiles,
-                                    L.block, L.grid, st, L.one);
+        cudaError_t e = launch_level(L, ops, L.flat, L.block, L.grid, st, dep);
         if (e != cudaSuccess) return e;
+        dep = true;
     }
     return cudaSuccess;
 }
 
-static int capture(const std::vector<LevelLaunch> &levels, cudaGraphExec_t *exec) {
+static int capture(const std::vector<LevelLaunch> &levels, const std::vector<HostOp> *ops, cudaGraphExec_t *exec) {
     cudaStream_t cs;
     GBX_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t e2 = enqueue_levels(levels, cs);
+        cudaError_t e2 = enqueue_levels(levels, ops, cs);
         e = cudaStreamEndCapture(cs, &graph);
         if (e == cudaSuccess) e = e2;
     }
@@ -873,7 +867,8 @@ static int finalize(gbx_request_s *req) {
     for (HostOp &op : req->ops) { ptrs.push_back(&op); dts.push_back(req->dtype); }
     const int what = req->kind == 1 ? 2 : req->algorithm == GBX_ALG_LOCALITY ? 1 : 0;
     GBX_TRY(build_levels(req->mem, ptrs, dts, req->launches, 0, req->stream, 0, req->max_ctas, what));
-    if (req->use_graph && !req->launches.empty()) GBX_TRY(capture(req->launches, &req->exec));
+    // a single launch goes out directly; several are replayed as one graph until a rebind
+    if (req->use_graph && req->launches.size() > 1) GBX_TRY(capture(req->launches, &req->ops, &req->exec));
     fill_info(req);
     return GBX_SUCCESS;
 }
@@ -882,7 +877,7 @@ static void destroy_batch(Batch *b) {
     for (gbx_request_s *m : b->members) {
         auto &v = m->batches;
         v.erase(std::remove(v.begin(), v.end(), b), v.end());
-        if (m->pending == &b->done) {
+        if (m->pending == b) {
             cudaEventSynchronize(b->done);
             m->pending = nullptr;
             m->active = 0;
@@ -905,8 +900,7 @@ static void destroy_request(gbx_request_s *req) {
         req->active = 0;
     }
     if (req->active) {
-        cudaEvent_t ev = req->pending ? *req->pending : req->done;
-        cudaEventSynchronize(ev);
+        cudaEventSynchronize(req->pending ? req->pending->done : req->done);
     }
     while (!req->batches.empty()) destroy_batch(req->batches.back());
     if (req->host_down_pending) cudaEventSynchronize(req->host_down_ev);
@@ -928,6 +922,22 @@ static void destroy_request(gbx_request_s *req) {
 // waiting on a disable-timing event held back the work queued behind the wait (an early-bird
 // exchange of 8 partitions took 2.99 ms against 2.47 ms with timing-enabled events).
 static cudaError_t gbx_event_create(cudaEvent_t *ev) { return cudaEventCreateWithFlags(ev, cudaEventDefault); }
+
+// The event a start records for gbx_wait / gbx_test has timing off: recording one with timing
+// takes 2.1 us of the stream and 2.6 us of the host (start + wait of a 3 us kernel: 13.2 against
+// 10.0 us).  A request or batch that another stream has waited on once gets an event with timing
+// for its later starts (above).
+static cudaError_t done_event_create(cudaEvent_t *ev) { return cudaEventCreateWithFlags(ev, cudaEventDisableTiming); }
+
+static int done_event_for_other_streams(cudaEvent_t *done, int *timed) {
+    if (*timed) return GBX_SUCCESS;
+    cudaEvent_t ev;
+    GBX_CUDA_TRY(gbx_event_create(&ev));
+    cudaEventDestroy(*done);   // (waits already enqueued on it keep it until they are done)
+    *done = ev;
+    *timed = 1;
+    return GBX_SUCCESS;
+}
 
 static gbx_request_s *new_request(const Opts &o, void *stream) {
     gbx_request_s *req = new gbx_request_s();
@@ -951,7 +961,7 @@ static gbx_request_s *new_request(const Opts &o, void *stream) {
     req->wait_limit = o.wait_limit;
     req->allow_stream = o.stream;
     req->forced_form = o.form;
-    if (gbx_event_create(&req->done) != cudaSuccess) {
+    if (done_event_create(&req->done) != cudaSuccess) {
         cudaGetLastError();
         req->done = nullptr;
     }
@@ -974,11 +984,11 @@ static float program_ms(gbx_request_s *req) {
     // time of one eager pass over the levels (used by algorithm=auto)
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return 1e30f;
-    enqueue_levels(req->launches, req->stream);
+    enqueue_levels(req->launches, &req->ops, req->stream);
     float best = 1e30f;
     for (int r = 0; r < 3; r++) {
         cudaEventRecord(a, req->stream);
-        enqueue_levels(req->launches, req->stream);
+        enqueue_levels(req->launches, &req->ops, req->stream);
         cudaEventRecord(b, req->stream);
         cudaEventSynchronize(b);
         float t = 0;
@@ -1174,16 +1184,31 @@ extern "C" int gbx_partitioned_init(gbx_request_t forward, int npart, const int6
     return GBX_SUCCESS;
 }
 
+// The request's kernels on `st`.  graph=1: one launch with its descriptor by value, or the graph
+// captured at init, or after a rebind the launches one by one; none of these may be captured
+// into a caller's graph, whose replays would keep the buffers bound now.  graph=0: launches that
+// read the descriptors in device memory, which a rebind rewrites, so that they can be.
+static int launch_program(gbx_request_s *req, cudaStream_t st) {
+    if (!req->use_graph) {
+        GBX_CUDA_TRY(enqueue_levels(req->launches, nullptr, st));
+    } else if (req->exec) {
+        GBX_CUDA_TRY(cudaGraphLaunch(req->exec, st));
+    } else if (!req->launches.empty()) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        GBX_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return GBX_ERR_CUDA;
+        GBX_CUDA_TRY(enqueue_levels(req->launches, &req->ops, st));
+    }
+    return GBX_SUCCESS;
+}
+
 extern "C" int gbx_pready(gbx_request_t req, int p, void *stream) {
     if (!req || req->kind != 2 || p < 0 || p >= req->npart) return GBX_ERR_ARG;
     GbxRange range("gbx.pready");
     if (!req->active || req->part_ready[p]) return GBX_ERR_STATE;
     cudaStream_t st = stream ? (cudaStream_t)stream : req->stream;
     gbx_request_s *c = req->parts[p];
-    if (c) {
-        if (c->use_graph && c->exec) GBX_CUDA_TRY(cudaGraphLaunch(c->exec, st));
-        else GBX_CUDA_TRY(enqueue_levels(c->launches, st));
-    }
+    if (c) GBX_TRY(launch_program(c, st));
     GBX_CUDA_TRY(cudaEventRecord(req->part_ev[p], st));
     req->part_ready[p] = 1;
     req->nready++;
@@ -1262,12 +1287,9 @@ static int enqueue_start(gbx_request_s *req) {
                    : req->algorithm == GBX_ALG_LOCALITY ? "gbx.start.locality" : "gbx.start.standard");
     // the exchange overwrites the bound destination: it follows the last host read-back of it
     if (req->host_down_pending) GBX_CUDA_TRY(cudaStreamWaitEvent(req->stream, req->host_down_ev, 0));
-    if (req->use_graph && req->exec) {
-        GBX_CUDA_TRY(cudaGraphLaunch(req->exec, req->stream));
-    } else {
-        GBX_CUDA_TRY(enqueue_levels(req->launches, req->stream));
-    }
+    GBX_TRY(launch_program(req, req->stream));
     GBX_CUDA_TRY(cudaEventRecord(req->done, req->stream));
+    req->done_on = req->stream;
     req->pending = nullptr;
     req->active = 1;
     return GBX_SUCCESS;
@@ -1285,7 +1307,7 @@ extern "C" int gbx_start(gbx_request_t req) {
     return enqueue_start(req);
 }
 
-static cudaEvent_t pending_event(gbx_request_s *req) { return req->pending ? *req->pending : req->done; }
+static cudaEvent_t pending_event(gbx_request_s *req) { return req->pending ? req->pending->done : req->done; }
 
 // partitioned: 1 when every marked partition's moves are done (0 if still running)
 static int parts_done(gbx_request_s *req, int *flag) {
@@ -1325,7 +1347,9 @@ extern "C" int gbx_test(gbx_request_t req, int *flag) {
             if (c && take_status(c) != GBX_SUCCESS) rc = GBX_ERR_DEVICE_WAIT;
         return rc;
     }
-    cudaError_t e = cudaEventQuery(pending_event(req));
+    Batch *b = req->pending;
+    cudaError_t e = b && b->finished ? cudaSuccess : cudaEventQuery(pending_event(req));
+    if (b && e == cudaSuccess) b->finished = 1;   // (each further query takes a microsecond: 16 members, 13 us)
     if (e == cudaErrorNotReady) { *flag = 0; return GBX_SUCCESS; }
     if (e != cudaSuccess) {
         gbx_note_cuda_error(e, "event query", __FILE__, __LINE__);
@@ -1366,7 +1390,13 @@ extern "C" int gbx_wait_stream(gbx_request_t req, void *stream) {
         req->active = 0;
         return GBX_SUCCESS;
     }
-    GBX_CUDA_TRY(cudaStreamWaitEvent((cudaStream_t)stream, pending_event(req), 0));
+    // (a stream is ordered after its own work; the per-thread handle names a stream per thread)
+    Batch *b = req->pending;
+    if ((cudaStream_t)stream != (b ? b->on : req->done_on) || (cudaStream_t)stream == cudaStreamPerThread) {
+        GBX_CUDA_TRY(cudaStreamWaitEvent((cudaStream_t)stream, pending_event(req), 0));
+        if (!b) GBX_TRY(done_event_for_other_streams(&req->done, &req->done_timed));
+        else b->other_streams = 1;   // (other members may still wait on this start's event)
+    }
     req->active = 0;
     req->pending = nullptr;
     return GBX_SUCCESS;
@@ -1437,6 +1467,13 @@ extern "C" int gbx_startall(int count, gbx_request_t *reqs) {
         std::vector<int> dts;
         int rc0 = GBX_SUCCESS;
         size_t nwide = 0;
+        for (gbx_request_s *r : key)   // the pooled launches read the device descriptors
+            if (r->desc_stale) {
+                for (HostOp &op : r->ops)
+                    if (rc0 == GBX_SUCCESS) rc0 = upload_desc(r, op);
+                if (rc0 == GBX_SUCCESS && cudaStreamSynchronize(r->stream) != cudaSuccess) rc0 = GBX_ERR_CUDA;
+                r->desc_stale = rc0 != GBX_SUCCESS;
+            }
         for (gbx_request_s *r : key)
             for (HostOp &op : r->ops) nwide += widen_candidate(op);
         b->widened.reserve(nwide);   // stable addresses for the pointers below
@@ -1462,9 +1499,9 @@ extern "C" int gbx_startall(int count, gbx_request_t *reqs) {
             if (r->max_ctas > 0) cap = cap > 0 ? std::min(cap, r->max_ctas) : r->max_ctas;
         }
         int rc = build_levels(b->mem, ops, dts, b->launches, 1, st, tune, cap);
-        if (rc == GBX_SUCCESS && gbx_event_create(&b->done) != cudaSuccess)
+        if (rc == GBX_SUCCESS && done_event_create(&b->done) != cudaSuccess)
             rc = GBX_ERR_CUDA;
-        if (rc == GBX_SUCCESS && !b->launches.empty()) rc = capture(b->launches, &b->exec);
+        if (rc == GBX_SUCCESS && !b->launches.empty()) rc = capture(b->launches, nullptr, &b->exec);
         if (rc != GBX_SUCCESS) {
             if (b->exec) cudaGraphExecDestroy(b->exec);
             if (b->done) cudaEventDestroy(b->done);
@@ -1475,10 +1512,13 @@ extern "C" int gbx_startall(int count, gbx_request_t *reqs) {
     }
     cudaStream_t st = reqs[0]->stream;
     if (b->exec) GBX_CUDA_TRY(cudaGraphLaunch(b->exec, st));
+    if (b->other_streams) GBX_TRY(done_event_for_other_streams(&b->done, &b->done_timed));
     GBX_CUDA_TRY(cudaEventRecord(b->done, st));
+    b->on = st;
+    b->finished = 0;
     for (gbx_request_s *r : key) {
         r->active = 1;
-        r->pending = &b->done;
+        r->pending = b;
     }
     return GBX_SUCCESS;
 }
@@ -1515,7 +1555,20 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
             if (op.fd.out_role == ROLE_DST) op.fd.out = nd;
             if (op.fd.a_role == ROLE_SRC) op.fd.bufA = ns;
         }
-        GBX_TRY(upload_desc(req, op));
+    }
+    // launches of one op take the new descriptor with their next start; the device descriptors
+    // are rewritten only where a launch reads them
+    bool lists = !req->use_graph || !req->batches.empty();
+    for (const LevelLaunch &L : req->launches) lists |= L.one_op < 0;
+    if (lists) {
+        for (HostOp &op : req->ops) GBX_TRY(upload_desc(req, op));
+        req->desc_stale = 0;
+    } else {
+        req->desc_stale = 1;
+    }
+    if (req->exec && (ns != req->src || nd != req->dst)) {   // (a running replay keeps it until it ends)
+        cudaGraphExecDestroy(req->exec);
+        req->exec = nullptr;
     }
     req->src = ns;
     req->dst = nd;
@@ -1558,6 +1611,7 @@ extern "C" int gbx_start_host_async(gbx_request_t req, const void *host_src, voi
     if (req->kind == 2) return GBX_ERR_UNSUPPORTED;
     if (req->active) return GBX_ERR_ACTIVE;
     GBX_TRY(host_streams(req));
+    GBX_TRY(done_event_for_other_streams(&req->done, &req->done_timed));
     if (host_src && req->src_bytes > 0) {
         // the upload overwrites the bound source: it follows everything already queued on the
         // request's stream (earlier exchanges that read the source)
@@ -1574,6 +1628,7 @@ extern "C" int gbx_start_host_async(gbx_request_t req, const void *host_src, voi
         GBX_CUDA_TRY(cudaMemcpyAsync(host_dst, req->dst, req->dst_bytes, cudaMemcpyDefault, req->host_down));
         GBX_CUDA_TRY(cudaEventRecord(req->host_down_ev, req->host_down));
         GBX_CUDA_TRY(cudaEventRecord(req->done, req->host_down));   // complete once read back
+        req->done_on = req->host_down;
         req->host_down_pending = 1;
     }
     return GBX_SUCCESS;

@@ -82,19 +82,25 @@ int gbx_iota_i64(int64_t *p, int64_t n, cudaStream_t st);
 int gbx_read_i64(const int64_t *d, int64_t *h, cudaStream_t st);
 
 // ------------------------------------------------------------------ move kernels
-// Kernels are specialised per vector width (copy) or (payload type, vector width)
-// (fold); vec == 0 selects the generic kernel that dispatches per tile, used when one
-// launch mixes ops of different widths (batched patterns).
+// Kernels are specialised per vector width and form (copy) or payload type and vector width
+// (fold).
 int gbx_num_sms(void);
-int gbx_effective_block(int vec, int block);
 int gbx_occupancy(int kind, int dtype, int vec, int block, int flat);   // resident blocks per SM
-// flat: 0 every op in segment form, 1 every op in flat form, 2 decided per op
-cudaError_t gbx_launch_copy(const CopyDesc *const *ops, const int64_t *tile_prefix, int nops,
-                            int64_t total_tiles, int vec, int flat, int block, int grid, cudaStream_t st);
+// The ops of a launch: one op by its descriptor's value (one != null), or a list of nops
+// descriptors in device memory with their tile prefix.
+template <typename D>
+struct OpRef {
+    const D *one;
+    const D *const *ops;
+    const int64_t *prefix;
+    int nops;
+    int64_t ntiles;
+};
+// dep: a launch after another one of the same start, which it depends on
+cudaError_t gbx_launch_copy(const OpRef<CopyDesc> &r, int vec, int flat, int block, int grid, cudaStream_t st, bool dep);
 // form 0: the fold kernel; 1: its stream form (records and terms staged in shared memory)
-cudaError_t gbx_launch_fold(const FoldDesc *const *ops, const int64_t *tile_prefix, int nops,
-                            int64_t total_tiles, int dtype, int vec, int block, int grid,
-                            cudaStream_t st, int form);
+cudaError_t gbx_launch_fold(const OpRef<FoldDesc> &r, int dtype, int vec, int block, int grid, cudaStream_t st, int form,
+                            bool dep);
 int gbx_sfold_prepare(void);
 // Per-tile metadata: first unit (element / row) of each tile and, for copy ops, the
 // segment holding it (segs may be NULL for fold ops).
@@ -154,16 +160,14 @@ struct HostOp {
     ScatterPiece *d_scat;
     int64_t nscat;
     int64_t algo_bytes_scat;
-    void **d_self;          // one-entry descriptor list for launching the op alone
-    int64_t *d_self_prefix; // {0, ntiles}
 };
 
 // One kernel launch of a level.
 struct LevelLaunch {
     int kind;
     int dtype;              // fold: payload type
-    int vec;                // vector width of every op, or 0 when they differ
-    int flat;               // copy: 0 / 1 when every op uses the segment / flat form, 2 mixed
+    int vec;                // vector width of every op
+    int flat;               // copy: the form of every op; fold: 0, or 1 for the stream form
     int block;
     int grid;
     int nops;
@@ -171,6 +175,8 @@ struct LevelLaunch {
     int max_ctas;           // grid cap (0: none)
     const char *phase;      // NVTX name of the launch (a string literal)
     int one;                // copies: every op has one chunk per element (stream kernels specialise)
+    int one_op;             // index of the launch's only op in its request, whose descriptor is passed by
+                            // value; -1: pooled ops (and batches), read from d_ops
     void **d_ops;           // device array of descriptor pointers
     int64_t *d_prefix;      // device tile prefix (nops + 1)
 };
@@ -205,8 +211,10 @@ struct gbx_request_s {
     gbx_request_s *forward;  // backward: its forward request
     gbx_graph_s *owned_graph;  // graph built for this request (dense all-to-all-v), freed with it
     cudaStream_t stream;
-    cudaEvent_t done;
-    cudaEvent_t *pending;    // event to wait on while active (own or a batch's)
+    cudaEvent_t done;        // end of the last start, recorded on done_on
+    cudaStream_t done_on;
+    int done_timed;          // `done` has timing enabled (see done_event_for_other_streams)
+    Batch *pending;          // the batch whose start this request is part of, while active
     int active;
     // host-buffer starts: the request's own copy streams (upload, download), the event the
     // upload records, and the event of the last download (the next exchange waits for it)
@@ -221,7 +229,8 @@ struct gbx_request_s {
     DevPool mem;             // everything the request owns
     std::vector<HostOp> ops;
     std::vector<LevelLaunch> launches;
-    cudaGraphExec_t exec;
+    cudaGraphExec_t exec;    // several launches: the start sequence over the buffers bound at init
+    int desc_stale;          // the device descriptors lack the last rebind (no launch reads them)
     gbx_request_info_t info;
     // maps kept for building the backward of this (forward) request
     int64_t nseg;            // standard segments (nonzero edges) in receive order

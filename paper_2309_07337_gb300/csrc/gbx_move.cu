@@ -18,6 +18,16 @@
 // consecutive chunks: destination writes are fully coalesced 16-byte stores, source
 // reads are 16-byte vector gathers of whole elements.  No shared memory, no barriers,
 // no waits: a launch always terminates.
+//
+// Every kernel takes its ops in one of two ways (template parameter L).  A launch of one op
+// carries the op's descriptor by value (OneOp, read from the constant bank): no load of a
+// descriptor pointer and then of its fields stands between the start of the kernel and its
+// first index load, and a rebind only changes the next launch's argument.  A pooled launch
+// (OpList, the batches) reads a list of descriptors in device memory.  Measured together with
+// dependent launches and untimed events (start + wait, before and after): 3,072 8-byte points
+// 13.7 -> 11.8 us, a 3-launch locality exchange of 78 k 24-byte points 20.3 -> 14.1, 2.6 M 24-byte
+// records 46.6 -> 35.0, 1.7 M 8-byte values under datatypes 22.6 -> 16.8, 2^20-row SpMV halo fp64
+// 41.1 -> 39.0, forward + backward of the fp32 one through autograd 230 -> 196.
 #include "gbx_internal.cuh"
 
 template <int VEC> struct VecT;
@@ -27,48 +37,16 @@ template <> struct VecT<4> { typedef unsigned int T; };
 template <> struct VecT<2> { typedef unsigned short T; };
 template <> struct VecT<1> { typedef unsigned char T; };
 
-// Cache behaviour of the payload loads and stores (index and descriptor loads always go
-// through L1).  GBX_LD_MODE 0: ld.global.nc; 1: + L1::no_allocate; 2: + L1::no_allocate and
-// an L2 256-byte prefetch.  GBX_ST_MODE 0: st.global; 1: st.global.cs (evict first).
-#ifndef GBX_LD_MODE
-#define GBX_LD_MODE 0
-#endif
-#ifndef GBX_ST_MODE
-#define GBX_ST_MODE 0
-#endif
-
+// Payload loads are plain ld.global: within a chain of dependent launches the payload may be
+// written (by the launch before) after this kernel has started, which the non-coherent path does
+// not allow for.  Indices and descriptors, fixed at init, use it.  (The two run equally fast
+// here, and so did L1::no_allocate, L2 prefetch hints and evict-first stores.)
 template <int VEC>
 __device__ __forceinline__ typename VecT<VEC>::T ldv(const char *p) {
-#if GBX_LD_MODE == 0
-    return __ldg(reinterpret_cast<const typename VecT<VEC>::T *>(p));
-#else
-    if constexpr (VEC == 16) {
-        uint4 v;
-#if GBX_LD_MODE == 1
-        asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-            : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-#else
-        asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
-            : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-#endif
-        return v;
-    } else {
-        return __ldg(reinterpret_cast<const typename VecT<VEC>::T *>(p));
-    }
-#endif
-}
-template <int VEC>
-__device__ __forceinline__ typename VecT<VEC>::T ldv_plain(const char *p) {
     return *reinterpret_cast<const typename VecT<VEC>::T *>(p);
 }
 template <int VEC>
 __device__ __forceinline__ void stv(char *p, typename VecT<VEC>::T v) {
-#if GBX_ST_MODE == 1
-    if constexpr (VEC == 16) {
-        __stcs(reinterpret_cast<uint4 *>(p), v);
-        return;
-    }
-#endif
     *reinterpret_cast<typename VecT<VEC>::T *>(p) = v;
 }
 
@@ -80,6 +58,63 @@ __device__ __forceinline__ int find_op(const int64_t *__restrict__ prefix, int n
         if (__ldg(prefix + mid) <= t) lo = mid; else hi = mid - 1;
     }
     return lo;
+}
+
+template <typename D>
+struct OneOp {
+    static constexpr bool single = true;
+    D d;
+    int64_t ntiles;
+    __device__ __forceinline__ int64_t tiles() const { return ntiles; }
+    __device__ __forceinline__ const D *first() const { return &d; }
+    __device__ __forceinline__ const D *at(int64_t t, int64_t &lt) const {
+        lt = t;
+        return &d;
+    }
+    __device__ __forceinline__ int count() const { return 1; }
+    __device__ __forceinline__ const D *op(int) const { return &d; }
+};
+
+template <typename D>
+struct OpList {
+    static constexpr bool single = false;
+    const D *const *ops;
+    const int64_t *prefix;
+    int nops;
+    int64_t ntiles;
+    __device__ __forceinline__ int64_t tiles() const { return ntiles; }
+    __device__ __forceinline__ const D *first() const { return ops[0]; }
+    // the op whose tiles hold tile t of the launch, and the tile's number in that op
+    __device__ __forceinline__ const D *at(int64_t t, int64_t &lt) const {
+        const int op = nops > 1 ? find_op(prefix, nops, t) : 0;
+        lt = t - __ldg(prefix + op);
+        return ops[op];
+    }
+    __device__ __forceinline__ int count() const { return nops; }
+    __device__ __forceinline__ const D *op(int i) const { return ops[i]; }
+};
+
+// The launches of one request form a chain of programmatic dependent launches: a kernel lets
+// the next one of the chain start its set-up as soon as all of its own blocks run
+// (pdl_trigger), and touches payload only after the one before it has finished
+// (pdl_wait).  Both do nothing in a launch without that attribute.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// dep: the launch depends on the one before it in the stream (its chain's), as above
+template <typename L>
+static cudaError_t launch(void (*f)(const L), int grid, int block, size_t smem, cudaStream_t st, bool dep, const L &l) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = dep ? 1 : 0;
+    return cudaLaunchKernelEx(&c, f, l);
 }
 
 // Unit (element or row) and chunk-in-unit of local chunk x of a tile whose first chunk
@@ -201,6 +236,7 @@ __device__ __forceinline__ void copy_flat_pipelined(const CopyDesc *__restrict__
     int64_t e[U], j[U];
     bool ok[U];
     flat_indices<VEC, U, FORM>(d, t, gi, gd, e, j, ok);
+    pdl_wait();
     for (;;) {
         const int64_t tn = t + gridDim.x;
         V val[U];
@@ -280,56 +316,33 @@ __device__ __forceinline__ void copy_tile(const CopyDesc *__restrict__ d, int64_
         if ((int64_t)(u * B + threadIdx.x) < left) stv<VEC>(d->dst + pos[u], val[u]);
 }
 
-// VEC > 0: every op of the launch has that vector width; VEC == 0: mixed widths
-// (batched patterns), dispatched per tile.  FLAT 0: segment form, 1: flat form, 3: two-index
-// flat form, 2: per op.
+// Every op of a launch has vector width VEC and one form, FLAT 0: segment form, 1: flat form,
+// 3: two-index flat form.
 // GBX_COPY_OCC (threads per SM the register budget must allow; 0 = no constraint) trades
 // registers for resident warps.
 #ifndef GBX_COPY_OCC
 #define GBX_COPY_OCC 0
 #endif
-template <int VEC, int U>
-__device__ __forceinline__ void copy_tile_any(const CopyDesc *__restrict__ d, int64_t t, int flat) {
-    if ((flat & 3) == 3) copy_tile_flat2<VEC, U>(d, t);
-    else if (flat) copy_tile_flat<VEC, U>(d, t);
-    else copy_tile<VEC, U>(d, t);
-}
-
-template <int VEC, int U, int FLAT>
+template <int VEC, int U, int FLAT, typename L>
 __global__ void __launch_bounds__(GBX_TILE / U, GBX_COPY_OCC ? GBX_COPY_OCC / (GBX_TILE / U) : 1)
-gbx_copy_kernel(const CopyDesc *const *__restrict__ ops, const int64_t *__restrict__ prefix,
-                int nops, int64_t total_tiles) {
-    for (int64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
-        const int op = nops > 1 ? find_op(prefix, nops, t) : 0;
-        const CopyDesc *d = ops[op];
-        const int64_t lt = t - __ldg(prefix + op);
-        if (VEC) {
-            if (FLAT == 1) copy_tile_flat<VEC ? VEC : 1, U>(d, lt);
-            else if (FLAT == 3) copy_tile_flat2<VEC ? VEC : 1, U>(d, lt);
-            else if (FLAT == 0) copy_tile<VEC ? VEC : 1, U>(d, lt);
-            else copy_tile_any<VEC ? VEC : 1, U>(d, lt, d->flat);
-        } else {
-            const int fl = d->flat;
-            switch (d->vec) {
-                case 16: copy_tile_any<16, U>(d, lt, fl); break;
-                case 8: copy_tile_any<8, U>(d, lt, fl); break;
-                case 4: copy_tile_any<4, U>(d, lt, fl); break;
-                case 2: copy_tile_any<2, U>(d, lt, fl); break;
-                default: copy_tile_any<1, U>(d, lt, fl); break;
-            }
-        }
+gbx_copy_kernel(const __grid_constant__ L list) {
+    pdl_trigger();
+    pdl_wait();
+    for (int64_t t = blockIdx.x; t < list.tiles(); t += gridDim.x) {
+        int64_t lt;
+        const CopyDesc *d = list.at(t, lt);
+        if (FLAT == 1) copy_tile_flat<VEC, U>(d, lt);
+        else if (FLAT == 3) copy_tile_flat2<VEC, U>(d, lt);
+        else copy_tile<VEC, U>(d, lt);
     }
 }
 
 // Pipelined flat forms (descriptor flat = 5: gather, 7: two-index), one op per launch,
 // persistent grid; launch bounds keep two full waves of threads resident (<= 32 registers).
-template <int VEC, int U, int FORM>
-__global__ void __launch_bounds__(GBX_TILE / U, 2 * U)
-gbx_copy_pipe_kernel(const CopyDesc *const *__restrict__ ops, const int64_t *__restrict__ prefix, int nops,
-                     int64_t total_tiles) {
-    (void)prefix;
-    (void)nops;
-    copy_flat_pipelined<VEC, U, FORM>(ops[0], total_tiles);
+template <int VEC, int U, int FORM, typename L>
+__global__ void __launch_bounds__(GBX_TILE / U, 2 * U) gbx_copy_pipe_kernel(const __grid_constant__ L list) {
+    pdl_trigger();
+    copy_flat_pipelined<VEC, U, FORM>(list.first(), list.tiles());
 }
 
 // ------------------------------------------------------------------------ bulk
@@ -346,11 +359,11 @@ __device__ int gbx_bulk_status;
 // Records a status code (1: a bounded wait gave up, 2: a piece failed its check) in the
 // process-wide word and in the status word of every op of the launch: a launch that gives up
 // leaves pieces of any of its ops unfinished, so each request it serves must report it.
-template <typename D>
-__device__ __noinline__ void gbx_raise(const D *const *__restrict__ ops, int nops, int code) {
+template <typename L>
+__device__ __noinline__ void gbx_raise(const L &list, int code) {
     atomicExch(&gbx_bulk_status, code);
-    for (int i = 0; i < nops; i++) {
-        int *w = ops[i]->status;
+    for (int i = 0; i < list.count(); i++) {
+        int *w = list.op(i)->status;
         if (w) *reinterpret_cast<volatile int *>(w) = code;
     }
     __threadfence_system();
@@ -369,13 +382,14 @@ __device__ __forceinline__ bool bulk_wait(uint32_t bar, uint32_t parity, int lim
     return false;
 }
 
-__global__ void __launch_bounds__(32) gbx_bulk_kernel(const CopyDesc *const *__restrict__ ops,
-                                                      const int64_t *__restrict__ prefix, int nops,
-                                                      int64_t ntasks) {
+template <typename L>
+__global__ void __launch_bounds__(32) gbx_bulk_kernel(const __grid_constant__ L list) {
     extern __shared__ __align__(128) unsigned char gbx_bulk_smem[];
     __shared__ __align__(8) uint64_t bar[GBX_BULK_STAGES];
+    pdl_trigger();
     if (threadIdx.x != 0) return;
     constexpr int S = GBX_BULK_STAGES;
+    const int64_t ntasks = list.tiles();
     const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(gbx_bulk_smem);
     const uint32_t sbar = (uint32_t)__cvta_generic_to_shared(bar);
     for (int q = 0; q < S; q++) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sbar + 8 * q) : "memory");
@@ -391,15 +405,15 @@ __global__ void __launch_bounds__(32) gbx_bulk_kernel(const CopyDesc *const *__r
         len_of[q] = 0;
     }
     auto load = [&](int q, int64_t t) {
-        const int op = nops > 1 ? find_op(prefix, nops, t) : 0;
-        const CopyDesc *d = ops[op];
-        const BulkTask k = d->bulk[t - (nops > 1 ? __ldg(prefix + op) : 0)];
+        int64_t lt;
+        const CopyDesc *d = list.at(t, lt);
+        const BulkTask k = d->bulk[lt];
         const uint32_t b = sbar + 8 * q, len = (uint32_t)k.len;
         // pieces were validated at init; a piece that is not a whole number of aligned 16-byte
         // units within one stage is recorded and skipped
         if (k.len <= 0 || k.len > GBX_BULK_BYTES || ((k.len | k.src | k.dst |
                                                       (int64_t)(uintptr_t)d->src | (int64_t)(uintptr_t)d->dst) & 15)) {
-            gbx_raise(ops, nops, 2);
+            gbx_raise(list, 2);
             dst_of[q] = nullptr;
             len_of[q] = 0;
             pend[q] = false;
@@ -413,12 +427,13 @@ __global__ void __launch_bounds__(32) gbx_bulk_kernel(const CopyDesc *const *__r
         len_of[q] = len;
         pend[q] = true;
     };
+    pdl_wait();
 #pragma unroll
     for (int q = 0; q < S; q++) {
         const int64_t t = blockIdx.x + (int64_t)q * gridDim.x;
         if (t < ntasks) load(q, t);
     }
-    const int limit = ops[0]->wait_limit;
+    const int limit = list.first()->wait_limit;
     bool failed = false;
     for (int64_t k = 0;; k++) {
         const int64_t t = blockIdx.x + k * gridDim.x;
@@ -447,16 +462,22 @@ __global__ void __launch_bounds__(32) gbx_bulk_kernel(const CopyDesc *const *__r
         }
     }
     if (failed) {
-        gbx_raise(ops, nops, 1);
+        gbx_raise(list, 1);
         for (int q = 0; q < S; q++)
             if (pend[q]) bulk_wait(sbar + 8 * q, parity[q]);
     }
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
+// Allows `bytes` of dynamic shared memory to both ways of launching a kernel.
+static cudaError_t smem_attr(void (*one)(const OneOp<CopyDesc>), void (*pooled)(const OpList<CopyDesc>), int bytes) {
+    cudaError_t e = cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e == cudaSuccess ? cudaFuncSetAttribute(pooled, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) : e;
+}
+
 int gbx_bulk_prepare(void) {
-    cudaError_t e = cudaFuncSetAttribute(gbx_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         GBX_BULK_STAGES * GBX_BULK_BYTES);
+    cudaError_t e = smem_attr(gbx_bulk_kernel<OneOp<CopyDesc>>, gbx_bulk_kernel<OpList<CopyDesc>>,
+                              GBX_BULK_STAGES * GBX_BULK_BYTES);
     return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
 }
 
@@ -471,10 +492,10 @@ int gbx_bulk_prepare(void) {
 // refilling it.  No CTA-wide barrier is crossed after setup, so a slow warp holds back only
 // its own stage.  Every wait is bounded: a consumer that gives up raises `abort`, the producer
 // then stops issuing, waits (bounded) for the copies it has in flight, and every warp leaves.
-template <int NT, int S>
-__global__ void __launch_bounds__(NT) gbx_scatter_kernel(const CopyDesc *const *__restrict__ ops,
-                                                         const int64_t *__restrict__ prefix, int nops,
-                                                         int64_t npieces) {
+template <int NT, int S, typename L>
+__global__ void __launch_bounds__(NT) gbx_scatter_kernel(const __grid_constant__ L list) {
+    const int64_t npieces = list.tiles();
+    pdl_trigger();
     constexpr int NC = NT - 32;          // consumer threads
     constexpr int NCW = NC / 32;         // consumer warps: arrivals that release a stage
     extern __shared__ __align__(128) unsigned char gbx_scatter_smem[];
@@ -500,9 +521,9 @@ __global__ void __launch_bounds__(NT) gbx_scatter_kernel(const CopyDesc *const *
         if (lane != 0) return;
         // ---------------------------------------------------------------- producer
         auto fetch = [&](int64_t t, const CopyDesc *&d) {   // piece t into next_s, asynchronously
-            const int op = nops > 1 ? find_op(prefix, nops, t) : 0;
-            d = ops[op];
-            const char *g = reinterpret_cast<const char *>(d->scat + (t - (nops > 1 ? __ldg(prefix + op) : 0)));
+            int64_t lt;
+            d = list.at(t, lt);
+            const char *g = reinterpret_cast<const char *>(d->scat + lt);
             const uint32_t sl = (uint32_t)__cvta_generic_to_shared(&next_s);
 #pragma unroll
             for (int i = 0; i < (int)sizeof(ScatterPiece) / 16; i++)
@@ -514,8 +535,9 @@ __global__ void __launch_bounds__(NT) gbx_scatter_kernel(const CopyDesc *const *
         for (int q = 0; q < S; q++) last[q] = -1;
         bool stop = false;
         const CopyDesc *d = nullptr;
-        const int limit = ops[0]->wait_limit;
+        const int limit = list.first()->wait_limit;
         if (blockIdx.x < npieces) fetch(blockIdx.x, d);
+        pdl_wait();
         for (int64_t k = 0;; k++) {
             const int64_t t = blockIdx.x + k * gridDim.x;
             if (t >= npieces) break;
@@ -548,15 +570,15 @@ __global__ void __launch_bounds__(NT) gbx_scatter_kernel(const CopyDesc *const *
             }
             const uint32_t fb = sfull + 8 * q;
             if (!good) {   // validated at init; recorded, and the consumers skip it
-                gbx_raise(ops, nops, 2);
+                gbx_raise(list, 2);
                 P.n = 0;
                 piece_s[q] = P;
-                desc_s[q] = pd;
+                if (!L::single) desc_s[q] = pd;
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fb) : "memory");
                 continue;
             }
             piece_s[q] = P;
-            desc_s[q] = pd;
+            if (!L::single) desc_s[q] = pd;
             const uint32_t ilen = (uint32_t)(i1 - i0), stage = sbuf + q * GBX_SCAT_STAGE;
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(bytes + 2 * ilen)
                          : "memory");
@@ -577,7 +599,7 @@ __global__ void __launch_bounds__(NT) gbx_scatter_kernel(const CopyDesc *const *
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         if (stop) {   // leave no copy in flight: wait (bounded) for the last one issued on each stage
-            gbx_raise(ops, nops, 1);
+            gbx_raise(list, 1);
             for (int q = 0; q < S; q++)
                 if (last[q] >= 0) bulk_wait(sfull + 8 * q, (uint32_t)((last[q] / S) & 1));
         }
@@ -585,7 +607,8 @@ __global__ void __launch_bounds__(NT) gbx_scatter_kernel(const CopyDesc *const *
     }
     // -------------------------------------------------------------------- consumers
     const int ct = threadIdx.x - 32;
-    const int limit = ops[0]->wait_limit;
+    const int limit = list.first()->wait_limit;
+    pdl_wait();
     for (int64_t k = 0;; k++) {
         const int64_t t = blockIdx.x + k * gridDim.x;
         if (t >= npieces) break;
@@ -594,7 +617,7 @@ __global__ void __launch_bounds__(NT) gbx_scatter_kernel(const CopyDesc *const *
             abort_flag = 1;
             break;
         }
-        const CopyDesc *d = desc_s[q];
+        const CopyDesc *d = L::single ? list.first() : desc_s[q];
         const int64_t src0 = piece_s[q].src, m0 = piece_s[q].m0;
         const int s = (int)d->elem_size, cpe = s >> 4, len = piece_s[q].len, n = piece_s[q].n;
         const unsigned char *win = gbx_scatter_smem + q * GBX_SCAT_STAGE;
@@ -605,7 +628,7 @@ __global__ void __launch_bounds__(NT) gbx_scatter_kernel(const CopyDesc *const *
             const int j = i / cpe, c = i - j * cpe;
             const int64_t w = (int64_t)ps[j] * s - src0 + c * 16;
             if (w < 0 || w + 16 > len) {   // validated at init; recorded and skipped
-                gbx_raise(ops, nops, 2);
+                gbx_raise(list, 2);
                 continue;
             }
             const uint4 v = *reinterpret_cast<const uint4 *>(win + w);
@@ -628,29 +651,27 @@ static ScatShape scatter_shape(int block) {
     return {1024, 8, 1};
 }
 
-static cudaError_t scatter_launch(int block, int grid, cudaStream_t st, const CopyDesc *const *ops,
-                                  const int64_t *prefix, int nops, int64_t n) {
+template <typename L>
+static cudaError_t scatter_launch(int block, int grid, cudaStream_t st, bool dep, const L &l) {
     const ScatShape h = scatter_shape(block);
     const size_t smem = (size_t)h.stages * GBX_SCAT_STAGE;
-    if (h.stages == 2) gbx_scatter_kernel<288, 2><<<grid, 288, smem, st>>>(ops, prefix, nops, n);
-    else if (h.nt == 288) gbx_scatter_kernel<288, 4><<<grid, 288, smem, st>>>(ops, prefix, nops, n);
-    else if (h.nt == 544) gbx_scatter_kernel<544, 4><<<grid, 544, smem, st>>>(ops, prefix, nops, n);
-    else gbx_scatter_kernel<1024, 8><<<grid, 1024, smem, st>>>(ops, prefix, nops, n);
-    return cudaGetLastError();
+    if (h.stages == 2) return launch(gbx_scatter_kernel<288, 2, L>, grid, 288, smem, st, dep, l);
+    if (h.nt == 288) return launch(gbx_scatter_kernel<288, 4, L>, grid, 288, smem, st, dep, l);
+    if (h.nt == 544) return launch(gbx_scatter_kernel<544, 4, L>, grid, 544, smem, st, dep, l);
+    return launch(gbx_scatter_kernel<1024, 8, L>, grid, 1024, smem, st, dep, l);
+}
+
+template <int NT, int S>
+static cudaError_t scatter_attr() {
+    return smem_attr(gbx_scatter_kernel<NT, S, OneOp<CopyDesc>>, gbx_scatter_kernel<NT, S, OpList<CopyDesc>>,
+                     S * GBX_SCAT_STAGE);
 }
 
 int gbx_scatter_prepare(void) {
-    cudaError_t e = cudaFuncSetAttribute(gbx_scatter_kernel<288, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         2 * GBX_SCAT_STAGE);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gbx_scatter_kernel<288, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 4 * GBX_SCAT_STAGE);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gbx_scatter_kernel<544, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 4 * GBX_SCAT_STAGE);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gbx_scatter_kernel<1024, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 8 * GBX_SCAT_STAGE);
+    cudaError_t e = scatter_attr<288, 2>();
+    if (e == cudaSuccess) e = scatter_attr<288, 4>();
+    if (e == cudaSuccess) e = scatter_attr<544, 4>();
+    if (e == cudaSuccess) e = scatter_attr<1024, 8>();
     return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
 }
 
@@ -669,10 +690,10 @@ int gbx_scatter_prepare(void) {
 // up raises `abort`, the producer stops issuing and drains its copies in flight).
 #define GBX_STREAM_IDX ((GBX_TILE + 8) * 4)   // bytes of one index array per stage
 
-template <int VEC, int FORM, int NT, int S, int U, int PS, bool ONE>
-__global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const CopyDesc *const *__restrict__ ops,
-                                                        const int64_t *__restrict__ prefix, int nops,
-                                                        int64_t ntiles) {
+template <int VEC, int FORM, int NT, int S, int U, int PS, bool ONE, typename L>
+__global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const __grid_constant__ L list) {
+    const int64_t ntiles = list.tiles();
+    pdl_trigger();
     typedef typename VecT<VEC>::T V;
     constexpr int NC = NT - 32, NCW = NC / 32;
     constexpr int STAGE = GBX_STREAM_IDX * (FORM == 3 ? 2 : 1);
@@ -694,7 +715,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const CopyDesc *cons
     }
     __syncthreads();   // the only CTA-wide barrier
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int limit = ops[0]->wait_limit;
+    const int limit = list.first()->wait_limit;
     if (warp == 0) {
         if (lane != 0) return;
         // ---------------------------------------------------------------- producer
@@ -715,9 +736,8 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const CopyDesc *cons
                 stop = true;
                 break;
             }
-            const int op = nops > 1 ? find_op(prefix, nops, t) : 0;
-            const CopyDesc *d = ops[op];
-            const int64_t lt = t - __ldg(prefix + op);
+            int64_t lt;
+            const CopyDesc *d = list.at(t, lt);
             const int64_t cpe = d->cpe;
             const int64_t c0 = lt * GBX_TILE;
             const int64_t c1 = min(d->nchunks, c0 + GBX_TILE);
@@ -725,12 +745,12 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const CopyDesc *cons
             const int64_t e_al = e_first & ~(int64_t)3, e_end = (e_last + 4) & ~(int64_t)3;
             const uint32_t bytes = (uint32_t)((e_end - e_al) * 4);
             const uint32_t fb = sfull + 8 * q, stage = sbuf + q * STAGE;
-            desc_s[q] = d;
+            if (!L::single) desc_s[q] = d;
             tile_s[q] = lt;
             efirst_s[q] = e_first;
             const uintptr_t al = (uintptr_t)d->flat_idx | (FORM == 3 ? (uintptr_t)d->flat_didx : 0);
             if ((al & 15) || bytes > GBX_STREAM_IDX || c1 <= c0) {   // validated at init; recorded, skipped
-                gbx_raise(ops, nops, 2);
+                gbx_raise(list, 2);
                 ebase_s[q] = -1;
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fb) : "memory");
                 continue;
@@ -750,7 +770,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const CopyDesc *cons
             last[q] = k;
         }
         if (stop) {   // leave no copy in flight: wait (bounded) for the last one issued on each stage
-            gbx_raise(ops, nops, 1);
+            gbx_raise(list, 1);
             for (int q = 0; q < S; q++)
                 if (last[q] >= 0) bulk_wait(sfull + 8 * q, (uint32_t)((last[q] / S) & 1));
         }
@@ -758,6 +778,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const CopyDesc *cons
     }
     // -------------------------------------------------------------------- consumers
     const int ct = threadIdx.x - 32;
+    pdl_wait();
     for (int64_t k = 0;; k++) {
         const int64_t t = blockIdx.x + k * gridDim.x;
         if (t >= ntiles) break;
@@ -770,7 +791,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const CopyDesc *cons
         if (ONE && e_al >= 0) {
             // ONE (every op of the launch has one chunk per element, elem_size == VEC): chunk x
             // of the tile is element e0 + x, every offset a multiple of VEC
-            const CopyDesc *d = desc_s[q];
+            const CopyDesc *d = L::single ? list.first() : desc_s[q];
             const int64_t e0 = efirst_s[q];
             const int left = (int)min((int64_t)GBX_TILE, d->nchunks - tile_s[q] * GBX_TILE);
             const int32_t *is = reinterpret_cast<const int32_t *>(gbx_stream_smem + q * STAGE) + (e0 - e_al);
@@ -799,7 +820,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const CopyDesc *cons
                 }
             }
         } else if (!ONE && e_al >= 0) {
-            const CopyDesc *d = desc_s[q];
+            const CopyDesc *d = L::single ? list.first() : desc_s[q];
             const int cpe = d->cpe, sh = d->cpe_shift;
             const uint32_t magic = d->cpe_magic;
             const int64_t s = d->elem_size, e0 = efirst_s[q], c0 = tile_s[q] * GBX_TILE;
@@ -853,62 +874,56 @@ static StreamShape stream_shape(int block) {
     return {544, 6, 2, 2};
 }
 
-template <int VEC, int FORM, bool ONE>
-static cudaError_t stream_launch_v(int block, int grid, cudaStream_t st, const CopyDesc *const *ops,
-                                   const int64_t *prefix, int nops, int64_t n) {
+template <int VEC, int FORM, bool ONE, typename L>
+static cudaError_t stream_launch_v(int block, int grid, cudaStream_t st, bool dep, const L &l) {
     const StreamShape h = stream_shape(block);
     constexpr int SC = FORM == 3 ? 3 : 4;   // stages of the narrow shape
     const size_t smem = (size_t)(h.nt == 160 ? SC : h.stages) * GBX_STREAM_IDX * (FORM == 3 ? 2 : 1);
     if (h.nt == 160) {
         if constexpr (ONE && VEC <= 8)
-            gbx_stream_kernel<VEC, FORM, 160, SC, 8, 8, ONE><<<grid, 160, smem, st>>>(ops, prefix, nops, n);
+            return launch(gbx_stream_kernel<VEC, FORM, 160, SC, 8, 8, ONE, L>, grid, 160, smem, st, dep, l);
         else
             return cudaErrorInvalidValue;   // never chosen: only one-chunk ops of vectors up to 8 bytes
-    } else if (h.nt == 288)
-        gbx_stream_kernel<VEC, FORM, 288, 4, 4, 4, ONE><<<grid, 288, smem, st>>>(ops, prefix, nops, n);
-    else
-        gbx_stream_kernel<VEC, FORM, 544, 6, 2, 2, ONE><<<grid, 544, smem, st>>>(ops, prefix, nops, n);
-    return cudaGetLastError();
+    }
+    if (h.nt == 288) return launch(gbx_stream_kernel<VEC, FORM, 288, 4, 4, 4, ONE, L>, grid, 288, smem, st, dep, l);
+    return launch(gbx_stream_kernel<VEC, FORM, 544, 6, 2, 2, ONE, L>, grid, 544, smem, st, dep, l);
 }
 
-template <int VEC>
-static cudaError_t stream_launch_f(int flat, int block, int grid, cudaStream_t st, const CopyDesc *const *ops,
-                                   const int64_t *prefix, int nops, int64_t n) {
+template <int VEC, typename L>
+static cudaError_t stream_launch_f(int flat, int block, int grid, cudaStream_t st, bool dep, const L &l) {
     switch (flat) {
-        case 10: return stream_launch_v<VEC, 1, false>(block, grid, st, ops, prefix, nops, n);
-        case 11: return stream_launch_v<VEC, 3, false>(block, grid, st, ops, prefix, nops, n);
-        case 12: return stream_launch_v<VEC, 1, true>(block, grid, st, ops, prefix, nops, n);
-        default: return stream_launch_v<VEC, 3, true>(block, grid, st, ops, prefix, nops, n);
+        case 10: return stream_launch_v<VEC, 1, false>(block, grid, st, dep, l);
+        case 11: return stream_launch_v<VEC, 3, false>(block, grid, st, dep, l);
+        case 12: return stream_launch_v<VEC, 1, true>(block, grid, st, dep, l);
+        default: return stream_launch_v<VEC, 3, true>(block, grid, st, dep, l);
     }
 }
 
 // flat 10 / 11: the stream forms; 12 / 13: the same when every op of the launch has one chunk
 // per element (the kernel then skips the element / chunk split)
-static cudaError_t stream_launch(int vec, int flat, int block, int grid, cudaStream_t st, const CopyDesc *const *ops,
-                                 const int64_t *prefix, int nops, int64_t n) {
+template <typename L>
+static cudaError_t stream_launch(int vec, int flat, int block, int grid, cudaStream_t st, bool dep, const L &l) {
     switch (vec) {
-        case 16: return stream_launch_f<16>(flat, block, grid, st, ops, prefix, nops, n);
-        case 8: return stream_launch_f<8>(flat, block, grid, st, ops, prefix, nops, n);
-        case 4: return stream_launch_f<4>(flat, block, grid, st, ops, prefix, nops, n);
+        case 16: return stream_launch_f<16>(flat, block, grid, st, dep, l);
+        case 8: return stream_launch_f<8>(flat, block, grid, st, dep, l);
+        case 4: return stream_launch_f<4>(flat, block, grid, st, dep, l);
         default: return cudaErrorInvalidValue;   // the stream form is offered for vectors of 4..16 bytes
     }
 }
 
+template <int VEC, int FORM, int NT, int S, int U, int PS, bool ONE>
+static cudaError_t stream_attr_k() {
+    return smem_attr(gbx_stream_kernel<VEC, FORM, NT, S, U, PS, ONE, OneOp<CopyDesc>>,
+                     gbx_stream_kernel<VEC, FORM, NT, S, U, PS, ONE, OpList<CopyDesc>>,
+                     S * GBX_STREAM_IDX * (FORM == 3 ? 2 : 1));
+}
+
 template <int VEC, int FORM, bool ONE>
 static cudaError_t stream_attr_o() {
-    cudaError_t e = cudaFuncSetAttribute(gbx_stream_kernel<VEC, FORM, 288, 4, 4, 4, ONE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         4 * GBX_STREAM_IDX * (FORM == 3 ? 2 : 1));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gbx_stream_kernel<VEC, FORM, 544, 6, 2, 2, ONE>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * GBX_STREAM_IDX * (FORM == 3 ? 2 : 1));
-    if constexpr (ONE && VEC <= 8) {
-        constexpr int SC = FORM == 3 ? 3 : 4;
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(gbx_stream_kernel<VEC, FORM, 160, SC, 8, 8, ONE>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     SC * GBX_STREAM_IDX * (FORM == 3 ? 2 : 1));
-    }
+    cudaError_t e = stream_attr_k<VEC, FORM, 288, 4, 4, 4, ONE>();
+    if (e == cudaSuccess) e = stream_attr_k<VEC, FORM, 544, 6, 2, 2, ONE>();
+    if constexpr (ONE && VEC <= 8)
+        if (e == cudaSuccess) e = stream_attr_k<VEC, FORM, 160, FORM == 3 ? 3 : 4, 8, 8, ONE>();
     return e;
 }
 
@@ -954,7 +969,7 @@ __device__ __forceinline__ float2 padd(float2 a, float2 b) { return make_float2(
 __device__ __forceinline__ float padd(float a, float b) { return __fadd_rn(a, b); }
 
 template <typename P>
-__device__ __forceinline__ P pload(const char *p) { return __ldg(reinterpret_cast<const P *>(p)); }
+__device__ __forceinline__ P pload(const char *p) { return *reinterpret_cast<const P *>(p); }   // (as ldv)
 
 template <typename T, int VEC, int U>
 __device__ __forceinline__ void fold_tile(const FoldDesc *__restrict__ d, int64_t t) {
@@ -1044,10 +1059,10 @@ __device__ __forceinline__ void fold_tile(const FoldDesc *__restrict__ d, int64_
 // gradient loads in flight per thread: 8 of 4 or 8 bytes, 4 of 16 bytes (the registers of
 // 2 CTAs of 544 threads per SM)
 
-template <typename T, int VEC, int NT, int S, int PS>
-__global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const FoldDesc *const *__restrict__ ops,
-                                                           const int64_t *__restrict__ prefix, int nops,
-                                                           int64_t ntiles) {
+template <typename T, int VEC, int NT, int S, int PS, typename L>
+__global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const __grid_constant__ L list) {
+    const int64_t ntiles = list.tiles();
+    pdl_trigger();
     typedef typename PackT<T, VEC>::T PK;
     constexpr int NC = NT - 32, NCW = NC / 32;
     constexpr int GBX_SFOLD_K = VEC == 16 ? 4 : 8;
@@ -1069,7 +1084,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const FoldDesc *const
     }
     __syncthreads();   // the only CTA-wide barrier
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int limit = ops[0]->wait_limit;
+    const int limit = list.first()->wait_limit;
     if (warp == 0) {
         if (lane != 0) return;
         // ---------------------------------------------------------------- producer
@@ -1090,9 +1105,8 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const FoldDesc *const
                 stop = true;
                 break;
             }
-            const int op = nops > 1 ? find_op(prefix, nops, t) : 0;
-            const FoldDesc *d = ops[op];
-            const int64_t lt = t - __ldg(prefix + op);
+            int64_t lt;
+            const FoldDesc *d = list.at(t, lt);
             const int64_t cpe = d->cpe, c0 = lt * GBX_TILE, c1 = min(d->nchunks, c0 + GBX_TILE);
             const int64_t r_first = c0 / cpe, r_last = (c1 - 1) / cpe;
             const uint32_t rbytes = (uint32_t)((r_last - r_first + 1) * 16);
@@ -1101,13 +1115,13 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const FoldDesc *const
             const bool inl = (te_al - tb_al) <= GBX_SFOLD_TERMS;
             const uint32_t tbytes = inl ? (uint32_t)((te_al - tb_al) * 8) : 0u;
             const uint32_t fb = sfull + 8 * q, stage = sbuf + q * GBX_SFOLD_STAGE;
-            desc_s[q] = d;
+            if (!L::single) desc_s[q] = d;
             tile_s[q] = lt;
             rfirst_s[q] = r_first;
             tbase_s[q] = inl ? tb_al : -1;
             const uintptr_t al = (uintptr_t)d->rec | (uintptr_t)d->terms;
             if ((al & 15) || rbytes > GBX_SFOLD_REC || c1 <= c0) {   // validated at init; recorded, skipped
-                gbx_raise(ops, nops, 2);
+                gbx_raise(list, 2);
                 rfirst_s[q] = -1;
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fb) : "memory");
                 continue;
@@ -1125,7 +1139,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const FoldDesc *const
             last[q] = k;
         }
         if (stop) {
-            gbx_raise(ops, nops, 1);
+            gbx_raise(list, 1);
             for (int q = 0; q < S; q++)
                 if (last[q] >= 0) bulk_wait(sfull + 8 * q, (uint32_t)((last[q] / S) & 1));
         }
@@ -1133,6 +1147,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const FoldDesc *const
     }
     // -------------------------------------------------------------------- consumers
     const int ct = threadIdx.x - 32;
+    pdl_wait();
     for (int64_t k = 0;; k++) {
         const int64_t t = blockIdx.x + k * gridDim.x;
         if (t >= ntiles) break;
@@ -1143,7 +1158,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const FoldDesc *const
         }
         const int64_t r_first = rfirst_s[q];
         if (r_first >= 0) {
-            const FoldDesc *d = desc_s[q];
+            const FoldDesc *d = L::single ? list.first() : desc_s[q];
             const int cpe = d->cpe, sh = d->cpe_shift;
             const uint32_t magic = d->cpe_magic;
             const int64_t c0 = tile_s[q] * GBX_TILE, tb_al = tbase_s[q];
@@ -1208,18 +1223,21 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const FoldDesc *const
 #define GBX_SFOLD_NT 544
 #define GBX_SFOLD_S 3
 
-template <typename T, int VEC>
-static cudaError_t sfold_launch_v(int grid, cudaStream_t st, const FoldDesc *const *ops, const int64_t *prefix,
-                                  int nops, int64_t n) {
-    gbx_sfold_kernel<T, VEC, GBX_SFOLD_NT, GBX_SFOLD_S, 2>
-        <<<grid, GBX_SFOLD_NT, GBX_SFOLD_S * GBX_SFOLD_STAGE, st>>>(ops, prefix, nops, n);
-    return cudaGetLastError();
+template <typename T, int VEC, typename L>
+static cudaError_t sfold_launch_v(int grid, cudaStream_t st, bool dep, const L &l) {
+    return launch(gbx_sfold_kernel<T, VEC, GBX_SFOLD_NT, GBX_SFOLD_S, 2, L>, grid, GBX_SFOLD_NT,
+                  (size_t)GBX_SFOLD_S * GBX_SFOLD_STAGE, st, dep, l);
 }
 
+template <typename T, int VEC, typename L>
+static cudaError_t sfold_attr_l() {
+    return cudaFuncSetAttribute(gbx_sfold_kernel<T, VEC, GBX_SFOLD_NT, GBX_SFOLD_S, 2, L>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, GBX_SFOLD_S * GBX_SFOLD_STAGE);
+}
 template <typename T, int VEC>
 static cudaError_t sfold_attr_v() {
-    return cudaFuncSetAttribute(gbx_sfold_kernel<T, VEC, GBX_SFOLD_NT, GBX_SFOLD_S, 2>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, GBX_SFOLD_S * GBX_SFOLD_STAGE);
+    cudaError_t e = sfold_attr_l<T, VEC, OneOp<FoldDesc>>();
+    return e == cudaSuccess ? sfold_attr_l<T, VEC, OpList<FoldDesc>>() : e;
 }
 
 int gbx_sfold_prepare(void) {
@@ -1231,22 +1249,18 @@ int gbx_sfold_prepare(void) {
     return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
 }
 
-// CLS 1..5: every op of the launch is (f64,16) (f64,8) (f32,16) (f32,8) (f32,4);
-// CLS 0: mixed (batched patterns), dispatched per tile.  The single-payload kernels with one
-// chunk per thread (1024-thread blocks) are held to 32 registers so that two blocks fit on
-// an SM: the fold is bound by load latency, and the doubled occupancy outweighs the few
+// CLS 1..5: every op of the launch is (f64,16) (f64,8) (f32,16) (f32,8) (f32,4).  The kernels
+// with one chunk per thread (1024-thread blocks) are held to 32 registers so that two blocks
+// fit on an SM: the fold is bound by load latency, and the doubled occupancy outweighs the few
 // bytes of spill this costs (512^3 backward, all rows folded: 0.90 -> 0.82 ms).
-template <int CLS, int U>
-__global__ void __launch_bounds__(GBX_TILE / U, (U == 1 && CLS != 0) ? 2 : 1)
-gbx_fold_kernel(const FoldDesc *const *__restrict__ ops, const int64_t *__restrict__ prefix,
-                int nops, int64_t total_tiles) {
-    for (int64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
-        const int op = nops > 1 ? find_op(prefix, nops, t) : 0;
-        const FoldDesc *d = ops[op];
-        const int64_t lt = t - __ldg(prefix + op);
-        const int cls = CLS ? CLS : (d->dtype == GBX_F64 ? (d->vec == 16 ? 1 : 2)
-                                                         : (d->vec == 16 ? 3 : d->vec == 8 ? 4 : 5));
-        switch (cls) {
+template <int CLS, int U, typename L>
+__global__ void __launch_bounds__(GBX_TILE / U, U == 1 ? 2 : 1) gbx_fold_kernel(const __grid_constant__ L list) {
+    pdl_trigger();
+    pdl_wait();
+    for (int64_t t = blockIdx.x; t < list.tiles(); t += gridDim.x) {
+        int64_t lt;
+        const FoldDesc *d = list.at(t, lt);
+        switch (CLS) {
             case 1: fold_tile<double, 16, U>(d, lt); break;
             case 2: fold_tile<double, 8, U>(d, lt); break;
             case 3: fold_tile<float, 16, U>(d, lt); break;
@@ -1269,81 +1283,68 @@ int gbx_num_sms(void) {
     return g_num_sms;
 }
 
-typedef void (*CopyFn)(const CopyDesc *const *, const int64_t *, int, int64_t);
-typedef void (*FoldFn)(const FoldDesc *const *, const int64_t *, int, int64_t);
-
-template <int VEC, int FLAT>
-static CopyFn copy_fn_u(int block) {
+template <int VEC, int FLAT, typename L>
+static void (*copy_fn_u(int block))(const L) {
     switch (block) {
-        case 128: return gbx_copy_kernel<VEC, 8, FLAT>;
-        case 256: return gbx_copy_kernel<VEC, 4, FLAT>;
-        case 512: return gbx_copy_kernel<VEC, 2, FLAT>;
-        default: return gbx_copy_kernel<VEC, 1, FLAT>;
+        case 128: return gbx_copy_kernel<VEC, 8, FLAT, L>;
+        case 256: return gbx_copy_kernel<VEC, 4, FLAT, L>;
+        case 512: return gbx_copy_kernel<VEC, 2, FLAT, L>;
+        default: return gbx_copy_kernel<VEC, 1, FLAT, L>;
     }
 }
 
-template <int VEC, int FORM>
-static CopyFn pipe_fn_u(int block) {
-    return block == 1024 ? gbx_copy_pipe_kernel<VEC, 1, FORM> : gbx_copy_pipe_kernel<VEC, 2, FORM>;
+template <int VEC, int FORM, typename L>
+static void (*pipe_fn_u(int block))(const L) {
+    return block == 1024 ? gbx_copy_pipe_kernel<VEC, 1, FORM, L> : gbx_copy_pipe_kernel<VEC, 2, FORM, L>;
 }
 
-template <int VEC>
-static CopyFn copy_fn_v(int block, int flat) {
-    if (flat == 5) return pipe_fn_u<VEC, 1>(block);
-    if (flat == 7) return pipe_fn_u<VEC, 3>(block);
-    if (flat == 1) return copy_fn_u<VEC, 1>(block);
-    if (flat == 3) return copy_fn_u<VEC, 3>(block);
-    if (flat == 0) return copy_fn_u<VEC, 0>(block);
-    return copy_fn_u<VEC, 2>(block);
+template <int VEC, typename L>
+static void (*copy_fn_v(int block, int flat))(const L) {
+    if (flat == 5) return pipe_fn_u<VEC, 1, L>(block);
+    if (flat == 7) return pipe_fn_u<VEC, 3, L>(block);
+    if (flat == 1) return copy_fn_u<VEC, 1, L>(block);
+    if (flat == 3) return copy_fn_u<VEC, 3, L>(block);
+    return copy_fn_u<VEC, 0, L>(block);
 }
 
-// flat: 0 segment form, 1 flat form, 3 two-index flat form, 2 decided per op (mixed launches),
-// 5 / 7 the pipelined flat forms (one op, persistent grid, block 512 or 1024)
-static CopyFn copy_fn(int vec, int block, int flat) {
+// flat: 0 segment form, 1 flat form, 3 two-index flat form, 5 / 7 the pipelined flat forms (one
+// op, persistent grid, block 512 or 1024)
+template <typename L>
+static void (*copy_fn(int vec, int block, int flat))(const L) {
     switch (vec) {
-        case 16: return copy_fn_v<16>(block, flat);
-        case 8: return copy_fn_v<8>(block, flat);
-        case 4: return copy_fn_v<4>(block, flat);
-        case 2: return copy_fn_v<2>(block, flat);
-        case 1: return copy_fn_v<1>(block, flat);
-        default:   // mixed widths: U <= 4
-            switch (block) {
-                case 512: return gbx_copy_kernel<0, 2, 2>;
-                case 1024: return gbx_copy_kernel<0, 1, 2>;
-                default: return gbx_copy_kernel<0, 4, 2>;
-            }
+        case 16: return copy_fn_v<16, L>(block, flat);
+        case 8: return copy_fn_v<8, L>(block, flat);
+        case 4: return copy_fn_v<4, L>(block, flat);
+        case 2: return copy_fn_v<2, L>(block, flat);
+        default: return copy_fn_v<1, L>(block, flat);
     }
 }
 
-template <int CLS>
-static FoldFn fold_fn_u(int block) {
+template <int CLS, typename L>
+static void (*fold_fn_u(int block))(const L) {
     switch (block) {
-        case 128: return gbx_fold_kernel<CLS, 8>;
-        case 256: return gbx_fold_kernel<CLS, 4>;
-        case 512: return gbx_fold_kernel<CLS, 2>;
-        default: return gbx_fold_kernel<CLS, 1>;
+        case 128: return gbx_fold_kernel<CLS, 8, L>;
+        case 256: return gbx_fold_kernel<CLS, 4, L>;
+        case 512: return gbx_fold_kernel<CLS, 2, L>;
+        default: return gbx_fold_kernel<CLS, 1, L>;
     }
 }
 
 static int fold_cls(int dtype, int vec) {
-    if (vec == 0) return 0;
     if (dtype == GBX_F64) return vec == 16 ? 1 : 2;
     return vec == 16 ? 3 : vec == 8 ? 4 : 5;
 }
 
-static FoldFn fold_fn(int dtype, int vec, int block) {
+template <typename L>
+static void (*fold_fn(int dtype, int vec, int block))(const L) {
     switch (fold_cls(dtype, vec)) {
-        case 1: return fold_fn_u<1>(block);
-        case 2: return fold_fn_u<2>(block);
-        case 3: return fold_fn_u<3>(block);
-        case 4: return fold_fn_u<4>(block);
-        case 5: return fold_fn_u<5>(block);
-        default: return block == 128 ? gbx_fold_kernel<0, 4> : fold_fn_u<0>(block);
+        case 1: return fold_fn_u<1, L>(block);
+        case 2: return fold_fn_u<2, L>(block);
+        case 3: return fold_fn_u<3, L>(block);
+        case 4: return fold_fn_u<4, L>(block);
+        default: return fold_fn_u<5, L>(block);
     }
 }
-
-// Blocks of the mixed kernels never go below 256 threads (their unroll is capped at 4).
-int gbx_effective_block(int vec_class, int block) { return (vec_class == 0 && block < 256) ? 256 : block; }
 
 static int pipe_block(int flat, int block) { return (flat == 5 || flat == 7) && block < 512 ? 512 : block; }
 
@@ -1353,9 +1354,10 @@ int gbx_occupancy(int kind, int dtype, int vec, int block, int flat) {
     if (kind == 0 && flat == 9) return scatter_shape(block).per_sm;
     if (kind == 0 && flat >= 10 && flat <= 13) return stream_shape(block).per_sm;
     if (kind == 0) block = pipe_block(flat, block);
-    const void *f = kind == 0 ? (const void *)copy_fn(vec, block, flat) : (const void *)fold_fn(dtype, vec, block);
+    const void *f = kind == 0 ? (const void *)copy_fn<OneOp<CopyDesc>>(vec, block, flat)
+                              : (const void *)fold_fn<OneOp<FoldDesc>>(dtype, vec, block);
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, gbx_effective_block(vec, block), 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, block, 0);
     return n > 0 ? n : 1;
 }
 
@@ -1364,45 +1366,48 @@ static int clamp_grid(int grid, int64_t total_tiles) {
     return grid;
 }
 
-cudaError_t gbx_launch_copy(const CopyDesc *const *ops, const int64_t *tile_prefix, int nops, int64_t total_tiles,
-                            int vec, int flat, int block, int grid, cudaStream_t st) {
-    if (total_tiles <= 0) return cudaSuccess;
-    if (flat == 8) {   // bulk form: a "tile" is one piece
-        gbx_bulk_kernel<<<clamp_grid(grid, total_tiles), 32, GBX_BULK_STAGES * GBX_BULK_BYTES, st>>>(
-            ops, tile_prefix, nops, total_tiles);
-        return cudaGetLastError();
-    }
-    if (flat == 9) {   // scatter form: a "tile" is one source window
-        return scatter_launch(block, clamp_grid(grid, total_tiles), st, ops, tile_prefix, nops, total_tiles);
-    }
+template <typename L>
+static cudaError_t launch_copy(const L &l, int nops, int vec, int flat, int block, int grid, cudaStream_t st, bool dep) {
+    grid = clamp_grid(grid, l.ntiles);
+    if (flat == 8)   // bulk form: a "tile" is one piece
+        return launch(gbx_bulk_kernel<L>, grid, 32, (size_t)GBX_BULK_STAGES * GBX_BULK_BYTES, st, dep, l);
+    if (flat == 9)   // scatter form: a "tile" is one source window
+        return scatter_launch(block, grid, st, dep, l);
     if (flat >= 10 && flat <= 13) {   // stream forms: the flat forms' tiles, indices through shared memory
         if (block <= 128 && !(flat >= 12 && vec <= 8)) block = 256;   // the narrow shape needs ONE, vec <= 8
-        return stream_launch(vec, flat, block, clamp_grid(grid, total_tiles), st, ops, tile_prefix, nops, total_tiles);
+        return stream_launch(vec, flat, block, grid, st, dep, l);
     }
-    if ((flat == 5 || flat == 7) && (nops > 1 || vec == 0)) flat -= 4;   // the pipelined kernels take one op
+    if ((flat == 5 || flat == 7) && nops > 1) flat -= 4;   // the pipelined kernels take one op
     block = pipe_block(flat, block);
-    CopyFn f = copy_fn(vec, block, flat);
-    f<<<clamp_grid(grid, total_tiles), gbx_effective_block(vec, block), 0, st>>>(ops, tile_prefix, nops, total_tiles);
-    return cudaGetLastError();
+    return launch(copy_fn<L>(vec, block, flat), grid, block, 0, st, dep, l);
 }
 
-cudaError_t gbx_launch_fold(const FoldDesc *const *ops, const int64_t *tile_prefix, int nops, int64_t total_tiles,
-                            int dtype, int vec, int block, int grid, cudaStream_t st, int form) {
-    if (total_tiles <= 0) return cudaSuccess;
-    if (form == 1 && vec != 0) {   // stream form: one payload class per launch
-        const int g = clamp_grid(grid, total_tiles);
+template <typename L>
+static cudaError_t launch_fold(const L &l, int dtype, int vec, int block, int grid, cudaStream_t st, int form, bool dep) {
+    grid = clamp_grid(grid, l.ntiles);
+    if (form == 1) {   // stream form
         switch (fold_cls(dtype, vec)) {
-            case 1: return sfold_launch_v<double, 16>(g, st, ops, tile_prefix, nops, total_tiles);
-            case 2: return sfold_launch_v<double, 8>(g, st, ops, tile_prefix, nops, total_tiles);
-            case 3: return sfold_launch_v<float, 16>(g, st, ops, tile_prefix, nops, total_tiles);
-            case 4: return sfold_launch_v<float, 8>(g, st, ops, tile_prefix, nops, total_tiles);
-            case 5: return sfold_launch_v<float, 4>(g, st, ops, tile_prefix, nops, total_tiles);
-            default: return cudaErrorInvalidValue;
+            case 1: return sfold_launch_v<double, 16>(grid, st, dep, l);
+            case 2: return sfold_launch_v<double, 8>(grid, st, dep, l);
+            case 3: return sfold_launch_v<float, 16>(grid, st, dep, l);
+            case 4: return sfold_launch_v<float, 8>(grid, st, dep, l);
+            default: return sfold_launch_v<float, 4>(grid, st, dep, l);
         }
     }
-    FoldFn f = fold_fn(dtype, vec, block);
-    f<<<clamp_grid(grid, total_tiles), gbx_effective_block(vec, block), 0, st>>>(ops, tile_prefix, nops, total_tiles);
-    return cudaGetLastError();
+    return launch(fold_fn<L>(dtype, vec, block), grid, block, 0, st, dep, l);
+}
+
+cudaError_t gbx_launch_copy(const OpRef<CopyDesc> &r, int vec, int flat, int block, int grid, cudaStream_t st, bool dep) {
+    if (r.ntiles <= 0) return cudaSuccess;
+    if (r.one) return launch_copy(OneOp<CopyDesc>{*r.one, r.ntiles}, 1, vec, flat, block, grid, st, dep);
+    return launch_copy(OpList<CopyDesc>{r.ops, r.prefix, r.nops, r.ntiles}, r.nops, vec, flat, block, grid, st, dep);
+}
+
+cudaError_t gbx_launch_fold(const OpRef<FoldDesc> &r, int dtype, int vec, int block, int grid, cudaStream_t st, int form,
+                            bool dep) {
+    if (r.ntiles <= 0) return cudaSuccess;
+    if (r.one) return launch_fold(OneOp<FoldDesc>{*r.one, r.ntiles}, dtype, vec, block, grid, st, form, dep);
+    return launch_fold(OpList<FoldDesc>{r.ops, r.prefix, r.nops, r.ntiles}, dtype, vec, block, grid, st, form, dep);
 }
 
 // tile_e0[t] = first unit of tile t; tile_seg[t] = segment holding it (copy ops);

@@ -1,0 +1,90 @@
+"""GPU: the ways a start reaches the device.  A launch of one op carries its descriptor by value,
+a start of several launches replays a graph until the first rebind and launches them one by one
+afterwards, graph=0 and batches read descriptors in device memory (rewritten by a rebind, or by
+the first batch after one).  Every way writes the oracle's bytes into the buffers bound at that
+moment, whether the start is completed by the host, on the request's own stream or on another."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import oracle  # noqa: E402
+import paper_2309_07337_gb300 as gbx  # noqa: E402
+from paper_2309_07337_gb300 import patterns as pt  # noqa: E402
+from gpu_util import assert_bytes_equal, dev_bytes, payload  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _complete(how, r, side):
+    if how == "host":
+        r.wait()
+    elif how == "own":
+        r.wait_stream()
+    else:
+        r.wait_stream(side)
+
+
+@pytest.mark.parametrize("alg", ["standard", "locality"])
+@pytest.mark.parametrize("info", ["", "graph=0"])
+@pytest.mark.parametrize("how", ["host", "own", "other"])
+def test_rebinds_between_starts(alg, info, how):
+    p = pt.stencil((20, 15, 12), (4, 3, 3), ppn=5, comps=3)
+    xs = [payload(p, 60 + k) for k in range(3)]
+    want = [oracle.standard(p, x) for x in xs]
+    sends = [dev_bytes(x) for x in xs]
+    outs = [torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda") for _ in range(3)]
+    ex = gbx.Exchange(p, sends[0], outs[0], alg, info=info)
+    other = gbx.Exchange(p, sends[0], torch.empty_like(outs[0]), alg, dp=ex.dp, graph=ex.graph)
+    side = torch.cuda.Stream()
+    bound = 0
+    for k in (0, 0, 1, 2, 0, 1):         # the first two starts run on the buffers bound at init
+        if k != bound:
+            ex.request.bind(sends[k], outs[k])
+            bound = k
+        outs[k].fill_(0xA5)
+        ex.start()
+        _complete(how, ex.request, side)
+        with torch.cuda.stream(side if how == "other" else torch.cuda.current_stream()):
+            got = outs[k].cpu().numpy()
+        assert_bytes_equal(got, want[k], f"{alg} {info} {how} buffers {k}")
+    # a batch built after the last rebind runs on those buffers, and again after one more
+    for k in (1, 2):
+        if k == 2:
+            ex.request.bind(sends[k], outs[k])
+        outs[k].fill_(0xA5)
+        gbx.startall([ex.request, other.request])
+        _complete(how, ex.request, side)
+        other.request.wait()
+        torch.cuda.synchronize()
+        assert_bytes_equal(outs[k].cpu().numpy(), want[k], f"{alg} {info} {how} batch, buffers {k}")
+
+
+def test_start_under_capture_is_refused():
+    """A graph=1 start launches with the buffers bound now, which a caller's graph would keep: it
+    returns ERR_CUDA inside a stream capture and works again after it."""
+    p = pt.config1()
+    x = payload(p, 3)
+    recv = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+    s = torch.cuda.Stream()
+    ex = gbx.Exchange(p, dev_bytes(x), recv, stream=s)
+    s.synchronize()
+    torch.cuda.synchronize()
+    probe = torch.zeros(4, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        probe.add_(1)
+        with pytest.raises(gbx.GbxError) as e:
+            ex.start()
+    assert e.value.code == gbx.ERR_CUDA
+    ex.start()
+    ex.wait()
+    assert_bytes_equal(recv.cpu().numpy(), oracle.standard(p, x), "after the capture")
