@@ -107,7 +107,7 @@ static Opts parse_info(const char *info) {
     if (o.block && !(o.block == 128 || o.block == 256 || o.block == 512 || o.block == 1024)) o.ok = false;
     if (o.timeout_ms <= 0 || o.min_run < 0 || o.piece < 0 || o.split_order < 0) o.ok = false;
     if (o.bulk < 0 || o.bulk > 2 || o.max_ctas < 0 || o.wait_limit < 0 || o.stream < 0 || o.stream > 2) o.ok = false;
-    if (o.form < -1 || o.form > 11) o.ok = false;
+    if (o.form < -1 || o.form > 14) o.ok = false;
     return o;
 }
 
@@ -210,6 +210,24 @@ static int stream_ok_for(const gbx_request_s *req, const int32_t *g, const int32
     return 1;
 }
 
+// The async gather takes flat gathers of 16-byte chunks, where it was measured ahead of the
+// register-pipelined and stream forms (512^3 stencil halo 558 us against 561-576 and 569); with
+// narrower chunks it was behind (2^20-row SpMV halo, 8 bytes: 45 us against 38).  Info stream=0
+// leaves it out with the other forms that stage in shared memory.
+static int agather_ok_for(const gbx_request_s *req, int max_vec) {
+    static int prepared = 0;
+    if (!req->allow_stream || max_vec < 16) return 0;
+    if (!prepared) {
+        if (gbx_agather_prepare() != GBX_SUCCESS) return 0;
+        prepared = 1;
+    }
+    return 1;
+}
+
+// The async gather's bulk stores write device memory only (their run is 16-byte aligned, as
+// every offset of a 16-byte vector op and every buffer bound to it).
+static void set_bulk_dst(CopyDesc &d) { d.bulk_dst = !host_mem(d.dst); }
+
 int gbx_make_copy_op(gbx_request_s *req, int level, const char *src, int src_role, char *dst, int dst_role,
                      const Seg *segs, int64_t nseg, const int32_t *idx, int64_t idx_len, int64_t nelem,
                      int64_t algo_bytes) {
@@ -261,6 +279,8 @@ int gbx_make_copy_op(gbx_request_s *req, int level, const char *src, int src_rol
         d.dst_flat0 = op.flat_dst0;
         op.algo_bytes_flat = 2 * nelem * req->elem_size + 4 * nelem;
         op.stream_ok = op.flat_ok && stream_ok_for(req, op.d_flat_idx, nullptr, op.max_vec);
+        op.ag_ok = op.flat_ok && agather_ok_for(req, op.max_vec);
+        set_bulk_dst(d);
     }
     if (req->allow_bulk && !host_mem(src) && !host_mem(dst)) {
         GBX_TRY(gbx_make_bulk(req, segs, nseg, nelem, src_role == ROLE_AGG && dst_role == ROLE_AGG, &op.d_bulk,
@@ -299,6 +319,8 @@ int gbx_make_flat_op(gbx_request_s *req, int level, const char *src, int src_rol
     d.flat = 1; d.flat_idx = g; d.dst_flat0 = dst0; d.src2 = src2; d.src2_role = src2_role;
     d.status = req->status_dev; d.wait_limit = req->wait_limit;
     op.stream_ok = stream_ok_for(req, g, nullptr, op.max_vec);
+    op.ag_ok = agather_ok_for(req, op.max_vec);
+    set_bulk_dst(d);
     const int64_t max_tiles = ceil_div(nelem * (req->elem_size / op.min_vec), GBX_TILE);
     GBX_TRY(req->mem.get(&op.d_tile_e0, max_tiles + 1));
     d.tile_e0 = op.d_tile_e0;
@@ -319,6 +341,7 @@ int gbx_make_flat2_op(gbx_request_s *req, int level, const char *src, int src_ro
     GBX_TRY(gbx_make_flat_op(req, level, src, src_role, src2, src2_role, dst, dst_role, gs, nelem, 0));
     HostOp &op = req->ops.back();
     op.cd.flat = 3;
+    op.ag_ok = 0;
     op.cd.flat_didx = gd;
     op.stream_ok = op.stream_ok && stream_ok_for(req, gs, gd, op.max_vec);
     op.algo_bytes = op.algo_bytes_flat = 2 * nelem * req->elem_size + 8 * nelem;
@@ -544,7 +567,8 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
     key.flat_ok = op.kind == 1 ? op.sfold_ok + 2 * (req->forced_form + 1)
                 : op.kind == 0 ? op.flat_ok + 2 * op.flat_only + 4 * ((op.cd.flat & 3) == 3) + 8 * op.bulk_ok +
                                      16 * op.scat_ok + 32 * (req->allow_bulk == 2) + 64 * op.stream_ok +
-                                     128 * (req->allow_stream == 2) + 256 * (req->forced_form + 1)   // forced forms tune apart
+                                     128 * (req->allow_stream == 2) + 256 * (req->forced_form + 1) +   // forced forms tune apart
+                                     8192 * op.ag_ok
                 : 0;
     int blocks[4] = {128, 256, 512, 1024};
     if (!req->autotune || req->forced_block) {
@@ -553,6 +577,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
         if (op.kind == 1) op.fold_form = op.sfold_ok && req->allow_stream == 2;
         if (op.kind == 0 && !op.flat_only) op.cd.flat = op.flat_ok && req->forced_flat != 0;
         if (op.kind == 0 && op.stream_ok && req->allow_stream == 2) op.cd.flat = (op.cd.flat & 3) == 3 ? 11 : 10;
+        if (op.kind == 0 && op.ag_ok && req->forced_form == 14) op.cd.flat = 14;
         if (op.kind == 0 && op.bulk_ok && req->allow_bulk == 2) op.cd.flat = 8;
         if (op.kind == 0 && op.scat_ok && req->allow_bulk == 2) op.cd.flat = 9;
         set_form_bytes(op);
@@ -595,6 +620,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
     else forms.push_back(0);
     if (op.kind == 0 && op.stream_ok && (op.flat_only || (op.flat_ok && req->forced_flat != 0)))
         forms.push_back((op.cd.flat & 3) == 3 ? 11 : 10);
+    if (op.kind == 0 && op.ag_ok && (op.flat_only || (op.flat_ok && req->forced_flat != 0))) forms.push_back(14);
     // (bulk_ok implies 16-byte aligned pieces; between the library's own aggregates the element
     // size need not be a multiple of 16)
     if (op.kind == 0 && op.bulk_ok && req->forced_flat != 1) forms.push_back(8);
@@ -609,15 +635,15 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
         if (op.kind == 0) op.cd.flat = form;
         else op.fold_form = form;
         const bool pipe = op.kind == 0 && form >= 4 && form < 8, bulk = op.kind == 0 && (form == 8 || form == 9);
-        const bool strm = op.kind == 0 ? form >= 10 : form == 1;
+        const bool strm = op.kind == 0 ? form >= 10 : form == 1, ag = op.kind == 0 && form == 14;
         // (the op's tile tables are sized for min_vec: no width below it)
         // (the bulk and scatter kernels do not use the vector width: one pass, at max_vec)
-        for (int vec = op.max_vec; vec >= (bulk ? op.max_vec : strm ? std::max(4, op.min_vec) : op.min_vec);
+        for (int vec = op.max_vec; vec >= (bulk || ag ? op.max_vec : strm ? std::max(4, op.min_vec) : op.min_vec);
              vec >>= 1) {
             GBX_TRY(set_vec(req, op, vec));
             // stream forms: persistent grid only; block 256 and 512 select the two wide shapes,
             // block 128 the narrow one, offered only with one chunk per element (cpe == 1)
-            const int b0 = pipe ? 2 : form == 8 ? 3 : strm ? (op.kind == 0 && op.cd.cpe == 1 && vec <= 8 ? 0 : 1) : 0;
+            const int b0 = pipe ? 2 : form == 8 ? 3 : ag ? 0 : strm ? (op.kind == 0 && op.cd.cpe == 1 && vec <= 8 ? 0 : 1) : 0;
             for (int bi = b0; bi < (strm ? 3 : 4); bi++)
                 for (int pers = 1; pers >= (pipe || strm ? 1 : 0); pers--) {
                     float ms = 0;
@@ -661,12 +687,14 @@ static int tune_launch(LevelLaunch &L, cudaStream_t st) {
     float best = 1e30f;
     int bb = L.block, bg = L.grid, bf = L.flat;
     cudaError_t e = cudaSuccess;
-    // a stream-form launch is also timed in the plain flat form (same tiles, same bytes)
-    const int nforms = (L.flat == 10 || L.flat == 11) ? 2 : 1;
+    // a stream-form launch is also timed in the plain flat form and, for gathers, in the async
+    // form (same tiles, same bytes)
+    const int nforms = L.flat == 10 && L.vec == 16 ? 3 : L.flat == 10 || L.flat == 11 ? 2 : 1;
+    const int first = L.flat;
     for (int fi = 0; fi < nforms && e == cudaSuccess; fi++) {
-        const int fl = fi == 0 ? L.flat : (L.flat == 10 ? 1 : 3);
+        const int fl = fi == 0 ? first : fi == 2 ? 14 : (first == 10 ? 1 : 3);
         const bool strm = fl >= 10;
-        for (int bi = strm ? (L.one && L.vec <= 8 ? 0 : 1) : 0; bi < (strm ? 3 : 4) && e == cudaSuccess; bi++)
+        for (int bi = strm ? (fl == 14 || (L.one && L.vec <= 8) ? 0 : 1) : 0; bi < (strm ? 3 : 4) && e == cudaSuccess; bi++)
             for (int pers = 1; pers >= (strm ? 1 : 0) && e == cudaSuccess; pers--) {
                 const int blk = blocks[bi];
                 const int grid = grid_for(L.kind, L.dtype, L.vec, fl, blk, pers, L.total_tiles, L.max_ctas);
@@ -1551,6 +1579,7 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
         if (op.kind == 0) {
             if (op.cd.src_role == ROLE_SRC) op.cd.src = ns;
             if (op.cd.dst_role == ROLE_DST) op.cd.dst = nd;
+            set_bulk_dst(op.cd);
         } else {
             if (op.fd.out_role == ROLE_DST) op.fd.out = nd;
             if (op.fd.a_role == ROLE_SRC) op.fd.bufA = ns;
@@ -1583,6 +1612,7 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
             HostOp &c = b->widened[k];
             c.cd.src = o.cd.src;
             c.cd.dst = o.cd.dst;
+            c.cd.bulk_dst = o.cd.bulk_dst;
             if (((uintptr_t)c.cd.src | (uintptr_t)c.cd.dst) & (uintptr_t)(c.cd.vec - 1)) {
                 stale.push_back(b);
                 break;

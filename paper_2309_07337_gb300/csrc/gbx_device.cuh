@@ -44,6 +44,7 @@ struct CopyDesc {
     int32_t flat;
     const int32_t *flat_idx;
     int64_t dst_flat0;
+    int32_t bulk_dst;   // dst is device memory: the bulk-copy engine may write the run
     // flat form with two sources: an index with bit 31 set reads src2 (e.g. the receive
     // aggregate) instead of src
     const char *src2;

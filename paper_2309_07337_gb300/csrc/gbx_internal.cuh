@@ -153,6 +153,7 @@ struct HostOp {
     int64_t nbulk;
     int stream_ok;          // the flat form's index arrays are 16-byte aligned and padded: the
                             // stream forms (10 gather, 11 two-index) are available
+    int ag_ok;              // a flat gather with the async form (14) available
     int sfold_ok;           // fold: records and terms aligned and padded, one payload class: the
                             // stream form of the fold is available
     int fold_form;          // fold: 0 the fold kernel, 1 its stream form (tuned)
@@ -304,6 +305,7 @@ int gbx_make_bulk(gbx_request_s *req, const Seg *segs, int64_t nseg, int64_t nel
 int gbx_bulk_prepare(void);
 int gbx_scatter_prepare(void);
 int gbx_stream_prepare(void);
+int gbx_agather_prepare(void);
 int gbx_check_data_buf(const void *p, int64_t bytes);   // GBX_ERR_ARG unless the GPU can address p
 // Scatter-form windows of a two-index copy whose pairs are sorted by source (gs, the source
 // indices, decide the windows) and whose index arrays carry 4 elements of padding; *ok = 0

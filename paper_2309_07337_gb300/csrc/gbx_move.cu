@@ -943,6 +943,136 @@ int gbx_stream_prepare(void) {
     return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
 }
 
+// ------------------------------------------------------------ async gather
+// Async form of the flat gather of 16-byte chunks (destinations one contiguous run): every warp
+// gathers its chunks straight into shared memory (cp.async, one chunk per lane and step) and
+// has the bulk-copy engine write them out as one contiguous store, through a ring of S stages
+// of its own.  A unit is 32 * K consecutive chunks of the op's tiles; a warp keeps the loads of
+// S - 2 units in flight while the store of the unit before them drains, and loads a unit's
+// indices one unit ahead.  The gathers hold no registers and the stores no load / store slots,
+// so the bytes in flight per SM are set by the ring (192 KB) and not by the register file
+// (32 KB with one chunk per thread at full occupancy).  A warp waits only for copies it has
+// issued itself (cp.async.wait_group), never on a flag.  Bound by HBM: 512^3 stencil halo (64-byte
+// points, 3.57 GB of whole 128-byte lines) 558 us = 6.4 TB/s of line traffic; register-pipelined
+// form 561-576 us, stream form 569 us.  Chunks of 4 and 8 bytes gain nothing (2^20-row SpMV halo
+// 45 us, stream form 38: a request per line and element bounds them, not bytes in flight).
+// Destinations in host memory (bulk_dst = 0) are stored by the lanes.
+template <int K, int S, int NW, int PS, typename L>
+__global__ void __launch_bounds__(NW * 32, PS) gbx_agather_kernel(const __grid_constant__ L list) {
+    constexpr int D = S - 2;                      // units of loads in flight
+    constexpr int UNIT = 32 * K, SUB = GBX_TILE / UNIT;
+    extern __shared__ __align__(128) unsigned char gbx_agather_smem[];
+    pdl_trigger();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint4 *ring = reinterpret_cast<uint4 *>(gbx_agather_smem) + warp * S * UNIT;
+    const uint32_t sring = (uint32_t)__cvta_generic_to_shared(ring);
+    const int64_t stride = (int64_t)gridDim.x * NW, nunits = list.tiles() * SUB;
+    int64_t u = (int64_t)blockIdx.x * NW + warp;  // next unit to load
+    int64_t us = u;                               // next unit to store
+
+    // unit x: its op, its first chunk c0, the element e0 that holds it and the chunk r0 in it
+    auto locate = [&](int64_t x, int64_t &c0, int64_t &e0, uint32_t &r0) {
+        int64_t lt;
+        const CopyDesc *d = list.at(x / SUB, lt);
+        const int cpe = d->cpe, sh = d->cpe_shift;
+        c0 = lt * GBX_TILE + (x % SUB) * UNIT;
+        e0 = sh >= 0 ? c0 >> sh : c0 >> 32 ? c0 / cpe : (int64_t)((uint32_t)c0 / (uint32_t)cpe);
+        r0 = (uint32_t)(c0 - e0 * cpe);
+        return d;
+    };
+    uint32_t gi[K];   // indices of the next unit's chunks (0 past the op's end)
+    auto indices = [&](int64_t x) {
+        int64_t c0, e0;
+        uint32_t r0;
+        const CopyDesc *d = locate(x, c0, e0, r0);
+        const int64_t left = d->nchunks - c0;
+        const int32_t *g = d->flat_idx + e0;
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            const int x0 = k * 32 + lane;
+            gi[k] = x0 < left ? (uint32_t)__ldg(g + unit_of(r0 + (uint32_t)x0, d->cpe, d->cpe_shift, d->cpe_magic)) : 0u;
+        }
+    };
+    if (u < nunits) indices(u);
+    pdl_wait();
+    for (int i = 0; us < nunits; i++) {
+        if (u < nunits) {
+            const int q = i % S;
+            if (i >= S) {   // the last store from this stage has read it
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                __syncwarp();
+            }
+            int64_t c0, e0;
+            uint32_t r0;
+            const CopyDesc *d = locate(u, c0, e0, r0);
+            const int64_t left = d->nchunks - c0, s = d->elem_size;
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                const int x0 = k * 32 + lane;
+                if (x0 < left) {
+                    const uint32_t xx = r0 + (uint32_t)x0;
+                    const uint32_t j = xx - unit_of(xx, d->cpe, d->cpe_shift, d->cpe_magic) * (uint32_t)d->cpe;
+                    const char *b = (gi[k] & GBX_FLAT_SRC2) ? d->src2 : d->src;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                                 ::"r"(sring + (uint32_t)((q * UNIT + x0) * 16)),
+                                 "l"(b + (int64_t)(gi[k] & ~GBX_FLAT_SRC2) * s + (int64_t)(j * 16))
+                                 : "memory");
+                }
+            }
+            u += stride;
+            if (u < nunits) indices(u);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (i < D) continue;
+        asm volatile("cp.async.wait_group %0;" ::"n"(D) : "memory");   // unit us has landed
+        const int q = (i - D) % S;
+        int64_t lt;
+        const CopyDesc *d = list.at(us / SUB, lt);
+        const int64_t c0 = lt * GBX_TILE + (us % SUB) * UNIT;
+        const int n = (int)min((int64_t)UNIT, d->nchunks - c0);   // (0 or less: past the op's last chunk)
+        us += stride;
+        if (n > 0) {
+            char *out = d->dst + d->dst_flat0 + c0 * 16;
+            if (d->bulk_dst) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                                 ::"l"(out), "r"(sring + (uint32_t)(q * UNIT * 16)), "r"((uint32_t)(n * 16))
+                                 : "memory");
+            } else {
+                for (int x = lane; x < n; x += 32) stv<16>(out + (int64_t)x * 16, ring[q * UNIT + x]);   // its own chunks
+            }
+        }
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");   // one store group per unit
+    }
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+// Shapes of the async gather, chosen by the launch's block value: steps per unit, stages, warps
+// per CTA, CTAs per SM (each fills 192 KB of shared memory per SM).
+template <typename L>
+static cudaError_t agather_launch(int block, int grid, cudaStream_t st, bool dep, const L &l) {
+    if (block <= 128) return launch(gbx_agather_kernel<8, 4, 4, 3, L>, grid, 128, 65536, st, dep, l);
+    if (block <= 256) return launch(gbx_agather_kernel<4, 6, 4, 4, L>, grid, 128, 49152, st, dep, l);
+    return launch(gbx_agather_kernel<4, 4, 8, 3, L>, grid, 256, 65536, st, dep, l);
+}
+
+static int agather_per_sm(int block) { return block <= 128 || block > 256 ? 3 : 4; }
+
+template <int K, int S, int NW, int PS>
+static cudaError_t agather_attr() {
+    return smem_attr(gbx_agather_kernel<K, S, NW, PS, OneOp<CopyDesc>>, gbx_agather_kernel<K, S, NW, PS, OpList<CopyDesc>>,
+                     NW * S * K * 512);
+}
+
+int gbx_agather_prepare(void) {
+    cudaError_t e = agather_attr<8, 4, 4, 3>();
+    if (e == cudaSuccess) e = agather_attr<4, 6, 4, 4>();
+    if (e == cudaSuccess) e = agather_attr<4, 4, 8, 3>();
+    return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
+}
+
 int gbx_bulk_status_take(int *status) {
     int zero = 0;
     GBX_CUDA_TRY(cudaMemcpyFromSymbol(status, gbx_bulk_status, sizeof(int)));
@@ -1353,6 +1483,7 @@ int gbx_occupancy(int kind, int dtype, int vec, int block, int flat) {
     if (kind == 0 && flat == 8) return 1;   // bulk kernel: one CTA per SM (its ring)
     if (kind == 0 && flat == 9) return scatter_shape(block).per_sm;
     if (kind == 0 && flat >= 10 && flat <= 13) return stream_shape(block).per_sm;
+    if (kind == 0 && flat == 14) return agather_per_sm(block);
     if (kind == 0) block = pipe_block(flat, block);
     const void *f = kind == 0 ? (const void *)copy_fn<OneOp<CopyDesc>>(vec, block, flat)
                               : (const void *)fold_fn<OneOp<FoldDesc>>(dtype, vec, block);
@@ -1377,6 +1508,7 @@ static cudaError_t launch_copy(const L &l, int nops, int vec, int flat, int bloc
         if (block <= 128 && !(flat >= 12 && vec <= 8)) block = 256;   // the narrow shape needs ONE, vec <= 8
         return stream_launch(vec, flat, block, grid, st, dep, l);
     }
+    if (flat == 14) return agather_launch(block, grid, st, dep, l);   // async gather (vec 16)
     if ((flat == 5 || flat == 7) && nops > 1) flat -= 4;   // the pipelined kernels take one op
     block = pipe_block(flat, block);
     return launch(copy_fn<L>(vec, block, flat), grid, block, 0, st, dep, l);
