@@ -107,7 +107,7 @@ static Opts parse_info(const char *info) {
     if (o.block && !(o.block == 128 || o.block == 256 || o.block == 512 || o.block == 1024)) o.ok = false;
     if (o.timeout_ms <= 0 || o.min_run < 0 || o.piece < 0 || o.split_order < 0) o.ok = false;
     if (o.bulk < 0 || o.bulk > 2 || o.max_ctas < 0 || o.wait_limit < 0 || o.stream < 0 || o.stream > 2) o.ok = false;
-    if (o.form < -1 || o.form > 14) o.ok = false;
+    if (o.form < -1 || o.form > 15) o.ok = false;
     return o;
 }
 
@@ -228,6 +228,36 @@ static int agather_ok_for(const gbx_request_s *req, int max_vec) {
 // every offset of a 16-byte vector op and every buffer bound to it).
 static void set_bulk_dst(CopyDesc &d) { d.bulk_dst = !host_mem(d.dst); }
 
+// The window form reads its windows with the bulk-copy engine from 16-byte aligned device memory
+// (every window starts at a multiple of 16 bytes), with plain loads otherwise.
+static void set_win_bulk(CopyDesc &d) {
+    d.win_bulk = d.src && !((uintptr_t)d.src & 15) && !host_mem(d.src);
+    d.win_bulk2 = d.src2 && !((uintptr_t)d.src2 & 15) && !host_mem(d.src2);
+}
+
+// Elements of the buffer an op's pointer of this role reads.
+static int64_t role_elems(const gbx_request_s *req, int role) {
+    return (role == ROLE_SRC ? req->src_bytes : role == ROLE_AGG ? 2 * req->Ur * req->elem_size : 0) / req->elem_size;
+}
+
+static int add_window(gbx_request_s *req, HostOp &op) {
+    CopyDesc &d = op.cd;
+    if (!req->allow_stream || op.max_vec != req->elem_size) return GBX_SUCCESS;   // one chunk per element
+    WinTables t;
+    GBX_TRY(gbx_make_window(req, d.flat_idx, d.nelem, role_elems(req, d.src_role),
+                            d.src2 ? role_elems(req, d.src2_role) : 0, &t, &op.win_ok));
+    if (!op.win_ok) return GBX_SUCCESS;
+    d.win = t.pieces;
+    d.win_idx = t.idx;
+    d.win_grp = t.grp;
+    d.win_run = t.run;
+    d.win_elems = t.elems;
+    d.nwin = op.nwin = t.npieces;
+    op.algo_bytes_win = d.nelem * (2 * req->elem_size + 2) + d.nelem / 4 + 4 * t.nruns + 32 * t.npieces;
+    set_win_bulk(d);
+    return GBX_SUCCESS;
+}
+
 int gbx_make_copy_op(gbx_request_s *req, int level, const char *src, int src_role, char *dst, int dst_role,
                      const Seg *segs, int64_t nseg, const int32_t *idx, int64_t idx_len, int64_t nelem,
                      int64_t algo_bytes) {
@@ -281,6 +311,7 @@ int gbx_make_copy_op(gbx_request_s *req, int level, const char *src, int src_rol
         op.stream_ok = op.flat_ok && stream_ok_for(req, op.d_flat_idx, nullptr, op.max_vec);
         op.ag_ok = op.flat_ok && agather_ok_for(req, op.max_vec);
         set_bulk_dst(d);
+        if (op.flat_ok && idx) GBX_TRY(add_window(req, op));
     }
     if (req->allow_bulk && !host_mem(src) && !host_mem(dst)) {
         GBX_TRY(gbx_make_bulk(req, segs, nseg, nelem, src_role == ROLE_AGG && dst_role == ROLE_AGG, &op.d_bulk,
@@ -295,7 +326,7 @@ int gbx_make_copy_op(gbx_request_s *req, int level, const char *src, int src_rol
 }
 
 int gbx_make_flat_op(gbx_request_s *req, int level, const char *src, int src_role, const char *src2, int src2_role,
-                     char *dst, int dst_role, const int32_t *g, int64_t nelem, int64_t dst0) {
+                     char *dst, int dst_role, const int32_t *g, int64_t nelem, int64_t dst0, bool windows) {
     if (nelem <= 0) return GBX_SUCCESS;
     HostOp op;
     memset(&op, 0, sizeof(op));
@@ -321,6 +352,7 @@ int gbx_make_flat_op(gbx_request_s *req, int level, const char *src, int src_rol
     op.stream_ok = stream_ok_for(req, g, nullptr, op.max_vec);
     op.ag_ok = agather_ok_for(req, op.max_vec);
     set_bulk_dst(d);
+    if (windows) GBX_TRY(add_window(req, op));
     const int64_t max_tiles = ceil_div(nelem * (req->elem_size / op.min_vec), GBX_TILE);
     GBX_TRY(req->mem.get(&op.d_tile_e0, max_tiles + 1));
     d.tile_e0 = op.d_tile_e0;
@@ -338,7 +370,7 @@ static bool pairs_in_source_order(const gbx_request_s *req) {
 
 int gbx_make_flat2_op(gbx_request_s *req, int level, const char *src, int src_role, const char *src2, int src2_role,
                       char *dst, int dst_role, const int32_t *gs, const int32_t *gd, int64_t nelem) {
-    GBX_TRY(gbx_make_flat_op(req, level, src, src_role, src2, src2_role, dst, dst_role, gs, nelem, 0));
+    GBX_TRY(gbx_make_flat_op(req, level, src, src_role, src2, src2_role, dst, dst_role, gs, nelem, 0, false));
     HostOp &op = req->ops.back();
     op.cd.flat = 3;
     op.ag_ok = 0;
@@ -421,6 +453,11 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
     return GBX_SUCCESS;
 }
 
+// Tiles of a copy in form `flat`: pieces, windows, or GBX_TILE chunks.
+static int64_t form_tiles(const HostOp &op, int flat) {
+    return flat == 8 ? op.nbulk : flat == 9 ? op.nscat : (flat & 31) == 15 ? op.nwin : ceil_div(op.cd.nchunks, GBX_TILE);
+}
+
 static int64_t op_tiles(const HostOp &op) { return op.kind == 0 ? op.cd.ntiles : op.fd.ntiles; }
 
 static int upload_desc(gbx_request_s *req, HostOp &op) {
@@ -445,14 +482,13 @@ static int set_vec(gbx_request_s *req, HostOp &op, int vec) {
         d.vec = vec; d.cpe = cpe; d.cpe_shift = shift; d.cpe_magic = magic;
         d.nchunks = d.nelem * cpe;
         d.ntiles = ceil_div(d.nchunks, GBX_TILE);
-        if (d.flat == 8)   // bulk form: one "tile" per piece, no tile table
-            d.ntiles = d.nbulk;
-        else if (d.flat == 9)   // scatter form: one "tile" per source window
-            d.ntiles = d.nscat;
+        if (d.flat == 8 || d.flat == 9)   // bulk, scatter: no tile table
+            ;
         else if (op.flat_only)
             GBX_TRY(gbx_build_tile_meta(nullptr, 0, cpe, d.ntiles, nullptr, op.d_tile_e0, req->stream));
         else
             GBX_TRY(gbx_build_tile_meta(d.segs, d.nseg, cpe, d.ntiles, op.d_tile_seg, op.d_tile_e0, req->stream));
+        d.ntiles = form_tiles(op, d.flat);
     } else {
         FoldDesc &d = op.fd;
         d.vec = vec; d.cpe = cpe; d.cpe_shift = shift; d.cpe_magic = magic;
@@ -486,9 +522,12 @@ static int op_flat(const HostOp &op) { return op.kind == 0 ? op.cd.flat : op.fol
 // every op of the launch has one chunk per element (one).
 static int launch_code(int flat, int one) { return (flat == 10 || flat == 11) && one ? flat + 2 : flat; }
 
+// The window form's launch code carries the window size (15: 1024 elements, 47: 2048).
+static int window_code(const CopyDesc &d) { return d.win_elems > 1024 ? 47 : 15; }
+
 static cudaError_t launch_op_alone(gbx_request_s *req, HostOp &op, int block, int persistent) {
     const int64_t tiles = op_tiles(op);
-    const int vec = op_vec(op), flat = op_flat(op);
+    const int vec = op_vec(op), flat = op.kind == 0 && op_flat(op) == 15 ? window_code(op.cd) : op_flat(op);
     const int grid = grid_for(op.kind, req->dtype, vec, flat, block, persistent, tiles, req->max_ctas);
     if (op.kind == 0)
         return gbx_launch_copy({&op.cd, nullptr, nullptr, 1, tiles}, vec, launch_code(flat, op.cd.cpe == 1), block, grid,
@@ -554,6 +593,7 @@ static void set_form_bytes(HostOp &op) {
     if (op.kind != 0) return;
     op.algo_bytes = op.cd.flat == 8 ? op.algo_bytes_bulk
                   : op.cd.flat == 9 ? op.algo_bytes_scat
+                  : op.cd.flat == 15 ? op.algo_bytes_win
                   : op.cd.flat ? op.algo_bytes_flat : op.algo_bytes_seg;
 }
 
@@ -568,7 +608,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
                 : op.kind == 0 ? op.flat_ok + 2 * op.flat_only + 4 * ((op.cd.flat & 3) == 3) + 8 * op.bulk_ok +
                                      16 * op.scat_ok + 32 * (req->allow_bulk == 2) + 64 * op.stream_ok +
                                      128 * (req->allow_stream == 2) + 256 * (req->forced_form + 1) +   // forced forms tune apart
-                                     8192 * op.ag_ok
+                                     8192 * op.ag_ok + 16384 * op.win_ok
                 : 0;
     int blocks[4] = {128, 256, 512, 1024};
     if (!req->autotune || req->forced_block) {
@@ -578,6 +618,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
         if (op.kind == 0 && !op.flat_only) op.cd.flat = op.flat_ok && req->forced_flat != 0;
         if (op.kind == 0 && op.stream_ok && req->allow_stream == 2) op.cd.flat = (op.cd.flat & 3) == 3 ? 11 : 10;
         if (op.kind == 0 && op.ag_ok && req->forced_form == 14) op.cd.flat = 14;
+        if (op.kind == 0 && op.win_ok && req->forced_form == 15) op.cd.flat = 15;
         if (op.kind == 0 && op.bulk_ok && req->allow_bulk == 2) op.cd.flat = 8;
         if (op.kind == 0 && op.scat_ok && req->allow_bulk == 2) op.cd.flat = 9;
         set_form_bytes(op);
@@ -621,6 +662,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
     if (op.kind == 0 && op.stream_ok && (op.flat_only || (op.flat_ok && req->forced_flat != 0)))
         forms.push_back((op.cd.flat & 3) == 3 ? 11 : 10);
     if (op.kind == 0 && op.ag_ok && (op.flat_only || (op.flat_ok && req->forced_flat != 0))) forms.push_back(14);
+    if (op.kind == 0 && op.win_ok && req->forced_flat != 0) forms.push_back(15);
     // (bulk_ok implies 16-byte aligned pieces; between the library's own aggregates the element
     // size need not be a multiple of 16)
     if (op.kind == 0 && op.bulk_ok && req->forced_flat != 1) forms.push_back(8);
@@ -635,7 +677,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
         if (op.kind == 0) op.cd.flat = form;
         else op.fold_form = form;
         const bool pipe = op.kind == 0 && form >= 4 && form < 8, bulk = op.kind == 0 && (form == 8 || form == 9);
-        const bool strm = op.kind == 0 ? form >= 10 : form == 1, ag = op.kind == 0 && form == 14;
+        const bool strm = op.kind == 0 ? form >= 10 : form == 1, ag = op.kind == 0 && form >= 14;
         // (the op's tile tables are sized for min_vec: no width below it)
         // (the bulk and scatter kernels do not use the vector width: one pass, at max_vec)
         for (int vec = op.max_vec; vec >= (bulk || ag ? op.max_vec : strm ? std::max(4, op.min_vec) : op.min_vec);
@@ -749,6 +791,16 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
                         int what = 3) {
     int nlev = 0;
     for (HostOp *op : ops) nlev = std::max(nlev, op->level + 1);
+    // A batch runs a level's window-capable gathers of one vector width in the window form, all of
+    // them, when at least half of their elements were tuned to it alone (one launch for each
+    // form costs more than the form that suits an op less).
+    std::map<std::pair<int, int>, int64_t> by_window;   // (level, vector width) -> elements for minus against
+    for (const HostOp *op : ops)
+        if (op->kind == 0 && op->win_ok)
+            by_window[{op->level, op_vec(*op)}] += op->cd.flat == 15 ? op->units : -op->units;
+    auto windows = [&](const HostOp &op) {
+        return op.kind == 0 && op.win_ok && op_vec(op) == op.max_vec && by_window[{op.level, op_vec(op)}] >= 0;
+    };
     for (int lv = 0; lv < nlev; lv++)
         for (int kind = 0; kind < 2; kind++) {
             std::vector<std::vector<size_t>> groups;
@@ -765,11 +817,12 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
                 // it, else the plain flat launch
                 const int f0 = op_flat(*op);
                 const bool strm = op->stream_ok && op_vec(*op) >= 4;
-                const int form = !batch || f0 == 8 || f0 == 9 ? f0
-                               : op->flat_ok ? ((f0 & 3) == 3 ? (strm ? 11 : 3) : (strm ? 10 : 1)) : 0;
+                const int form = !batch ? (kind == 0 && f0 == 15 ? window_code(op->cd) : f0) : f0 == 8 || f0 == 9 ? f0
+                               : windows(*op) ? window_code(op->cd)
+                               : op->flat_ok ? (op->cd.flat_didx ? (strm ? 11 : 3) : (strm ? 10 : 1)) : 0;
                 // stream-form copies with one chunk per element get a launch of their own, which
                 // runs the specialised kernel (one op with more chunks would hold back the rest)
-                const int one = kind == 0 && form >= 10 && op->cd.cpe == 1 ? 16 : 0;
+                const int one = kind == 0 && form >= 10 && form < 14 && op->cd.cpe == 1 ? 64 : 0;
                 std::pair<int, int> k = kind ? std::make_pair(dtypes[i] + 8 * op->fold_form, op_vec(*op))
                                              : std::make_pair(form + one, op_vec(*op));
                 size_t g = 0;
@@ -786,7 +839,8 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
                 L.vec = op_vec(*ops[groups[g][0]]);
                 // (a pooled class of one op keeps the form it was tuned to, pipelined included)
                 L.flat = kind ? ops[groups[g][0]]->fold_form
-                              : (groups[g].size() == 1 ? op_flat(*ops[groups[g][0]]) : keys[g].first & 15);
+                              : (groups[g].size() == 1 && (keys[g].first & 15) != 15 && op_flat(*ops[groups[g][0]]) != 15
+                                     ? op_flat(*ops[groups[g][0]]) : keys[g].first & 63);
                 L.one_op = !batch && groups[g].size() == 1 ? (int)groups[g][0] : -1;
                 L.one = 1;
                 for (size_t i : groups[g])
@@ -796,7 +850,7 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
                 const HostOp *big = ops[groups[g][0]];
                 for (size_t i : groups[g]) {
                     ptrs.push_back(ops[i]->d_desc);
-                    pre.push_back(pre.back() + op_tiles(*ops[i]));
+                    pre.push_back(pre.back() + (kind ? op_tiles(*ops[i]) : form_tiles(*ops[i], L.flat)));
                     if (op_tiles(*ops[i]) > op_tiles(*big)) big = ops[i];
                 }
                 L.total_tiles = pre.back();
@@ -1586,6 +1640,7 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
             if (op.cd.src_role == ROLE_SRC) op.cd.src = ns;
             if (op.cd.dst_role == ROLE_DST) op.cd.dst = nd;
             set_bulk_dst(op.cd);
+            if (op.win_ok) set_win_bulk(op.cd);
         } else {
             if (op.fd.out_role == ROLE_DST) op.fd.out = nd;
             if (op.fd.a_role == ROLE_SRC) op.fd.bufA = ns;
@@ -1619,6 +1674,7 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
             c.cd.src = o.cd.src;
             c.cd.dst = o.cd.dst;
             c.cd.bulk_dst = o.cd.bulk_dst;
+            c.cd.win_bulk = o.cd.win_bulk;
             if (((uintptr_t)c.cd.src | (uintptr_t)c.cd.dst) & (uintptr_t)(c.cd.vec - 1)) {
                 stale.push_back(b);
                 break;

@@ -59,6 +59,15 @@ struct CopyDesc {
     // scattered from shared memory by the threads
     const struct ScatterPiece *scat;
     int64_t nscat;
+    // window form (flat == 15) of a flat gather with one chunk per element: the elements grouped by
+    // source window, each window read by the bulk-copy engine and gathered from shared memory
+    const struct WinPiece *win;
+    const uint16_t *win_idx;      // per slot: element of the window
+    const uint2 *win_grp;         // per 32 slots: run starts (bit mask), runs started before
+    const int32_t *win_run;       // per run: destination element minus slot
+    int64_t nwin;
+    int32_t win_elems;            // source elements per window: 1024 or 2048
+    int32_t win_bulk, win_bulk2;  // src / src2 is 16-byte aligned device memory
     // the waiting kernels (bulk, scatter): the request's status word (host-mapped memory,
     // read by gbx_wait / gbx_test), set to 1 when a bounded wait gave up and 2 when a piece
     // failed its in-kernel check; and the spin limit of their main waits (the waits that
@@ -79,6 +88,17 @@ struct ScatterPiece {
     int32_t len, n, nrun, pad;
     uint16_t run_off[GBX_SCAT_RUNS], run_len[GBX_SCAT_RUNS];
 };
+
+// One piece of a window-form gather: its n slots k = 0 .. n-1 (at p * GBX_WIN_N + k in win_idx, for
+// piece p) read element win_idx of the `bytes` source bytes at `src` (of src2 when buf is set)
+// and write destination element win_run[run] + k, run = the number of run starts up to k minus
+// one (runs of piece p at p * GBX_WIN_RUNS).
+struct WinPiece {
+    int64_t src;
+    int32_t bytes, n, nrun, buf, pad[2];
+};
+#define GBX_WIN_N 2048        // slots per piece
+#define GBX_WIN_RUNS 1024     // runs per piece at most
 
 // One piece of a bulk-form copy: len bytes (a multiple of 16, at most GBX_BULK_BYTES) from
 // byte src of the op's source to byte dst of its destination, both 16-byte aligned.

@@ -154,6 +154,9 @@ struct HostOp {
     int stream_ok;          // the flat form's index arrays are 16-byte aligned and padded: the
                             // stream forms (10 gather, 11 two-index) are available
     int ag_ok;              // a flat gather with the async form (14) available
+    int win_ok;             // a flat gather with the window form (15) available
+    int64_t nwin;
+    int64_t algo_bytes_win;
     int sfold_ok;           // fold: records and terms aligned and padded, one payload class: the
                             // stream form of the fold is available
     int fold_form;          // fold: 0 the fold kernel, 1 its stream form (tuned)
@@ -292,7 +295,7 @@ int gbx_validate_program(gbx_request_s *req, int64_t agg_bytes);
 int gbx_split_runs(gbx_request_s *req, const Seg *segs, int64_t nseg, const int32_t *idx, int64_t nelem,
                    int min_run, Seg **out, int64_t *out_nseg);
 int gbx_make_flat_op(gbx_request_s *req, int level, const char *src, int src_role, const char *src2, int src2_role,
-                     char *dst, int dst_role, const int32_t *g, int64_t nelem, int64_t dst0);
+                     char *dst, int dst_role, const int32_t *g, int64_t nelem, int64_t dst0, bool windows);
 int gbx_split_single_rows(gbx_request_s *req, const int64_t *row_ptr, const int64_t *row_out, const int64_t *terms,
                           int64_t nrows, int32_t **gs, int32_t **gd, int64_t *nsingle, int64_t **row_ptr2,
                           int64_t **row_out2, int64_t **terms2, int64_t *nmulti, int64_t *nmterms, int *ok);
@@ -304,6 +307,19 @@ int gbx_make_bulk(gbx_request_s *req, const Seg *segs, int64_t nseg, int64_t nel
                   int *ok);
 int gbx_bulk_prepare(void);
 int gbx_scatter_prepare(void);
+// Window-form tables of a flat gather of nelem elements of s bytes (g: source element of each,
+// bit 31 = second source); *ok = 0 where the form does not apply (see gbx_make_window).
+struct WinTables {
+    WinPiece *pieces;
+    uint16_t *idx;
+    uint2 *grp;
+    int32_t *run;
+    int64_t npieces, nruns;
+    int elems;   // source elements per window
+};
+int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t src_elems, int64_t src2_elems,
+                    WinTables *t, int *ok);
+int gbx_window_prepare(void);
 int gbx_stream_prepare(void);
 int gbx_agather_prepare(void);
 int gbx_check_data_buf(const void *p, int64_t bytes);   // GBX_ERR_ARG unless the GPU can address p

@@ -1073,6 +1073,215 @@ int gbx_agather_prepare(void) {
     return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
 }
 
+// ------------------------------------------------------------------ window
+// Window form of a flat gather of elements of VEC bytes (tables: WinPiece).  Warp 0 is the
+// producer: per piece it has the bulk-copy engine read the source window and the piece's tables
+// into one of S shared-memory stages (or, from a source that is not 16-byte aligned device
+// memory, its lanes copy the window), completing on the stage's "full" mbarrier.  The consumer
+// warps pick the elements out of the window and store them: 32 consecutive slots of a piece per
+// warp and step, whose destinations are runs of consecutive elements.  The element index costs 2
+// bytes and its share of a run instead of 4, every source line is read whole by the copy
+// engine, and no load of a single element goes through L1.  That is what bounds the other forms
+// here: a request to L2 and an L1 line for every scattered element (2^20-row SpMV halo, 10.8 M
+// elements of 8 bytes: L1-to-L2 requests 55 %, DRAM 27 % of peak).  The halo took 39.0 us in the
+// best of them and takes 30.3 (fp32: 28.5 -> 21.0), its locality form 63.5 -> 52.5, a start of 16
+// uneven patterns 115 -> 78; now shared-memory and store wavefronts (54 %) and the 2-CTA ramp
+// weigh most.  Waits bounded as in the stream form.
+#define GBX_WIN_TABLES (GBX_WIN_N * 2 + GBX_WIN_N / 32 * 8 + GBX_WIN_RUNS * 4)
+
+template <int VEC, int WE, int NT, int S, int PS, typename L>
+__global__ void __launch_bounds__(NT, PS) gbx_window_kernel(const __grid_constant__ L list) {
+    typedef typename VecT<VEC>::T V;
+    constexpr int NCW = NT / 32 - 1, U = 4;
+    constexpr int WB = WE * VEC, STAGE = WB + GBX_WIN_TABLES;
+    constexpr int OFF_IDX = WB, OFF_GRP = OFF_IDX + GBX_WIN_N * 2, OFF_RUN = OFF_GRP + GBX_WIN_N / 32 * 8;
+    extern __shared__ __align__(128) unsigned char gbx_window_smem[];
+    __shared__ __align__(8) uint64_t full[S], empty[S];
+    __shared__ char *dst_s[S];
+    __shared__ int n_s[S];
+    __shared__ volatile int abort_flag;
+    pdl_trigger();
+    const int64_t npieces = list.tiles();
+    const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(gbx_window_smem);
+    const uint32_t sfull = (uint32_t)__cvta_generic_to_shared(full);
+    const uint32_t sempty = (uint32_t)__cvta_generic_to_shared(empty);
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < S; q++) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sfull + 8 * q) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sempty + 8 * q), "r"(NCW) : "memory");
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        abort_flag = 0;
+    }
+    __syncthreads();   // the only CTA-wide barrier
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int limit = list.first()->wait_limit;
+    if (warp == 0) {
+        // ---------------------------------------------------------------- producer (whole warp)
+        int64_t last[S];
+#pragma unroll
+        for (int q = 0; q < S; q++) last[q] = -1;
+        bool stop = false;
+        int64_t lt = 0;
+        const CopyDesc *d = list.first();
+        WinPiece P = {};
+        if (blockIdx.x < npieces) {
+            d = list.at(blockIdx.x, lt);
+            P = d->win[lt];
+        }
+        pdl_wait();
+        for (int64_t k = 0;; k++) {
+            const int64_t t = blockIdx.x + k * gridDim.x;
+            if (t >= npieces) break;
+            const int q = (int)(k % S);
+            bool go = k < S || bulk_wait(sempty + 8 * q, (uint32_t)((k / S - 1) & 1), limit);
+            go = __all_sync(0xffffffffu, go && !abort_flag);
+            if (!go) {
+                abort_flag = 1;
+                stop = true;
+                break;
+            }
+            const uint32_t fb = sfull + 8 * q, stage = sbuf + q * STAGE;
+            const char *src = (P.buf ? d->src2 : d->src) + P.src;
+            const bool good = P.n > 0 && P.n <= GBX_WIN_N && P.nrun > 0 && P.nrun <= GBX_WIN_RUNS && P.bytes > 0 && P.bytes <= WB;
+            const bool bulk = P.buf ? d->win_bulk2 : d->win_bulk;
+            const uint32_t b16 = bulk ? (uint32_t)P.bytes & ~15u : 0u;   // the rest goes through the lanes
+            if (good)
+                for (uint32_t o = b16 + lane * VEC; o < (uint32_t)P.bytes; o += 32 * VEC)
+                    *reinterpret_cast<V *>(gbx_window_smem + q * STAGE + o) = ldv<VEC>(src + o);
+            __syncwarp();
+            if (lane == 0) {
+                dst_s[q] = d->dst + d->dst_flat0;
+                n_s[q] = good ? P.n : 0;
+                if (!good) {   // validated at init; recorded, skipped
+                    gbx_raise(list, 2);
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fb) : "memory");
+                } else {
+                    const int64_t slot = lt * GBX_WIN_N;
+                    const uint32_t ib = ((uint32_t)P.n * 2 + 15) & ~15u, gb = (((uint32_t)P.n + 31) / 32 * 8 + 15) & ~15u,
+                                   rb = ((uint32_t)P.nrun * 4 + 15) & ~15u;
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // consumers' reads before the refill
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
+                                 "r"(b16 + ib + gb + rb)
+                                 : "memory");
+                    if (b16)
+                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                     ::"r"(stage), "l"(src), "r"(b16), "r"(fb) : "memory");
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(stage + OFF_IDX), "l"(d->win_idx + slot), "r"(ib), "r"(fb) : "memory");
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(stage + OFF_GRP), "l"(d->win_grp + slot / 32), "r"(gb), "r"(fb) : "memory");
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(stage + OFF_RUN), "l"(d->win_run + lt * GBX_WIN_RUNS), "r"(rb), "r"(fb) : "memory");
+                    last[q] = k;
+                }
+            }
+            const int64_t tn = t + gridDim.x;
+            if (tn < npieces) {
+                d = list.at(tn, lt);
+                P = d->win[lt];
+            }
+        }
+        if (stop && lane == 0) {   // leave no copy in flight: wait (bounded) for the last one on each stage
+            gbx_raise(list, 1);
+            for (int q = 0; q < S; q++)
+                if (last[q] >= 0) bulk_wait(sfull + 8 * q, (uint32_t)((last[q] / S) & 1));
+        }
+        return;
+    }
+    // -------------------------------------------------------------------- consumers
+    const uint32_t upto = 0xffffffffu >> (31 - lane);   // this lane and the ones before it
+    pdl_wait();
+    for (int64_t k = 0;; k++) {
+        const int64_t t = blockIdx.x + k * gridDim.x;
+        if (t >= npieces) break;
+        const int q = (int)(k % S);
+        if (!bulk_wait(sfull + 8 * q, (uint32_t)((k / S) & 1), limit)) {
+            abort_flag = 1;
+            break;
+        }
+        const unsigned char *stage = gbx_window_smem + q * STAGE;
+        const V *win = reinterpret_cast<const V *>(stage);
+        const uint16_t *idx = reinterpret_cast<const uint16_t *>(stage + OFF_IDX);
+        const uint2 *grp = reinterpret_cast<const uint2 *>(stage + OFF_GRP);
+        const int32_t *run = reinterpret_cast<const int32_t *>(stage + OFF_RUN);
+        const int n = n_s[q], ng = (n + 31) >> 5;
+        char *dst = dst_s[q];
+        for (int g0 = warp - 1; g0 < ng; g0 += NCW * U) {
+            V val[U];
+            int32_t e[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int g = g0 + u * NCW, x = g * 32 + lane;
+                if (x < n) {
+                    const uint2 m = grp[g];
+                    e[u] = run[m.y + __popc(m.x & upto) - 1] + x;
+                    val[u] = win[idx[x]];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if ((g0 + u * NCW) * 32 + lane < n) stv<VEC>(dst + (int64_t)e[u] * VEC, val[u]);
+        }
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sempty + 8 * q) : "memory");
+        if (abort_flag) break;
+    }
+}
+
+// Shapes of the window kernel, chosen by the launch's block value: threads per CTA, stages, CTAs
+// per SM (about 200 KB of shared memory per SM), by the bytes of a window.
+template <int WB> struct WinShape;
+template <> struct WinShape<4096> { static constexpr int S0 = 2, P0 = 8, S1 = 3, P1 = 5, S2 = 6, P2 = 2; };
+template <> struct WinShape<8192> { static constexpr int S0 = 2, P0 = 6, S1 = 3, P1 = 4, S2 = 6, P2 = 2; };
+template <> struct WinShape<16384> { static constexpr int S0 = 2, P0 = 4, S1 = 2, P1 = 4, S2 = 4, P2 = 2; };
+
+template <int VEC, int WE, typename L>
+static cudaError_t window_launch_v(int block, int grid, cudaStream_t st, bool dep, const L &l) {
+    typedef WinShape<VEC * WE> H;
+    constexpr size_t B = VEC * WE + GBX_WIN_TABLES;
+    if (block <= 128) return launch(gbx_window_kernel<VEC, WE, 160, H::S0, H::P0, L>, grid, 160, H::S0 * B, st, dep, l);
+    if (block <= 256) return launch(gbx_window_kernel<VEC, WE, 288, H::S1, H::P1, L>, grid, 288, H::S1 * B, st, dep, l);
+    return launch(gbx_window_kernel<VEC, WE, 544, H::S2, H::P2, L>, grid, 544, H::S2 * B, st, dep, l);
+}
+
+template <int WB> static int win_per_sm(int block) {
+    return block <= 128 ? WinShape<WB>::P0 : block <= 256 ? WinShape<WB>::P1 : WinShape<WB>::P2;
+}
+static int window_per_sm(int vec, int wide, int block) {
+    const int wb = vec * (wide ? 2048 : 1024);
+    return wb == 4096 ? win_per_sm<4096>(block) : wb == 8192 ? win_per_sm<8192>(block) : win_per_sm<16384>(block);
+}
+
+template <typename L>
+static cudaError_t window_launch(int vec, int wide, int block, int grid, cudaStream_t st, bool dep, const L &l) {
+    if (vec == 8) return wide ? window_launch_v<8, 2048>(block, grid, st, dep, l) : window_launch_v<8, 1024>(block, grid, st, dep, l);
+    if (vec == 4) return wide ? window_launch_v<4, 2048>(block, grid, st, dep, l) : window_launch_v<4, 1024>(block, grid, st, dep, l);
+    return cudaErrorInvalidValue;   // offered for elements of 4 and 8 bytes
+}
+
+template <int VEC, int WE, int NT, int S, int PS>
+static cudaError_t window_attr_k() {
+    return smem_attr(gbx_window_kernel<VEC, WE, NT, S, PS, OneOp<CopyDesc>>,
+                     gbx_window_kernel<VEC, WE, NT, S, PS, OpList<CopyDesc>>, S * (VEC * WE + GBX_WIN_TABLES));
+}
+template <int VEC, int WE>
+static cudaError_t window_attr() {
+    typedef WinShape<VEC * WE> H;
+    cudaError_t e = window_attr_k<VEC, WE, 160, H::S0, H::P0>();
+    if (e == cudaSuccess) e = window_attr_k<VEC, WE, 288, H::S1, H::P1>();
+    if (e == cudaSuccess) e = window_attr_k<VEC, WE, 544, H::S2, H::P2>();
+    return e;
+}
+
+int gbx_window_prepare(void) {
+    cudaError_t e = window_attr<8, 1024>();
+    if (e == cudaSuccess) e = window_attr<8, 2048>();
+    if (e == cudaSuccess) e = window_attr<4, 1024>();
+    if (e == cudaSuccess) e = window_attr<4, 2048>();
+    return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
+}
+
 int gbx_bulk_status_take(int *status) {
     int zero = 0;
     GBX_CUDA_TRY(cudaMemcpyFromSymbol(status, gbx_bulk_status, sizeof(int)));
@@ -1483,6 +1692,7 @@ int gbx_occupancy(int kind, int dtype, int vec, int block, int flat) {
     if (kind == 0 && flat == 8) return 1;   // bulk kernel: one CTA per SM (its ring)
     if (kind == 0 && flat == 9) return scatter_shape(block).per_sm;
     if (kind == 0 && flat >= 10 && flat <= 13) return stream_shape(block).per_sm;
+    if (kind == 0 && (flat & 31) == 15) return window_per_sm(vec, flat >> 5, block);
     if (kind == 0 && flat == 14) return agather_per_sm(block);
     if (kind == 0) block = pipe_block(flat, block);
     const void *f = kind == 0 ? (const void *)copy_fn<OneOp<CopyDesc>>(vec, block, flat)
@@ -1508,6 +1718,8 @@ static cudaError_t launch_copy(const L &l, int nops, int vec, int flat, int bloc
         if (block <= 128 && !(flat >= 12 && vec <= 8)) block = 256;   // the narrow shape needs ONE, vec <= 8
         return stream_launch(vec, flat, block, grid, st, dep, l);
     }
+    if ((flat & 31) == 15)   // window form: a "tile" is one piece (code 47: the wide windows)
+        return window_launch(vec, flat >> 5, block, grid, st, dep, l);
     if (flat == 14) return agather_launch(block, grid, st, dep, l);   // async gather (vec 16)
     if ((flat == 5 || flat == 7) && nops > 1) flat -= 4;   // the pipelined kernels take one op
     block = pipe_block(flat, block);

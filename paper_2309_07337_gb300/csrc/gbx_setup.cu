@@ -875,7 +875,7 @@ int gbx_setup_forward(gbx_request_s *req, const int64_t *send_base, const int *s
                                  2 * U * s + npairs * (int64_t)sizeof(Seg)));
         if (combined)
             GBX_TRY(gbx_make_flat_op(req, 2, req->src, ROLE_SRC, req->agg, ROLE_AGG, req->dst, ROLE_DST, gfin, V,
-                                     dst0));
+                                     dst0, true));
         else
             GBX_TRY(gbx_make_copy_op(req, 2, req->agg, ROLE_AGG, req->dst, ROLE_DST, seg3, n3, idx3, Vx, Vx,
                                      2 * Vx * s + 4 * Vx + n3 * (int64_t)sizeof(Seg)));
@@ -1333,6 +1333,190 @@ __global__ void check_scatter_kernel(const ScatterPiece *pieces, int64_t np, con
     }
 }
 
+// ----------------------------------------------------------------- window form
+// A flat gather of small elements can run a source window at a time: its elements are grouped by
+// (source buffer, aligned window of `we` source elements), in destination order inside a
+// window, and cut into pieces of at most GBX_WIN_N.  Consecutive destinations inside a piece
+// form runs: a slot's destination is its run's offset plus its number.
+__device__ __forceinline__ int64_t win_of(uint32_t x, int64_t we, int64_t nw1) {
+    return (int64_t)(x & ~GBX_FLAT_SRC2) / we + ((x & GBX_FLAT_SRC2) ? nw1 : 0);
+}
+
+// runs[0], runs[1]: stretches of consecutive elements in one window of 1024 / 2048 elements (the
+// second source is a window of its own: bit 31 is part of the window number)
+__global__ void win_runs_kernel(const int32_t *g, int64_t n, unsigned long long *runs) {
+    unsigned long long c0 = 0, c1 = 0;
+    FOR_EACH(e, n) {
+        const uint32_t x = (uint32_t)g[e], y = e ? (uint32_t)g[e - 1] : ~x;
+        c0 += (x >> 10) != (y >> 10);
+        c1 += (x >> 11) != (y >> 11);
+    }
+    for (int o = 16; o; o >>= 1) {
+        c0 += __shfl_down_sync(0xffffffffu, c0, o);
+        c1 += __shfl_down_sync(0xffffffffu, c1, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(runs, c0);
+        atomicAdd(runs + 1, c1);
+    }
+}
+
+__global__ void win_key_kernel(const int32_t *g, int64_t n, int64_t we, int64_t nw1, uint64_t *key, int64_t *val) {
+    FOR_EACH(e, n) {
+        key[e] = (uint64_t)win_of((uint32_t)g[e], we, nw1);
+        val[e] = e;
+    }
+}
+
+__global__ void win_count_kernel(const int64_t *start, int64_t nw, int64_t n, int64_t *cnt) {
+    FOR_EACH(w, nw) cnt[w] = ((w + 1 < nw ? start[w + 1] : n) - start[w] + GBX_WIN_N - 1) / GBX_WIN_N;
+}
+
+#define WIN_FILL_T 256
+__global__ void win_fill_kernel(const int32_t *g, const uint64_t *key, const int64_t *elem, const int64_t *start,
+                                const int64_t *first_piece, int64_t nw, int64_t n, int64_t s, int64_t we, int64_t nw1,
+                                int64_t src_elems, int64_t src2_elems, WinPiece *pieces, uint16_t *idx, uint2 *grp,
+                                int32_t *run, int *bad) {
+    __shared__ uint32_t mask_s[GBX_WIN_N / 32], base_s[GBX_WIN_N / 32];
+    const int64_t p = blockIdx.x;
+    const int64_t wi = upper_index(first_piece, nw, p);
+    const int64_t m0 = start[wi] + (p - first_piece[wi]) * GBX_WIN_N;
+    const int64_t end = wi + 1 < nw ? start[wi + 1] : n;
+    const int cnt = (int)(end - m0 < GBX_WIN_N ? end - m0 : GBX_WIN_N);
+    const int64_t w = (int64_t)key[m0];
+    const int buf = w >= nw1;
+    const int64_t first = (buf ? w - nw1 : w) * we, lim = buf ? src2_elems : src_elems;
+    for (int k = threadIdx.x; k < GBX_WIN_N; k += WIN_FILL_T) {
+        const bool starts = k < cnt && (k == 0 || elem[m0 + k] != elem[m0 + k - 1] + 1);
+        const uint32_t m = __ballot_sync(0xffffffffu, starts);
+        if ((k & 31) == 0) mask_s[k >> 5] = m;
+        idx[p * GBX_WIN_N + k] =
+            k < cnt ? (uint16_t)((int64_t)((uint32_t)g[elem[m0 + k]] & ~GBX_FLAT_SRC2) - first) : (uint16_t)0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t b = 0;
+        for (int q = 0; q < GBX_WIN_N / 32; q++) {
+            base_s[q] = b;
+            b += __popc(mask_s[q]);
+        }
+        WinPiece P;
+        P.src = first * s;
+        P.bytes = (int32_t)((lim - first < we ? lim - first : we) * s);
+        P.n = cnt;
+        P.nrun = (int32_t)b;
+        P.buf = buf;
+        P.pad[0] = P.pad[1] = 0;
+        pieces[p] = P;
+        if (b > GBX_WIN_RUNS) *bad = 1;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < GBX_WIN_N; k += WIN_FILL_T) {
+        const uint32_t m = mask_s[k >> 5];
+        const uint32_t r = base_s[k >> 5] + __popc(m & ((1u << (k & 31)) - 1u));
+        if (((m >> (k & 31)) & 1u) && r < GBX_WIN_RUNS) run[p * GBX_WIN_RUNS + r] = (int32_t)(elem[m0 + k] - k);
+        if ((k & 31) == 0) grp[p * (GBX_WIN_N / 32) + (k >> 5)] = make_uint2(m, base_s[k >> 5]);
+    }
+}
+
+// every slot of every piece names the element that the flat gather reads for its destination
+__global__ void check_window_kernel(const WinPiece *pieces, int64_t np, const uint16_t *idx, const uint2 *grp,
+                                    const int32_t *run, const int32_t *g, int64_t n, int64_t s, int64_t we,
+                                    int64_t src_bytes, int64_t src2_bytes, int *err) {
+    FOR_EACH(x, np * GBX_WIN_N) {
+        const int64_t p = x / GBX_WIN_N;
+        const int k = (int)(x % GBX_WIN_N);
+        const WinPiece P = pieces[p];
+        if (k == 0 && (P.src < 0 || (P.src & 15) || P.bytes <= 0 || P.bytes > we * s || P.n <= 0 ||
+                       P.n > GBX_WIN_N || P.nrun <= 0 || P.nrun > GBX_WIN_RUNS ||
+                       P.src + P.bytes > (P.buf ? src2_bytes : src_bytes)))
+            set_err(err, GBX_ERR_INTERNAL);
+        if (k >= P.n) continue;
+        const uint2 q = grp[p * (GBX_WIN_N / 32) + (k >> 5)];
+        const int r = (int)q.y + __popc(q.x & (0xffffffffu >> (31 - (k & 31)))) - 1;
+        bool ok = r >= 0 && r < P.nrun;
+        const int64_t e = ok ? (int64_t)run[p * GBX_WIN_RUNS + r] + k : -1;
+        ok = ok && e >= 0 && e < n && ((int64_t)idx[x] + 1) * s <= P.bytes;
+        if (ok) {
+            const uint32_t v = (uint32_t)g[e];
+            ok = (int)(v >> 31) == P.buf && (int64_t)(v & ~GBX_FLAT_SRC2) * s == P.src + (int64_t)idx[x] * s;
+        }
+        if (!ok) set_err(err, GBX_ERR_INTERNAL);
+    }
+}
+
+// Applies to elements of 4 or 8 bytes, at least GBX_WIN_MIN of them, where runs average at least
+// two elements and no piece has more than GBX_WIN_RUNS (shorter runs cost a partly written sector
+// each, as much as the scattered reads they replace) and reading whole windows costs at most
+// twice the elements' bytes.
+#define GBX_WIN_MIN 65536
+int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t src_elems, int64_t src2_elems,
+                    WinTables *t, int *ok) {
+    cudaStream_t st = req->stream;
+    const int64_t s = req->elem_size;
+    *ok = 0;
+    if (nelem < GBX_WIN_MIN || nelem > 0x7fffffffll - GBX_WIN_N || (s != 4 && s != 8)) return GBX_SUCCESS;
+    DevPool ws;
+    uint64_t *key, *key_alt;
+    int64_t *elem, *elem_alt, *flag, *wid, *start, *cnt, *first;
+    unsigned long long *dn;
+    int *bad;
+    GBX_TRY(ws.get(&dn, 2));
+    GBX_CUDA_TRY(cudaMemsetAsync(dn, 0, 2 * sizeof(*dn), st));
+    win_runs_kernel<<<std::min(grid_of(nelem), 2048u), SETUP_T, 0, st>>>(g, nelem, dn);
+    GBX_CUDA_TRY(cudaGetLastError());
+    unsigned long long runs[2] = {0, 0};
+    GBX_CUDA_TRY(cudaMemcpyAsync(runs, dn, sizeof(runs), cudaMemcpyDeviceToHost, st));
+    GBX_CUDA_TRY(cudaStreamSynchronize(st));
+    // Windows of 2048 elements where the runs of 1024-element ones average under 32 elements: they
+    // merge the messages of neighbouring ranks into longer stores (2^20 rows over 1024 ranks, runs of
+    // 10 elements: 34.6 -> 30.3 us fp64, 27.5 -> 21.0 fp32).  With long runs the second half of
+    // each window is only read (615 k rows over 244 ranks, locality form, runs of 55 and 393:
+    // 22.5 us with 1024, 24.9 with 2048); between the two they tie (runs of 58 and 126: 53.1, 52.0).
+    const int wide = nelem < 32 * (int64_t)runs[0];
+    t->elems = wide ? 2048 : 1024;
+    t->nruns = (int64_t)runs[wide];
+    if (2 * t->nruns > nelem) return GBX_SUCCESS;
+    const int64_t we = t->elems, nw1 = ceil_div(src_elems, we), nw2 = ceil_div(src2_elems, we);
+    GBX_TRY(ws.get(&key, nelem)); GBX_TRY(ws.get(&elem, nelem + 1)); GBX_TRY(ws.get(&key_alt, nelem));
+    GBX_TRY(ws.get(&elem_alt, nelem + 1));
+    uint64_t *const key0 = key;
+    int64_t *const elem0 = elem;
+    win_key_kernel<<<grid_of(nelem), SETUP_T, 0, st>>>(g, nelem, we, nw1, key, elem);
+    GBX_CUDA_TRY(cudaGetLastError());
+    GBX_TRY(gbx_sort_pairs(&key, &elem, key_alt, elem_alt, nelem, std::max(1, bitlen_u64((uint64_t)(nw1 + nw2))), st, ws));
+    flag = (int64_t *)(key == key0 ? key_alt : key0);   // the sort's other buffers, free now
+    wid = elem == elem0 ? elem_alt : elem0;
+    row_flag_kernel<<<grid_of(nelem), SETUP_T, 0, st>>>(key, nelem, flag);
+    GBX_CUDA_TRY(cudaGetLastError());
+    GBX_TRY(gbx_scan_i64(flag, wid, nelem, st, ws));
+    int64_t nw = 0, np = 0;
+    GBX_TRY(gbx_read_i64(wid + nelem, &nw, st));
+    GBX_TRY(ws.get(&start, nw)); GBX_TRY(ws.get(&cnt, nw)); GBX_TRY(ws.get(&first, nw + 1)); GBX_TRY(ws.get(&bad, 1));
+    GBX_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), st));
+    scatter_start_kernel<<<grid_of(nelem), SETUP_T, 0, st>>>(flag, wid, nelem, start);
+    win_count_kernel<<<grid_of(nw), SETUP_T, 0, st>>>(start, nw, nelem, cnt);
+    GBX_CUDA_TRY(cudaGetLastError());
+    GBX_TRY(gbx_scan_i64(cnt, first, nw, st, ws));
+    GBX_TRY(gbx_read_i64(first + nw, &np, st));
+    t->npieces = np;
+    if (np * we > 2 * nelem) return GBX_SUCCESS;
+    GBX_TRY(req->mem.get(&t->pieces, np));
+    GBX_TRY(req->mem.get(&t->idx, np * GBX_WIN_N));
+    GBX_TRY(req->mem.get(&t->grp, np * (GBX_WIN_N / 32)));
+    GBX_TRY(req->mem.get(&t->run, np * GBX_WIN_RUNS));
+    win_fill_kernel<<<(unsigned)np, WIN_FILL_T, 0, st>>>(g, key, elem, start, first, nw, nelem, s, we, nw1, src_elems,
+                                                         src2_elems, t->pieces, t->idx, t->grp, t->run, bad);
+    GBX_CUDA_TRY(cudaGetLastError());
+    int hb = 0;
+    GBX_CUDA_TRY(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
+    GBX_CUDA_TRY(cudaStreamSynchronize(st));
+    if (hb) return GBX_SUCCESS;   // (the tables stay allocated with the request, unused)
+    GBX_TRY(gbx_window_prepare());
+    *ok = 1;
+    return GBX_SUCCESS;
+}
+
 __global__ void check_bulk_kernel(const BulkTask *tasks, int64_t n, int64_t src_bytes, int64_t dst_bytes, int *err) {
     FOR_EACH(m, n) {
         const BulkTask k = tasks[m];
@@ -1368,6 +1552,10 @@ int gbx_validate_program(gbx_request_s *req, int64_t agg_bytes) {
                 check_scatter_kernel<<<grid_of(op.nscat), SETUP_T, 0, st>>>(
                     op.d_scat, op.nscat, d.flat_idx, d.flat_didx, d.nelem, d.elem_size, bytes_of(d.src_role),
                     bytes_of(d.dst_role), err);
+            if (op.win_ok)
+                check_window_kernel<<<grid_of(op.nwin * GBX_WIN_N), SETUP_T, 0, st>>>(
+                    d.win, op.nwin, d.win_idx, d.win_grp, d.win_run, d.flat_idx, d.nelem, d.elem_size, d.win_elems,
+                    bytes_of(d.src_role), d.src2 ? bytes_of(d.src2_role) : 0, err);
             if (op.flat_ok && (d.flat & 3) == 3)
                 check_flat2_kernel<<<grid_of(d.nelem), SETUP_T, 0, st>>>(d.flat_idx, d.flat_didx, d.nelem, d.elem_size,
                                                                          bytes_of(d.src_role),

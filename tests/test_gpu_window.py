@@ -1,0 +1,126 @@
+"""GPU: the window form of the flat gather (source windows and 16-bit indices through shared
+memory, forced with info form=15), at the edges of its pieces (2048 slots) and windows (1024 or 2048
+elements), on buffers whose ends and starts are not 16-byte aligned, through both sources
+(locality form), rebound to unaligned and to host memory, and pooled in batches."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import oracle  # noqa: E402
+import paper_2309_07337_gb300 as gbx  # noqa: E402
+from paper_2309_07337_gb300 import patterns as pt  # noqa: E402
+from gpu_util import assert_bytes_equal, dev_bytes, forward  # noqa: E402
+
+FORM = 1 << 15
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+    gbx.device_status()
+
+
+@pytest.fixture(autouse=True)
+def status_clean():
+    yield
+    assert gbx.device_status() == 0
+
+
+def ring(P, n, region, s, seed, deg=4, dtype="bytes"):
+    """Every rank sends n ascending random elements of its region to each of the next deg ranks."""
+    rng = np.random.default_rng(seed)
+    deg = min(deg, P - 1)
+    src = np.repeat(np.arange(P), deg)
+    dst = (src + np.tile(np.arange(1, deg + 1), P)) % P
+    o = np.lexsort((dst, src))
+    src, dst = src[o], dst[o]
+    el = np.sort(rng.integers(0, region, (P * deg, n)), axis=1)
+    i = np.lexsort((src, dst))
+    g = src[:, None] * region + el
+    return pt._assemble(f"ring_{P}_{n}_{s}", P, 2, src, dst, np.full(P * deg, n), el.ravel(), g.ravel(), dst[i], src[i],
+                        np.full(P * deg, n), g[i].ravel(), s, dtype, np.full(P, region), {})
+
+
+# runs of 12 and 20 elements (windows of 2048 source elements) up to whole pieces (of 1024)
+CASES = [(130, 4, 200, 129), (90, 9, 701, 89), (8, 2048, 1024, 4), (5, 4097, 1025, 4), (16, 1500, 999, 4),
+         (3, 40000, 300, 2), (33, 700, 4099, 4), (40, 512, 2048, 4)]
+
+
+@pytest.mark.parametrize("s", [4, 8])
+@pytest.mark.parametrize("P,n,region,deg", CASES)
+def test_edges(P, n, region, deg, s):
+    p = ring(P, n, region, s, n + s, deg)
+    assert oracle.validate(p) == 0
+    x = pt.random_bytes(p.sendbuf_bytes, n)
+    init = pt.random_bytes(p.recvbuf_bytes, 1)
+    want = oracle.standard(p, x, init)
+    for alg in ("standard", "locality"):
+        for info in ("block=128", "block=256;max_ctas=1", "block=512;max_ctas=3;graph=0", "autotune=1"):
+            got, ex = forward(p, x, alg, info="form=15;" + info, recv_init=init)
+            if alg == "standard":   # (an aggregate read by few ranks may cost too much in whole windows)
+                assert ex.info()["copy_forms"] & FORM, (p.name, alg, info)
+            assert_bytes_equal(got, want, f"{p.name} {alg} {info}")
+
+
+@pytest.mark.parametrize("s", [4, 8])
+def test_rebind_and_batch(s):
+    """Sources one element past a 16-byte boundary and in host memory (lane copies instead of the
+    bulk engine), destinations in host memory, then a batch of two patterns in one launch."""
+    p, q = ring(16, 1500, 999, s, 3), ring(5, 4097, 1025, s, 4)
+    xs = [pt.random_bytes(p.sendbuf_bytes, k) for k in range(3)]
+    y = pt.random_bytes(q.sendbuf_bytes, 9)
+    recv = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+    ex = gbx.Exchange(p, dev_bytes(xs[0]), recv, info="form=15;block=256")
+    off = torch.zeros(p.sendbuf_bytes + s, dtype=torch.uint8, device="cuda")
+    off[s:].copy_(dev_bytes(xs[1]))
+    host = torch.from_numpy(xs[2].copy()).pin_memory()
+    hout = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8).pin_memory()
+    qout = torch.zeros(q.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+    other = gbx.Exchange(q, dev_bytes(y), qout, info="form=15;block=256")
+    assert ex.info()["copy_forms"] & other.info()["copy_forms"] & FORM
+    for send, out, x in ((None, None, xs[0]), (off[s:], recv, xs[1]), (host, recv, xs[2]), (host, hout, xs[2]),
+                         (off[s:], recv, xs[1])):
+        if send is not None:
+            ex.request.bind(send, out)
+        out = recv if out is None else out
+        for batch in (False, True):
+            out.zero_()
+            qout.zero_()
+            if batch:
+                gbx.startall([ex.request, other.request])
+                gbx.waitall([ex.request, other.request])
+                assert_bytes_equal(qout.cpu().numpy(), oracle.standard(q, y), "batch partner")
+            else:
+                ex.start()
+                ex.wait()
+            assert_bytes_equal(out.cpu().numpy(), oracle.standard(p, x), f"batch={batch}")
+
+
+def test_wait_gives_up():
+    p = ring(16, 1500, 999, 8, 7)
+    x = pt.random_bytes(p.sendbuf_bytes, 7)
+    recv = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+    ex = gbx.Exchange(p, dev_bytes(x), recv, info="form=15;autotune=0;wait_limit=0")
+    assert ex.info()["copy_forms"] & FORM
+    ex.start()
+    with pytest.raises(gbx.GbxError) as e:
+        ex.wait()
+    assert e.value.code == gbx.ERR_DEVICE_WAIT
+    assert gbx.device_status() == 1
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_spmv_halo(dtype):
+    p = pt.spmv_halo(60007, 97, 11, 13, 5, dtype)
+    x = pt.spmv_x(p, 3)
+    want = oracle.standard(p, x)
+    for alg in ("standard", "locality"):
+        got, ex = forward(p, x, alg, info="form=15")
+        assert ex.info()["copy_forms"] & FORM
+        assert_bytes_equal(got, want, f"{dtype} {alg}")
