@@ -299,10 +299,8 @@ int gbx_make_copy_op(gbx_request_s *req, int level, const char *src, int src_rol
     d.status = req->status_dev; d.wait_limit = req->wait_limit;
     const int64_t max_tiles = ceil_div(nelem * (req->elem_size / op.min_vec), GBX_TILE);
     GBX_TRY(req->mem.get(&op.d_tile_seg, max_tiles + 1));
-    GBX_TRY(req->mem.get(&op.d_tile_e0, max_tiles + 1));
     GBX_TRY(req->mem.alloc(&op.d_desc, sizeof(CopyDesc)));
     d.tile_seg = op.d_tile_seg;
-    d.tile_e0 = op.d_tile_e0;
     if (req->allow_flat) {
         GBX_TRY(gbx_make_flat(req, segs, nseg, idx, nelem, &op.d_flat_idx, &op.flat_dst0, &op.flat_ok));
         d.flat_idx = op.d_flat_idx;
@@ -353,9 +351,6 @@ int gbx_make_flat_op(gbx_request_s *req, int level, const char *src, int src_rol
     op.ag_ok = agather_ok_for(req, op.max_vec);
     set_bulk_dst(d);
     if (windows) GBX_TRY(add_window(req, op));
-    const int64_t max_tiles = ceil_div(nelem * (req->elem_size / op.min_vec), GBX_TILE);
-    GBX_TRY(req->mem.get(&op.d_tile_e0, max_tiles + 1));
-    d.tile_e0 = op.d_tile_e0;
     GBX_TRY(req->mem.alloc(&op.d_desc, sizeof(CopyDesc)));
     req->ops.push_back(op);
     return GBX_SUCCESS;
@@ -432,9 +427,6 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
     d.nrows = nrows; d.elem_size = s; d.dtype = req->dtype; d.accumulate = accumulate;
     d.out_role = out_role; d.a_role = a_role; d.b_role = b_role;
     d.status = req->status_dev; d.wait_limit = req->wait_limit;
-    const int64_t max_tiles = ceil_div(nrows * (s / op.min_vec), GBX_TILE);
-    GBX_TRY(req->mem.get(&op.d_tile_e0, max_tiles + 1));
-    d.tile_e0 = op.d_tile_e0;
     GBX_TRY(req->mem.get(&op.d_rec, nrows));
     GBX_TRY(gbx_build_fold_records(row_ptr, row_out, terms, nrows, op.d_rec, req->stream));
     d.rec = op.d_rec;
@@ -468,33 +460,37 @@ static int upload_desc(gbx_request_s *req, HostOp &op) {
     return GBX_SUCCESS;
 }
 
-// Sets the op's vector width: chunk geometry, tiles, tile->segment table, descriptor.
-static int set_vec(gbx_request_s *req, HostOp &op, int vec) {
-    const int64_t s = req->elem_size;
-    // the tile tables were allocated for min_vec; a narrower vector would need more tiles
-    if (vec < op.min_vec || vec > op.max_vec) return GBX_ERR_INTERNAL;
-    const int cpe = (int)(s / vec);
+// The chunk geometry of elements of cpe chunks: log2 of it (-1: no power of two) and reciprocals,
+// rounded up.
+template <typename D>
+static void set_geometry(D &d, int vec, int cpe) {
     int shift = -1;
     if ((cpe & (cpe - 1)) == 0) { shift = 0; while ((1 << shift) < cpe) shift++; }
-    const uint32_t magic = shift >= 0 ? 0u : (uint32_t)(((1ull << 32) + (uint64_t)cpe - 1) / (uint64_t)cpe);
+    d.vec = vec;
+    d.cpe = cpe;
+    d.cpe_shift = shift;
+    d.cpe_magic = shift >= 0 ? 0u : (uint32_t)(((1ull << 32) + (uint64_t)cpe - 1) / (uint64_t)cpe);
+    d.cpe_magic64 = shift >= 0 ? 0u : ~0ull / (uint64_t)cpe + 1;
+}
+
+// Sets the op's vector width: chunk geometry, tiles, tile->segment table (segment form), descriptor.
+static int set_vec(gbx_request_s *req, HostOp &op, int vec) {
+    const int64_t s = req->elem_size;
+    // the tile->segment table was allocated for min_vec; a narrower vector would need more tiles
+    if (vec < op.min_vec || vec > op.max_vec) return GBX_ERR_INTERNAL;
+    const int cpe = (int)(s / vec);
     if (op.kind == 0) {
         CopyDesc &d = op.cd;
-        d.vec = vec; d.cpe = cpe; d.cpe_shift = shift; d.cpe_magic = magic;
+        set_geometry(d, vec, cpe);
         d.nchunks = d.nelem * cpe;
         d.ntiles = ceil_div(d.nchunks, GBX_TILE);
-        if (d.flat == 8 || d.flat == 9)   // bulk, scatter: no tile table
-            ;
-        else if (op.flat_only)
-            GBX_TRY(gbx_build_tile_meta(nullptr, 0, cpe, d.ntiles, nullptr, op.d_tile_e0, req->stream));
-        else
-            GBX_TRY(gbx_build_tile_meta(d.segs, d.nseg, cpe, d.ntiles, op.d_tile_seg, op.d_tile_e0, req->stream));
+        if (d.flat == 0) GBX_TRY(gbx_build_tile_meta(d.segs, d.nseg, cpe, d.ntiles, op.d_tile_seg, req->stream));
         d.ntiles = form_tiles(op, d.flat);
     } else {
         FoldDesc &d = op.fd;
-        d.vec = vec; d.cpe = cpe; d.cpe_shift = shift; d.cpe_magic = magic;
+        set_geometry(d, vec, cpe);
         d.nchunks = d.nrows * cpe;
         d.ntiles = ceil_div(d.nchunks, GBX_TILE);
-        GBX_TRY(gbx_build_tile_meta(nullptr, 0, cpe, d.ntiles, nullptr, op.d_tile_e0, req->stream));
     }
     GBX_TRY(upload_desc(req, op));
     GBX_CUDA_TRY(cudaStreamSynchronize(req->stream));
@@ -678,7 +674,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
         else op.fold_form = form;
         const bool pipe = op.kind == 0 && form >= 4 && form < 8, bulk = op.kind == 0 && (form == 8 || form == 9);
         const bool strm = op.kind == 0 ? form >= 10 : form == 1, ag = op.kind == 0 && form >= 14;
-        // (the op's tile tables are sized for min_vec: no width below it)
+        // (the op's tile->segment table is sized for min_vec: no width below it)
         // (the bulk and scatter kernels do not use the vector width: one pass, at max_vec)
         for (int vec = op.max_vec; vec >= (bulk || ag ? op.max_vec : strm ? std::max(4, op.min_vec) : op.min_vec);
              vec >>= 1) {
@@ -1505,7 +1501,7 @@ extern "C" int gbx_waitall(int count, gbx_request_t *reqs) {
 // A batch pools copies by vector width.  An op whose own tuning kept a narrower vector than its
 // alignment allows (common for small ops, whose timings are noise) would add a launch of its own;
 // in a batch it runs at its widest vector instead, through a batch-owned descriptor (same
-// elements, same bytes, its own tile table), so that it joins its dtype's main launch.
+// elements, same bytes), so that it joins its dtype's main launch.
 static int widen_candidate(const HostOp &op) {
     const uintptr_t a = (uintptr_t)op.cd.src | (uintptr_t)op.cd.dst | (uintptr_t)op.cd.src2;
     return op.kind == 0 && op.flat_ok && op.cd.flat != 8 && op.cd.flat != 9 && op.cd.vec < op.max_vec &&
@@ -1514,19 +1510,13 @@ static int widen_candidate(const HostOp &op) {
 
 static int widen_op(DevPool &mem, HostOp &c, int64_t s, cudaStream_t st) {
     const int vec = c.max_vec, cpe = (int)(s / vec);
-    int shift = -1;
-    if ((cpe & (cpe - 1)) == 0) { shift = 0; while ((1 << shift) < cpe) shift++; }
     CopyDesc &d = c.cd;
-    d.vec = vec; d.cpe = cpe; d.cpe_shift = shift;
-    d.cpe_magic = shift >= 0 ? 0u : (uint32_t)(((1ull << 32) + (uint64_t)cpe - 1) / (uint64_t)cpe);
+    set_geometry(d, vec, cpe);
     d.nchunks = d.nelem * cpe;
     d.ntiles = ceil_div(d.nchunks, GBX_TILE);
     // segment and pipelined forms run as the plain flat form the op also has (stream forms stay)
     if (d.flat < 10) d.flat = (d.flat & 3) == 3 ? 3 : 1;
-    GBX_TRY(mem.get(&c.d_tile_e0, d.ntiles + 1));
-    d.tile_e0 = c.d_tile_e0;
     d.tile_seg = nullptr;
-    GBX_TRY(gbx_build_tile_meta(nullptr, 0, cpe, d.ntiles, nullptr, c.d_tile_e0, st));
     GBX_TRY(mem.alloc(&c.d_desc, sizeof(CopyDesc)));
     GBX_CUDA_TRY(cudaMemcpyAsync(c.d_desc, &d, sizeof(CopyDesc), cudaMemcpyHostToDevice, st));
     return GBX_SUCCESS;

@@ -34,10 +34,10 @@ struct CopyDesc {
     const Seg *segs;
     const int32_t *idx;
     const int64_t *tile_seg;  // ntiles + 1: segment holding each tile's first element
-    const int64_t *tile_e0;   // ntiles: first element of each tile
     int64_t nseg, nelem, nchunks, ntiles, elem_size;
     int32_t vec, cpe, cpe_shift;  // chunks per element; log2 of it, or -1
     uint32_t cpe_magic;           // ceil(2^32 / cpe) when cpe is not a power of two
+    uint64_t cpe_magic64;         // likewise 2^64 / cpe
     int32_t src_role, dst_role;
     // flat form (when set): destinations are one contiguous run from dst_flat0 and element
     // e reads source element flat_idx[e]; no segment search
@@ -124,10 +124,10 @@ struct FoldDesc {
     const int64_t *row_out;   // byte offset of each row's output element (setup and validation)
     const longlong2 *rec;     // nrows packed row records (the kernel's view)
     const int64_t *terms;     // byte offset | GBX_TERM_GROUP | GBX_TERM_BUFB
-    const int64_t *tile_e0;   // ntiles: first row of each tile
     int64_t nrows, nchunks, ntiles, elem_size;
     int32_t vec, cpe, cpe_shift;
     uint32_t cpe_magic;
+    uint64_t cpe_magic64;
     int32_t dtype, accumulate;
     int32_t out_role, a_role, b_role;
     int *status;              // the request's status word (see CopyDesc)

@@ -102,10 +102,8 @@ cudaError_t gbx_launch_copy(const OpRef<CopyDesc> &r, int vec, int flat, int blo
 cudaError_t gbx_launch_fold(const OpRef<FoldDesc> &r, int dtype, int vec, int block, int grid, cudaStream_t st, int form,
                             bool dep);
 int gbx_sfold_prepare(void);
-// Per-tile metadata: first unit (element / row) of each tile and, for copy ops, the
-// segment holding it (segs may be NULL for fold ops).
-int gbx_build_tile_meta(const Seg *segs, int64_t nseg, int cpe, int64_t ntiles, int64_t *tile_seg,
-                        int64_t *tile_e0, cudaStream_t st);
+// Segment form: the segment holding each tile's first element.
+int gbx_build_tile_meta(const Seg *segs, int64_t nseg, int cpe, int64_t ntiles, int64_t *tile_seg, cudaStream_t st);
 
 // ------------------------------------------------------------------------ objects
 struct gbx_comm_s {
@@ -140,7 +138,6 @@ struct HostOp {
     void *d_desc;           // device descriptor
     longlong2 *d_rec;       // fold: packed row records
     int64_t *d_tile_seg;    // copy: tile_seg storage sized for min_vec
-    int64_t *d_tile_e0;     // tile_e0 storage sized for min_vec
     int32_t *d_flat_idx;    // copy: source element of every element when the flat form applies
     int64_t flat_dst0;
     int flat_ok;            // the flat form is available
