@@ -137,8 +137,8 @@ def _nbytes(t) -> int:
 
 def _stream_handle(stream) -> Optional[int]:
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:   # the current stream's handle, without building a Stream object (2.7 us)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream
 
 
