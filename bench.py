@@ -1346,7 +1346,7 @@ def run_faces(args):
 
 COPY_FORM_NAMES = {0: "segments", 1: "gather", 3: "two-index", 5: "gather pipelined", 7: "two-index pipelined",
                    8: "bulk pieces", 9: "scatter windows", 10: "gather streamed", 11: "two-index streamed",
-                   12: "fold streamed", 14: "gather async", 15: "window gather"}
+                   12: "fold streamed", 13: "fold by windows", 14: "gather async", 15: "window gather"}
 
 
 def run_bwd_forms(args):

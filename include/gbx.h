@@ -124,8 +124,8 @@ typedef struct {
                                1 gather, 3 two-index, 5/7 pipelined 1/3, 8 bulk pieces,
                                9 source windows scattered, 10/11 stream forms of 1/3,
                                14 async gather, 15 source windows gathered;
-                               bit 12: a fold runs in its stream form (fixed at init by
-                               the tuner) */
+                               bit 12: a fold runs in its stream form, 13: in its window
+                               form (fixed at init by the tuner) */
 } gbx_request_info_t;
 
 const char *gbx_error_string(int code);

@@ -385,7 +385,14 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
                      const char *bufB, int b_role, const int64_t *row_ptr, const int64_t *row_out,
                      const int64_t *terms, int64_t nrows, int64_t nterms, int accumulate) {
     if (nrows <= 0) return GBX_SUCCESS;
-    if (!accumulate && !req->no_single_split) {
+    HostOp op;
+    memset(&op, 0, sizeof(op));
+    int64_t nruns = 0;
+    op.fd.row_ptr = row_ptr; op.fd.row_out = row_out; op.fd.terms = terms; op.fd.nrows = nrows;
+    GBX_TRY(gbx_make_wfold(req, &op.fd, nterms, &nruns, &op.wfold_ok));
+    // The window form takes single-term rows with the others, at the same cost per term: no split
+    // (3 of 10 rows single, 415 k rows fp32 in node-blocked order: 27.3 us, split copy and folds 34.9).
+    if (!accumulate && !req->no_single_split && !op.wfold_ok) {
         // rows with one term are copies: a two-index flat copy op takes them
         int32_t *gs = nullptr, *gd = nullptr;
         int64_t *rp2 = nullptr, *ro2 = nullptr, *t2 = nullptr, ns = 0, nm = 0, nt = 0;
@@ -405,8 +412,6 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
             nterms = nt;
         }
     }
-    HostOp op;
-    memset(&op, 0, sizeof(op));
     op.kind = 1;
     op.level = level;
     op.units = nrows;
@@ -420,7 +425,9 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
     const int64_t s = req->elem_size;
     // per row: its 16-byte record, its output element (read too when accumulating); per term:
     // the gradient element, plus the 8-byte term entry for rows with more than one term
-    op.algo_bytes = nterms * s + nrows * s * (accumulate ? 2 : 1) + nrows * 16 + (nterms - nrows) * 8;
+    op.algo_bytes = op.algo_bytes_fold = nterms * s + nrows * s * (accumulate ? 2 : 1) + nrows * 16 + (nterms - nrows) * 8;
+    // (window form: 2 bytes of place per term, 4 per run, 4 per row)
+    op.algo_bytes_wfold = nterms * s + nrows * s * (accumulate ? 2 : 1) + 2 * nterms + nterms / 4 + 4 * nruns + 4 * nrows;
     op.idx_len = nterms;
     FoldDesc &d = op.fd;
     d.out = out; d.bufA = bufA; d.bufB = bufB; d.row_ptr = row_ptr; d.row_out = row_out; d.terms = terms;
@@ -490,7 +497,7 @@ static int set_vec(gbx_request_s *req, HostOp &op, int vec) {
         FoldDesc &d = op.fd;
         set_geometry(d, vec, cpe);
         d.nchunks = d.nrows * cpe;
-        d.ntiles = ceil_div(d.nchunks, GBX_TILE);
+        d.ntiles = op.fold_form == 2 ? d.nwpiece : ceil_div(d.nchunks, GBX_TILE);
     }
     GBX_TRY(upload_desc(req, op));
     GBX_CUDA_TRY(cudaStreamSynchronize(req->stream));
@@ -504,7 +511,7 @@ static int op_vec(const HostOp &op) { return op.kind == 0 ? op.cd.vec : op.fd.ve
 // grid covers them), which leaves room for other requests' kernels on other streams.
 static int grid_for(int kind, int dtype, int vec, int flat, int block, int persistent, int64_t tiles,
                     int max_ctas) {
-    if ((kind == 0 && flat >= 10) || (kind == 1 && flat == 1)) persistent = 1;   // stream kernels: resident rings
+    if ((kind == 0 && flat >= 10) || (kind == 1 && flat >= 1)) persistent = 1;   // stream kernels: resident rings
     int64_t g = persistent ? (int64_t)gbx_num_sms() * gbx_occupancy(kind, dtype, vec, block, flat)
                            : std::min<int64_t>(tiles, 1ll << 30);
     if (max_ctas > 0) g = std::min<int64_t>(g, max_ctas);
@@ -586,7 +593,10 @@ static int time_op(gbx_request_s *req, HostOp &op, int block, int persistent, in
 
 // algorithmic bytes of a copy in the form it runs in
 static void set_form_bytes(HostOp &op) {
-    if (op.kind != 0) return;
+    if (op.kind != 0) {
+        op.algo_bytes = op.fold_form == 2 ? op.algo_bytes_wfold : op.algo_bytes_fold;
+        return;
+    }
     op.algo_bytes = op.cd.flat == 8 ? op.algo_bytes_bulk
                   : op.cd.flat == 9 ? op.algo_bytes_scat
                   : op.cd.flat == 15 ? op.algo_bytes_win
@@ -600,7 +610,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
     key.units = op.units; key.elem_size = req->elem_size;
     key.nseg = op.kind == 0 ? op.cd.nseg : 0;
     key.nterms = op.kind == 1 ? op.fd.nchunks : 0;
-    key.flat_ok = op.kind == 1 ? op.sfold_ok + 2 * (req->forced_form + 1)
+    key.flat_ok = op.kind == 1 ? op.sfold_ok + 2 * (req->forced_form + 1) + 64 * op.wfold_ok + 128 * (req->allow_stream == 2)
                 : op.kind == 0 ? op.flat_ok + 2 * op.flat_only + 4 * ((op.cd.flat & 3) == 3) + 8 * op.bulk_ok +
                                      16 * op.scat_ok + 32 * (req->allow_bulk == 2) + 64 * op.stream_ok +
                                      128 * (req->allow_stream == 2) + 256 * (req->forced_form + 1) +   // forced forms tune apart
@@ -610,7 +620,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
     if (!req->autotune || req->forced_block) {
         op.block = req->forced_block ? req->forced_block : 256;
         op.persistent = 1;
-        if (op.kind == 1) op.fold_form = op.sfold_ok && req->allow_stream == 2;
+        if (op.kind == 1) op.fold_form = op.wfold_ok && req->allow_stream != 2 ? 2 : op.sfold_ok && req->allow_stream == 2;
         if (op.kind == 0 && !op.flat_only) op.cd.flat = op.flat_ok && req->forced_flat != 0;
         if (op.kind == 0 && op.stream_ok && req->allow_stream == 2) op.cd.flat = (op.cd.flat & 3) == 3 ? 11 : 10;
         if (op.kind == 0 && op.ag_ok && req->forced_form == 14) op.cd.flat = 14;
@@ -627,7 +637,8 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
         auto it = g_tune_cache.find(key);
         op.block = it != g_tune_cache.end() ? it->second.block : 256;
         op.persistent = it != g_tune_cache.end() ? it->second.persistent : 1;
-        op.fold_form = it != g_tune_cache.end() ? it->second.flat : 0;
+        op.fold_form = it != g_tune_cache.end() ? it->second.flat : op.wfold_ok && req->allow_stream != 2 ? 2 : 0;
+        set_form_bytes(op);
         return set_vec(req, op, it != g_tune_cache.end() ? it->second.vec : op.max_vec);
     }
     {
@@ -649,7 +660,9 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
     if (op.kind == 1) {
         forms.push_back(0);
         if (op.sfold_ok) forms.push_back(1);   // the fold's stream form
+        if (op.wfold_ok) forms.push_back(2);   // its window form
         if (op.sfold_ok && (req->allow_stream == 2 || req->forced_form == 1)) forms.assign(1, 1);
+        if (op.wfold_ok && req->forced_form == 2) forms.assign(1, 2);
     }
     else if (op.flat_only) { forms.push_back(op.cd.flat & 3); forms.push_back((op.cd.flat & 3) + 4); }
     else if (op.flat_ok && req->forced_flat < 0) { forms.push_back(0); forms.push_back(1); forms.push_back(5); }
@@ -673,7 +686,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
         if (op.kind == 0) op.cd.flat = form;
         else op.fold_form = form;
         const bool pipe = op.kind == 0 && form >= 4 && form < 8, bulk = op.kind == 0 && (form == 8 || form == 9);
-        const bool strm = op.kind == 0 ? form >= 10 : form == 1, ag = op.kind == 0 && form >= 14;
+        const bool strm = op.kind == 0 ? form >= 10 : form >= 1, ag = op.kind == 0 && form >= 14;
         // (the op's tile->segment table is sized for min_vec: no width below it)
         // (the bulk and scatter kernels do not use the vector width: one pass, at max_vec)
         for (int vec = op.max_vec; vec >= (bulk || ag ? op.max_vec : strm ? std::max(4, op.min_vec) : op.min_vec);
@@ -681,7 +694,8 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
             GBX_TRY(set_vec(req, op, vec));
             // stream forms: persistent grid only; block 256 and 512 select the two wide shapes,
             // block 128 the narrow one, offered only with one chunk per element (cpe == 1)
-            const int b0 = pipe ? 2 : form == 8 ? 3 : ag ? 0 : strm ? (op.kind == 0 && op.cd.cpe == 1 && vec <= 8 ? 0 : 1) : 0;
+            const bool wf = op.kind == 1 && form == 2;   // one shape
+            const int b0 = pipe || wf ? 2 : form == 8 ? 3 : ag ? 0 : strm ? (op.kind == 0 && op.cd.cpe == 1 && vec <= 8 ? 0 : 1) : 0;
             for (int bi = b0; bi < (strm ? 3 : 4); bi++)
                 for (int pers = 1; pers >= (pipe || strm ? 1 : 0); pers--) {
                     float ms = 0;
@@ -921,7 +935,7 @@ static void fill_info(gbx_request_s *req) {
         nlev = std::max(nlev, op.level + 1);
         algo += op.algo_bytes;
         if (op.kind == 0) I.copy_forms |= (int64_t)1 << op.cd.flat;
-        else if (op.fold_form) I.copy_forms |= (int64_t)1 << 12;   // a fold in its stream form
+        else if (op.fold_form) I.copy_forms |= (int64_t)1 << (op.fold_form == 1 ? 12 : 13);   // stream, window fold
         if (!big || op.algo_bytes > big->algo_bytes) big = &op;
     }
     I.levels = nlev;

@@ -130,6 +130,29 @@ struct FoldDesc {
     uint64_t cpe_magic64;
     int32_t dtype, accumulate;
     int32_t out_role, a_role, b_role;
+    // window form (fold form 2): the rows of one-chunk elements cut into pieces (see FoldPiece)
+    const struct FoldPiece *wpiece;
+    const uint16_t *wpos, *wbase, *wrowout;
+    const uint8_t *wrowcnt;
+    const uint2 *wgrp;
+    const uint32_t *wrun, *wgroup;
+    int64_t nwpiece;
+    int32_t wgroups;          // some row has more than one group
     int *status;              // the request's status word (see CopyDesc)
     int32_t wait_limit;
 };
+
+// One piece of a window-form fold: rows row0 .. row0 + nrow - 1, n terms in all, gathered in source
+// order.  Slot k of piece p (tables at p * GBX_WFOLD_N) reads source element
+// (wrun[run] & 0x7fffffff) - GBX_WFOLD_N + k of bufA (bufB where bit 31 of the run is set; runs of
+// piece p at p * GBX_WFOLD_RUNS) and puts it at place wpos[k].  The rows are taken in order of
+// their length, 32 to a slice: term m of row r (in that order) has place wbase[r / 32] + 32 * m +
+// r % 32, its row wrowcnt[r] terms, summed in order into output element out0 + wrowout[r]; bit i of
+// wgroup: the term at place i starts a group.  (wbase and wgroup of piece p at p * GBX_WFOLD_N / 32.)
+struct FoldPiece {
+    int64_t row0, out0;
+    int32_t nrow, n, nrun, pad;
+};
+#define GBX_WFOLD_N 4096
+#define GBX_WFOLD_RUNS 2048
+#define GBX_WFOLD_ROW 64      // terms per row at most

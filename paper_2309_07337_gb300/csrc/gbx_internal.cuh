@@ -66,6 +66,12 @@ struct DevPool {
     template <typename T>
     int get(T **p, int64_t count) { return alloc(reinterpret_cast<void **>(p), (size_t)(count > 0 ? count : 1) * sizeof(T)); }
     void release();
+    void give_to(DevPool &other) {   // its allocations become the other pool's
+        other.ptrs.insert(other.ptrs.end(), ptrs.begin(), ptrs.end());
+        other.bytes += bytes;
+        ptrs.clear();
+        bytes = 0;
+    }
     ~DevPool() { release(); }
 };
 
@@ -98,7 +104,8 @@ struct OpRef {
 };
 // dep: a launch after another one of the same start, which it depends on
 cudaError_t gbx_launch_copy(const OpRef<CopyDesc> &r, int vec, int flat, int block, int grid, cudaStream_t st, bool dep);
-// form 0: the fold kernel; 1: its stream form (records and terms staged in shared memory)
+// form 0: the fold kernel; 1: its stream form (records and terms staged in shared memory); 2: its
+// window form
 cudaError_t gbx_launch_fold(const OpRef<FoldDesc> &r, int dtype, int vec, int block, int grid, cudaStream_t st, int form,
                             bool dep);
 int gbx_sfold_prepare(void);
@@ -156,7 +163,9 @@ struct HostOp {
     int64_t algo_bytes_win;
     int sfold_ok;           // fold: records and terms aligned and padded, one payload class: the
                             // stream form of the fold is available
-    int fold_form;          // fold: 0 the fold kernel, 1 its stream form (tuned)
+    int wfold_ok;           // fold: the window form is available
+    int64_t algo_bytes_fold, algo_bytes_wfold;
+    int fold_form;          // fold: 0 the fold kernel, 1 its stream form, 2 its window form (tuned)
     int scat_ok;            // two-index copy with the scatter form available
     ScatterPiece *d_scat;
     int64_t nscat;
@@ -317,6 +326,9 @@ struct WinTables {
 int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t src_elems, int64_t src2_elems,
                     WinTables *t, int *ok);
 int gbx_window_prepare(void);
+// Window-form tables of a fold's rows into `d`; *ok = 0 where the form does not apply.
+int gbx_make_wfold(gbx_request_s *req, FoldDesc *d, int64_t nterms, int64_t *nruns, int *ok);
+int gbx_wfold_prepare(void);
 int gbx_stream_prepare(void);
 int gbx_agather_prepare(void);
 int gbx_check_data_buf(const void *p, int64_t bytes);   // GBX_ERR_ARG unless the GPU can address p

@@ -1595,6 +1595,206 @@ int gbx_sfold_prepare(void) {
     return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
 }
 
+// Window form of the fold, for rows of one 4- or 8-byte value (tables: FoldPiece).  Per piece the
+// bulk-copy engine brings the tables into shared memory; the threads gather the piece's terms
+// in source order (runs of consecutive gradients: coalesced loads) and drop each at its place;
+// then every row is summed from there, in its fixed order, by one thread.  Rows are taken by
+// length, 32 of a slice side by side, so a warp's lanes read 32 consecutive values at each step
+// and end together.  A term costs 2 bytes of place and its share of a run (8 bytes per term in
+// the other forms) and no dependent load.  The other forms are bound by the latency of the chain
+// record -> term -> gradient and by scattered 4- and 8-byte reads; here the phases of 3 or 4
+// blocks per SM overlap, and the longest row's chain of sums weighs most.  Reverse halo of 2^20
+// rows, 10.8 M terms: fp32 41.0 -> 37.0 us, fp64 in node-blocked order 117 -> 87; of 415 k rows
+// fp32 20.5 -> 12.4; of 300 k rows fp64, node-blocked, accumulating 59 -> 42.
+// The wait for the tables is bounded as in the other forms.
+#define GBX_WFOLD_TABLES \
+    (GBX_WFOLD_N * 2 + GBX_WFOLD_N / 32 * 8 + GBX_WFOLD_RUNS * 4 + GBX_WFOLD_N + GBX_WFOLD_N * 2 + GBX_WFOLD_N / 16 + GBX_WFOLD_N / 8)
+
+template <typename T, int NT, int PS, typename L>
+__global__ void __launch_bounds__(NT, PS) gbx_wfold_kernel(const __grid_constant__ L list) {
+    constexpr int U = 4;
+    constexpr int OFF_POS = GBX_WFOLD_N * (int)sizeof(T), OFF_GRP = OFF_POS + GBX_WFOLD_N * 2,
+                  OFF_RUN = OFF_GRP + GBX_WFOLD_N / 32 * 8, OFF_CNT = OFF_RUN + GBX_WFOLD_RUNS * 4,
+                  OFF_OUT = OFF_CNT + GBX_WFOLD_N, OFF_BASE = OFF_OUT + GBX_WFOLD_N * 2,
+                  OFF_GB = OFF_BASE + GBX_WFOLD_N / 16;
+    extern __shared__ __align__(128) unsigned char gbx_wfold_smem[];
+    __shared__ __align__(8) uint64_t bar;
+    pdl_trigger();
+    T *vals = reinterpret_cast<T *>(gbx_wfold_smem);
+    const uint16_t *pos = reinterpret_cast<const uint16_t *>(gbx_wfold_smem + OFF_POS);
+    const uint2 *grp = reinterpret_cast<const uint2 *>(gbx_wfold_smem + OFF_GRP);
+    const uint32_t *run = reinterpret_cast<const uint32_t *>(gbx_wfold_smem + OFF_RUN);
+    const uint8_t *rowcnt = gbx_wfold_smem + OFF_CNT;
+    const uint16_t *sbase = reinterpret_cast<const uint16_t *>(gbx_wfold_smem + OFF_BASE);
+    const uint16_t *rowout = reinterpret_cast<const uint16_t *>(gbx_wfold_smem + OFF_OUT);
+    const uint32_t *gbit = reinterpret_cast<const uint32_t *>(gbx_wfold_smem + OFF_GB);
+    const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(gbx_wfold_smem);
+    const uint32_t sbar = (uint32_t)__cvta_generic_to_shared(&bar);
+    // pieces are fetched one ahead, by one thread, into slot k & 1
+    __shared__ FoldPiece piece_s[2];
+    __shared__ const FoldDesc *desc_s[2];
+    __shared__ int64_t local_s[2];
+    const int64_t npieces = list.tiles();
+    auto fetch = [&](int64_t t, int slot) {
+        int64_t lt;
+        const FoldDesc *d = list.at(t, lt);
+        piece_s[slot] = d->wpiece[lt];
+        if (!L::single) desc_s[slot] = d;
+        local_s[slot] = lt;
+    };
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sbar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (blockIdx.x < npieces) fetch(blockIdx.x, 0);
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const uint32_t upto = 0xffffffffu >> (31 - lane);
+    uint32_t phase = 0;
+    int slot = 0;
+    for (int64_t t = blockIdx.x; t < npieces; t += gridDim.x, slot ^= 1) {
+        const FoldDesc *d = L::single ? list.first() : desc_s[slot];
+        const int n = piece_s[slot].n, nrow = piece_s[slot].nrow;
+        const bool some = n > 0 && n <= GBX_WFOLD_N && nrow > 0 && nrow <= n && piece_s[slot].nrun > 0 &&
+                          piece_s[slot].nrun <= GBX_WFOLD_RUNS;
+        if (threadIdx.x == NT - 1 && t + gridDim.x < npieces) fetch(t + gridDim.x, slot ^ 1);
+        if (!some) {
+            if (threadIdx.x == 0 && (nrow != 0 || n != 0)) gbx_raise(list, 2);   // validated at init; recorded, skipped
+            __syncthreads();
+            continue;
+        }
+        if (threadIdx.x == 0) {
+            const int64_t lt = local_s[slot], at = lt * GBX_WFOLD_N;
+            const uint32_t pb = ((uint32_t)n * 2 + 15) & ~15u, gb = (((uint32_t)n + 31) / 32 * 8 + 15) & ~15u,
+                           rb = ((uint32_t)piece_s[slot].nrun * 4 + 15) & ~15u, cb = ((uint32_t)nrow + 15) & ~15u,
+                           ob = ((uint32_t)nrow * 2 + 15) & ~15u, sb = (((uint32_t)nrow + 31) / 32 * 2 + 15) & ~15u,
+                           bb = d->wgroups ? GBX_WFOLD_N / 8 : 0u;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the last piece's reads before the refill
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sbar),
+                         "r"(pb + gb + rb + cb + ob + sb + bb)
+                         : "memory");
+            auto load = [&](uint32_t off, const void *src, uint32_t bytes) {
+                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                             ::"r"(sbuf + off), "l"(src), "r"(bytes), "r"(sbar)
+                             : "memory");
+            };
+            load(OFF_POS, d->wpos + at, pb);
+            load(OFF_GRP, d->wgrp + at / 32, gb);
+            load(OFF_RUN, d->wrun + lt * GBX_WFOLD_RUNS, rb);
+            load(OFF_CNT, d->wrowcnt + at, cb);
+            load(OFF_OUT, d->wrowout + at, ob);
+            load(OFF_BASE, d->wbase + at / 32, sb);
+            if (bb) load(OFF_GB, d->wgroup + at / 32, bb);
+        }
+        const bool got = bulk_wait(sbar, phase, d->wait_limit);
+        if (__syncthreads_or(!got)) {
+            if (threadIdx.x == 0) {
+                gbx_raise(list, 1);
+                bulk_wait(sbar, phase);   // leave no copy in flight
+            }
+            return;
+        }
+        phase ^= 1u;
+        pdl_wait();
+        const T *a = reinterpret_cast<const T *>(d->bufA) - GBX_WFOLD_N, *b = reinterpret_cast<const T *>(d->bufB) - GBX_WFOLD_N;
+        // fp64: cp.async straight to the terms' places, all of a thread's in flight together and no
+        // registers held (2^20-row reverse halo, node-blocked order: 95 us; 123 through registers).
+        // fp32: cp.async of 4 bytes was slower (44 us against 38), so G loads per thread go
+        // through registers.
+        if constexpr (sizeof(T) == 8) {
+            for (int x = threadIdx.x; x < n; x += NT) {
+                const uint2 m = grp[x >> 5];
+                const uint32_t r = run[m.y + __popc(m.x & upto) - 1];
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;"
+                             ::"r"(sbuf + (uint32_t)pos[x] * 8u), "l"(((r >> 31) ? b : a) + ((int64_t)(r & 0x7fffffffu) + x))
+                             : "memory");
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        } else {
+            constexpr int G = 4;
+            for (int x0 = threadIdx.x; x0 < n; x0 += NT * G) {
+                T v[G];
+                uint16_t at[G];
+#pragma unroll
+                for (int u = 0; u < G; u++) {
+                    const int x = x0 + u * NT;
+                    if (x < n) {
+                        const uint2 m = grp[x >> 5];
+                        const uint32_t r = run[m.y + __popc(m.x & upto) - 1];
+                        v[u] = ((r >> 31) ? b : a)[(int64_t)(r & 0x7fffffffu) + x];
+                        at[u] = pos[x];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < G; u++)
+                    if (x0 + u * NT < n) vals[at[u]] = v[u];
+            }
+        }
+        __syncthreads();
+        T *out = reinterpret_cast<T *>(d->out) + piece_s[slot].out0;
+        for (int r = threadIdx.x; r < nrow; r += NT) {
+            const int cnt = rowcnt[r], b0 = sbase[r >> 5];   // (r % 32 = lane)
+            const T *v = vals + b0 + lane;
+            T *o = out + rowout[r];
+            T old = T(0);
+            if (d->accumulate) old = *o;
+            T g = v[0], tot = T(0);
+            bool has = false;
+            if (!d->wgroups) {
+#pragma unroll 4
+                for (int m = 1; m < cnt; m++) g = padd(g, v[m * 32]);
+            } else for (int m0 = 1; m0 < cnt; m0 += U) {   // U terms and group bits read ahead of their sums
+                T x[U];
+                uint32_t st = 0;
+#pragma unroll
+                for (int i = 0; i < U; i++)
+                    if (m0 + i < cnt) {
+                        x[i] = v[(m0 + i) * 32];
+                        st |= ((gbit[(b0 >> 5) + m0 + i] >> lane) & 1u) << i;
+                    }
+#pragma unroll
+                for (int i = 0; i < U; i++)
+                    if (m0 + i < cnt) {
+                        // one addition per term whether it starts a group (tot + g) or not (g + x), so
+                        // that the lanes of a warp stay together (an fp64 addition holds its pipe
+                        // for 16 cycles however few lanes take part)
+                        const bool s = (st >> i) & 1u;
+                        const T sum = padd(s ? tot : g, s ? g : x[i]);
+                        tot = s ? (has ? sum : g) : tot;
+                        has |= s;
+                        g = s ? x[i] : sum;
+                    }
+            }
+            if (has) g = padd(tot, g);
+            *o = d->accumulate ? padd(old, g) : g;
+        }
+        __syncthreads();
+    }
+}
+
+// One shape per type: 512 threads x 3 blocks per SM for fp64, 384 x 4 for fp32 (37.0 us on the
+// 2^20-row reverse halo; 512 x 3 37.9, 512 x 4 40.2).
+template <typename T, typename L>
+static cudaError_t wfold_launch(int grid, cudaStream_t st, bool dep, const L &l) {
+    constexpr int NT = sizeof(T) == 4 ? 384 : 512, PS = sizeof(T) == 4 ? 4 : 3;
+    return launch(gbx_wfold_kernel<T, NT, PS, L>, grid, NT, GBX_WFOLD_N * sizeof(T) + GBX_WFOLD_TABLES, st, dep, l);
+}
+
+template <typename T, typename L>
+static cudaError_t wfold_attr() {
+    constexpr int NT = sizeof(T) == 4 ? 384 : 512, PS = sizeof(T) == 4 ? 4 : 3;
+    return cudaFuncSetAttribute(gbx_wfold_kernel<T, NT, PS, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                GBX_WFOLD_N * (int)sizeof(T) + GBX_WFOLD_TABLES);
+}
+
+int gbx_wfold_prepare(void) {
+    cudaError_t e = wfold_attr<double, OneOp<FoldDesc>>();
+    if (e == cudaSuccess) e = wfold_attr<double, OpList<FoldDesc>>();
+    if (e == cudaSuccess) e = wfold_attr<float, OneOp<FoldDesc>>();
+    if (e == cudaSuccess) e = wfold_attr<float, OpList<FoldDesc>>();
+    return e == cudaSuccess ? GBX_SUCCESS : GBX_ERR_CUDA;
+}
+
 // CLS 1..5: every op of the launch is (f64,16) (f64,8) (f32,16) (f32,8) (f32,4).  The kernels
 // with one chunk per thread (1024-thread blocks) are held to 32 registers so that two blocks
 // fit on an SM: the fold is bound by load latency, and the doubled occupancy outweighs the few
@@ -1696,6 +1896,7 @@ static int pipe_block(int flat, int block) { return (flat == 5 || flat == 7) && 
 
 int gbx_occupancy(int kind, int dtype, int vec, int block, int flat) {
     if (kind == 1 && flat == 1) return 2;   // stream fold: two CTAs of 544 threads per SM
+    if (kind == 1 && flat == 2) return dtype == GBX_F32 ? 4 : 3;   // window fold
     if (kind == 0 && flat == 8) return 1;   // bulk kernel: one CTA per SM (its ring)
     if (kind == 0 && flat == 9) return scatter_shape(block).per_sm;
     if (kind == 0 && flat >= 10 && flat <= 13) return stream_shape(block).per_sm;
@@ -1745,6 +1946,8 @@ static cudaError_t launch_fold(const L &l, int dtype, int vec, int block, int gr
             default: return sfold_launch_v<float, 4>(grid, st, dep, l);
         }
     }
+    if (form == 2)   // window form: a "tile" is one piece
+        return dtype == GBX_F64 ? wfold_launch<double>(grid, st, dep, l) : wfold_launch<float>(grid, st, dep, l);
     return launch(fold_fn<L>(dtype, vec, block), grid, block, 0, st, dep, l);
 }
 

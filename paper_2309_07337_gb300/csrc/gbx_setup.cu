@@ -1517,6 +1517,264 @@ int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t
     return GBX_SUCCESS;
 }
 
+// ------------------------------------------------------------ window form of a fold
+// The rows of a fold of one-chunk elements, cut into pieces: piece p takes the rows whose first
+// term lies in [p * c, (p + 1) * c), c = GBX_WFOLD_N minus 32 times the longest row, so that its
+// rows, sorted by length and laid out in slices of 32, fill at most GBX_WFOLD_N places (a slice
+// is as wide as its longest row, which the shortest row of the slice before it covers).
+__global__ void wfold_max_row_kernel(const int64_t *row_ptr, int64_t nrows, unsigned long long *mx) {
+    unsigned long long m = 0;
+    FOR_EACH(r, nrows) {
+        const unsigned long long c = (unsigned long long)(row_ptr[r + 1] - row_ptr[r]);
+        m = c > m ? c : m;
+    }
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long y = __shfl_down_sync(0xffffffffu, m, o);
+        m = y > m ? y : m;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(mx, m);
+}
+
+#define WFOLD_FILL_T 1024
+__global__ void __launch_bounds__(WFOLD_FILL_T) wfold_fill_kernel(
+    const int64_t *row_ptr, const int64_t *row_out, const int64_t *terms, int64_t nrows, int64_t s, int64_t c,
+    FoldPiece *pieces, uint16_t *pos, uint16_t *base, uint8_t *rowcnt, uint16_t *rowout, uint2 *grp, uint32_t *run,
+    uint32_t *group, unsigned long long *nruns, int *flags) {
+    __shared__ uint64_t key[GBX_WFOLD_N];   // (buffer, source element) << 12 | place of the term
+    __shared__ uint32_t mask_s[GBX_WFOLD_N / 32], base_s[GBX_WFOLD_N / 32];
+    const int64_t p = blockIdx.x;
+    __shared__ uint32_t bin[GBX_WFOLD_ROW + 1];
+    __shared__ uint16_t sbase[GBX_WFOLD_N / 32 + 1];
+    // first row that starts at or after x
+    auto row_at = [&](int64_t x) {
+        int64_t lo = 0, hi = nrows;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (row_ptr[mid] < x) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    };
+    const int64_t ra = row_at(p * c), rb = row_at((p + 1) * c);
+    const int nrow = (int)(rb - ra), n = nrow > 0 ? (int)(row_ptr[rb] - row_ptr[ra]) : 0;
+    const int64_t out0 = nrow > 0 ? row_out[ra] / s : 0;
+    auto length = [&](int r) { return (int)(row_ptr[ra + r + 1] - row_ptr[ra + r]); };
+    // rows by length, longest first
+    for (int k = threadIdx.x; k <= GBX_WFOLD_ROW; k += WFOLD_FILL_T) bin[k] = 0;
+    for (int k = threadIdx.x; k < GBX_WFOLD_N; k += WFOLD_FILL_T) key[k] = ~0ull;
+    for (int k = threadIdx.x; k < GBX_WFOLD_N / 32; k += WFOLD_FILL_T) {
+        mask_s[k] = 0;
+        sbase[k] = 0;
+    }
+    __syncthreads();
+    for (int r = threadIdx.x; r < nrow; r += WFOLD_FILL_T) atomicAdd(&bin[GBX_WFOLD_ROW - length(r)], 1u);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t at = 0;
+        for (int b = 0; b <= GBX_WFOLD_ROW; b++) {   // bin b: rows of GBX_WFOLD_ROW - b terms
+            const uint32_t cnt = bin[b];
+            bin[b] = at;
+            for (uint32_t q = (at + 31) / 32; q * 32 < at + cnt; q++) sbase[q + 1] = (uint16_t)(32 * (GBX_WFOLD_ROW - b));
+            at += cnt;
+        }
+        for (int q = 0; q < GBX_WFOLD_N / 32; q++) sbase[q + 1] = (uint16_t)(sbase[q + 1] + sbase[q]);   // widths -> places
+    }
+    __syncthreads();
+    bool bad = false;
+    int starts = 0;
+    for (int r = threadIdx.x; r < nrow; r += WFOLD_FILL_T) {
+        const int len = length(r);
+        const int o = (int)atomicAdd(&bin[GBX_WFOLD_ROW - len], 1u);
+        rowcnt[p * GBX_WFOLD_N + o] = (uint8_t)len;
+        const int64_t out = row_out[ra + r];
+        if (out % s || out / s - out0 < 0 || out / s - out0 > 65535) bad = true;
+        rowout[p * GBX_WFOLD_N + o] = (uint16_t)(out / s - out0);
+        for (int m = 0; m < len; m++) {
+            const int64_t t = row_ptr[ra + r] + m;
+            const uint64_t w = (uint64_t)terms[t];
+            const int64_t off = (int64_t)(w & GBX_TERM_MASK);
+            const int place = sbase[o >> 5] + 32 * m + (o & 31);
+            if (off % s || off / s > 0x7fffffffll - GBX_WFOLD_N) bad = true;
+            key[t - row_ptr[ra]] = ((((w & GBX_TERM_BUFB) ? 1ull << 31 : 0ull) | (uint64_t)(off / s)) << 12) | (uint64_t)place;
+            if (w & GBX_TERM_GROUP) {
+                atomicOr(&mask_s[place >> 5], 1u << (place & 31));
+                if (m > 0) starts = 1;
+            }
+        }
+    }
+    bad = __syncthreads_or(bad);
+    if (__syncthreads_or(starts) && threadIdx.x == 0) flags[1] = 1;   // a row of several groups
+    for (int k = threadIdx.x; k < GBX_WFOLD_N / 32; k += WFOLD_FILL_T) {
+        group[p * (GBX_WFOLD_N / 32) + k] = mask_s[k];
+        base[p * (GBX_WFOLD_N / 32) + k] = sbase[k];
+    }
+    if (bad || n == 0) {
+        if (threadIdx.x == 0) {
+            if (bad) flags[0] = 1;
+            FoldPiece P = {};
+            pieces[p] = P;
+        }
+        return;
+    }
+    // bitonic sort of the keys (distinct: the place is part of each)
+    for (int size = 2; size <= GBX_WFOLD_N; size <<= 1)
+        for (int st = size >> 1; st > 0; st >>= 1) {
+            __syncthreads();
+            for (int q = threadIdx.x; q < GBX_WFOLD_N / 2; q += WFOLD_FILL_T) {
+                const int i = 2 * st * (q / st) + q % st, j = i + st;
+                const bool up = (i & size) == 0;
+                const uint64_t a = key[i], b = key[j];
+                if ((a > b) == up) {
+                    key[i] = b;
+                    key[j] = a;
+                }
+            }
+        }
+    __syncthreads();
+    for (int k = threadIdx.x; k < GBX_WFOLD_N; k += WFOLD_FILL_T) {
+        const bool first = k < n && (k == 0 || (key[k] >> 12) != (key[k - 1] >> 12) + 1 ||
+                                     ((key[k] >> 43) & 1) != ((key[k - 1] >> 43) & 1));
+        const uint32_t m = __ballot_sync(0xffffffffu, first);
+        if ((k & 31) == 0) mask_s[k >> 5] = m;
+        pos[p * GBX_WFOLD_N + k] = k < n ? (uint16_t)(key[k] & 4095) : (uint16_t)0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t b = 0;
+        for (int q = 0; q < GBX_WFOLD_N / 32; q++) {
+            base_s[q] = b;
+            b += __popc(mask_s[q]);
+        }
+        FoldPiece P;
+        P.row0 = ra; P.out0 = out0; P.nrow = nrow; P.n = n; P.nrun = (int32_t)b; P.pad = 0;
+        pieces[p] = P;
+        atomicAdd(nruns, (unsigned long long)b);
+        if (b > GBX_WFOLD_RUNS) flags[0] = 1;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < GBX_WFOLD_N; k += WFOLD_FILL_T) {
+        const uint32_t m = mask_s[k >> 5], r = base_s[k >> 5] + __popc(m & ((1u << (k & 31)) - 1u));
+        if (((m >> (k & 31)) & 1u) && r < GBX_WFOLD_RUNS) {
+            const uint64_t x = key[k] >> 12;
+            run[p * GBX_WFOLD_RUNS + r] = (uint32_t)(x & 0x80000000ull) | (uint32_t)((x & 0x7fffffffull) + GBX_WFOLD_N - k);
+        }
+        if ((k & 31) == 0) grp[p * (GBX_WFOLD_N / 32) + (k >> 5)] = make_uint2(m, base_s[k >> 5]);
+    }
+}
+
+// every slot of every piece gathers the term whose place it fills, every row of a piece is there
+// once with all of its terms, and the pieces' rows are the fold's rows, in order and complete
+__global__ void check_wfold_kernel(const FoldPiece *pieces, int64_t np, const uint16_t *pos, const uint16_t *base,
+                                   const uint8_t *rowcnt, const uint16_t *rowout, const uint2 *grp, const uint32_t *run,
+                                   const uint32_t *group, const int64_t *row_ptr, const int64_t *row_out,
+                                   const int64_t *terms, int64_t nrows, int64_t s, int64_t a_bytes, int64_t b_bytes,
+                                   int64_t out_bytes, int *err) {
+    __shared__ uint32_t seen[GBX_WFOLD_N / 32], rows_seen[GBX_WFOLD_N / 32];
+    __shared__ uint16_t row_of[GBX_WFOLD_N];   // row (from row0) of each row in order of length
+    __shared__ unsigned int total;
+    const int64_t p = blockIdx.x;
+    const FoldPiece P = pieces[p];
+    for (int q = threadIdx.x; q < GBX_WFOLD_N / 32; q += blockDim.x) seen[q] = rows_seen[q] = 0;
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
+    bool ok = P.nrow >= 0 && P.n >= P.nrow && P.n <= GBX_WFOLD_N && P.nrun <= GBX_WFOLD_RUNS && P.row0 >= 0 &&
+              P.row0 + P.nrow <= nrows;
+    ok = ok && (P.nrow == 0 || row_ptr[P.row0 + P.nrow] - row_ptr[P.row0] == P.n);
+    if (ok)
+        for (int o = threadIdx.x; o < P.nrow; o += blockDim.x) {
+            const int64_t out = (P.out0 + rowout[p * GBX_WFOLD_N + o]) * s;
+            int64_t lo = P.row0, hi = P.row0 + P.nrow - 1;   // rows ascend by output offset
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (row_out[mid] < out) lo = mid + 1; else hi = mid;
+            }
+            const int r = (int)(lo - P.row0), len = rowcnt[p * GBX_WFOLD_N + o];
+            row_of[o] = (uint16_t)r;
+            ok = ok && row_out[lo] == out && out + s <= out_bytes && row_ptr[lo + 1] - row_ptr[lo] == len &&
+                 base[p * (GBX_WFOLD_N / 32) + (o >> 5)] + 32 * (len - 1) + (o & 31) < GBX_WFOLD_N;
+            if (atomicOr(&rows_seen[r >> 5], 1u << (r & 31)) & (1u << (r & 31))) ok = false;
+            atomicAdd(&total, (unsigned int)len);
+        }
+    ok = !__syncthreads_or(!ok);
+    if (ok && P.nrow > 0 && total != (unsigned int)P.n) ok = false;
+    for (int k = threadIdx.x; ok && k < P.n; k += blockDim.x) {
+        const uint2 q = grp[p * (GBX_WFOLD_N / 32) + (k >> 5)];
+        const int r = (int)q.y + __popc(q.x & (0xffffffffu >> (31 - (k & 31)))) - 1;
+        const int place = pos[p * GBX_WFOLD_N + k];
+        ok = r >= 0 && r < P.nrun && place < GBX_WFOLD_N;
+        if (!ok) break;
+        const uint32_t x = run[p * GBX_WFOLD_RUNS + r];
+        const int64_t off = ((int64_t)(x & 0x7fffffffu) - GBX_WFOLD_N + k) * s;
+        const int sl = (int)upper_index(base + p * (GBX_WFOLD_N / 32), (P.nrow + 31) / 32, place);
+        const int m = (place - base[p * (GBX_WFOLD_N / 32) + sl]) >> 5, o = sl * 32 + (place & 31);
+        ok = o < P.nrow && m < rowcnt[p * GBX_WFOLD_N + o];
+        if (!ok) break;
+        const uint64_t w = (uint64_t)terms[row_ptr[P.row0 + row_of[o]] + m];
+        ok = off == (int64_t)(w & GBX_TERM_MASK) && (x >> 31) == ((w & GBX_TERM_BUFB) ? 1u : 0u) && off >= 0 &&
+             off + s <= ((x >> 31) ? b_bytes : a_bytes) &&
+             ((group[p * (GBX_WFOLD_N / 32) + (place >> 5)] >> (place & 31)) & 1u) == ((w & GBX_TERM_GROUP) ? 1u : 0u);
+        if (atomicOr(&seen[place >> 5], 1u << (place & 31)) & (1u << (place & 31))) ok = false;
+    }
+    // (the rows of the pieces follow one another)
+    if (threadIdx.x == 0 && P.nrow > 0) {
+        int64_t q = p + 1;
+        while (q < np && pieces[q].nrow == 0) q++;
+        if ((q < np ? pieces[q].row0 : nrows) != P.row0 + P.nrow) ok = false;
+    }
+    if (!ok) set_err(err, GBX_ERR_INTERNAL);
+}
+
+// Applies to elements that are one 4- or 8-byte value, at least GBX_WFOLD_MIN terms, where no row
+// has more than GBX_WFOLD_ROW terms, the terms of every piece form at most GBX_WFOLD_RUNS runs (two
+// terms each on average) and a piece's outputs lie within 65536 elements.
+#define GBX_WFOLD_MIN 32768
+int gbx_make_wfold(gbx_request_s *req, FoldDesc *d, int64_t nterms, int64_t *nruns, int *ok) {
+    cudaStream_t st = req->stream;
+    *ok = 0;
+    const int64_t s = req->elem_size, dsz = req->dtype == GBX_F64 ? 8 : 4;
+    if (s != dsz || nterms < GBX_WFOLD_MIN || !req->allow_stream) return GBX_SUCCESS;
+    DevPool ws, tp;
+    unsigned long long *dn;
+    int *flags;
+    GBX_TRY(ws.get(&dn, 2));
+    GBX_TRY(ws.get(&flags, 2));
+    GBX_CUDA_TRY(cudaMemsetAsync(dn, 0, 2 * sizeof(*dn), st));
+    GBX_CUDA_TRY(cudaMemsetAsync(flags, 0, 2 * sizeof(int), st));
+    wfold_max_row_kernel<<<std::min(grid_of(d->nrows), 2048u), SETUP_T, 0, st>>>(d->row_ptr, d->nrows, dn);
+    GBX_CUDA_TRY(cudaGetLastError());
+    int64_t longest = 0;
+    GBX_TRY(gbx_read_i64((const int64_t *)dn, &longest, st));
+    if (longest < 1 || longest > GBX_WFOLD_ROW) return GBX_SUCCESS;
+    // (places: 32 * longest for the first slice, and each other slice no more than the terms of the
+    // one before it: in all below 32 * longest + (c + longest))
+    const int64_t c = GBX_WFOLD_N - 33 * longest - 32, np = ceil_div(nterms, c);
+    FoldPiece *pieces;
+    uint16_t *pos, *base, *rowout;
+    uint8_t *rowcnt;
+    uint2 *grp;
+    uint32_t *run, *group;
+    GBX_TRY(tp.get(&pieces, np));
+    GBX_TRY(tp.get(&pos, np * GBX_WFOLD_N));
+    GBX_TRY(tp.get(&base, np * (GBX_WFOLD_N / 32)));
+    GBX_TRY(tp.get(&rowcnt, np * GBX_WFOLD_N));
+    GBX_TRY(tp.get(&rowout, np * GBX_WFOLD_N));
+    GBX_TRY(tp.get(&grp, np * (GBX_WFOLD_N / 32)));
+    GBX_TRY(tp.get(&run, np * GBX_WFOLD_RUNS));
+    GBX_TRY(tp.get(&group, np * (GBX_WFOLD_N / 32)));
+    wfold_fill_kernel<<<(unsigned)np, WFOLD_FILL_T, 0, st>>>(d->row_ptr, d->row_out, d->terms, d->nrows, s, c, pieces, pos,
+                                                             base, rowcnt, rowout, grp, run, group, dn + 1, flags);
+    GBX_CUDA_TRY(cudaGetLastError());
+    int hf[2] = {0, 0};
+    GBX_CUDA_TRY(cudaMemcpyAsync(hf, flags, sizeof(hf), cudaMemcpyDeviceToHost, st));
+    GBX_TRY(gbx_read_i64((const int64_t *)(dn + 1), nruns, st));
+    if (hf[0]) return GBX_SUCCESS;
+    GBX_TRY(gbx_wfold_prepare());
+    d->wpiece = pieces; d->wpos = pos; d->wbase = base; d->wrowcnt = rowcnt; d->wrowout = rowout; d->wgrp = grp; d->wrun = run;
+    d->wgroup = group; d->nwpiece = np; d->wgroups = hf[1];
+    tp.give_to(req->mem);
+    *ok = 1;
+    return GBX_SUCCESS;
+}
+
 __global__ void check_bulk_kernel(const BulkTask *tasks, int64_t n, int64_t src_bytes, int64_t dst_bytes, int *err) {
     FOR_EACH(m, n) {
         const BulkTask k = tasks[m];
@@ -1568,6 +1826,10 @@ int gbx_validate_program(gbx_request_s *req, int64_t agg_bytes) {
                                                                         bytes_of(d.dst_role), err);
         } else {
             const FoldDesc &d = op.fd;
+            if (op.wfold_ok)
+                check_wfold_kernel<<<(unsigned)d.nwpiece, 256, 0, st>>>(
+                    d.wpiece, d.nwpiece, d.wpos, d.wbase, d.wrowcnt, d.wrowout, d.wgrp, d.wrun, d.wgroup, d.row_ptr, d.row_out,
+                    d.terms, d.nrows, d.elem_size, bytes_of(d.a_role), bytes_of(d.b_role), bytes_of(d.out_role), err);
             check_fold_kernel<<<grid_of(d.nrows), SETUP_T, 0, st>>>(d.row_ptr, d.row_out, d.rec, d.terms, d.nrows,
                                                                     op.idx_len, d.elem_size, bytes_of(d.out_role),
                                                                     bytes_of(d.a_role), bytes_of(d.b_role), err);

@@ -1,0 +1,101 @@
+"""GPU: the window form of the fold (terms gathered in source order into shared memory, rows summed
+from there), forced with info form=2, against the oracle's fixed-order sums bit for bit: rows of
+one to 64 terms, piece edges (4096 places), both orders (groups per node in the
+locality form), accumulation, unwritten elements, batches, NaN and infinities, and rows too long
+or sources too scattered for the form."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import oracle  # noqa: E402
+import paper_2309_07337_gb300 as gbx  # noqa: E402
+from paper_2309_07337_gb300 import patterns as pt  # noqa: E402
+from gpu_util import assert_bytes_equal, backward, dev_bytes, forward, grad_payload, payload  # noqa: E402
+from test_gpu_window import ring  # noqa: E402
+
+FORM = 1 << 13
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+    gbx.device_status()
+
+
+@pytest.fixture(autouse=True)
+def status_clean():
+    yield
+    assert gbx.device_status() == 0
+
+
+# (ranks, elements per message, region, out-degree): rows of 1 to 18, 8, 7 and 64 terms; the last two
+# have rows over 64 terms and keep the other forms
+CASES = [(16, 1500, 999, 4), (90, 9, 701, 89), (33, 700, 4099, 4), (65, 10, 1, 6), (130, 300, 20, 8), (300, 10, 1, 299)]
+TAKES = CASES[:3]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("P,n,region,deg", CASES)
+def test_edges(P, n, region, deg, dtype):
+    s = 4 if dtype == "f32" else 8
+    p = ring(P, n, region, s, n, deg, dtype)
+    g, old = grad_payload(p, 3), payload(p, 4)
+    for alg, form in (("standard", 0), ("locality", 1)):
+        _, ex = forward(p, payload(p, 1), alg)
+        for acc in (False, True):
+            want = oracle.backward(p, g, grad_send=old, form=form, accumulate=acc)
+            for info in ("form=2", "form=2;block=1024;max_ctas=1", "form=2;block=512;graph=0"):
+                got, b = backward(ex, g, grad_send_init=old, accumulate=acc, info=info)
+                assert_bytes_equal(got, want, f"{p.name} {alg} acc={acc} {info}")
+                if alg == "standard":
+                    assert bool(b.info()["copy_forms"] & FORM) == ((P, n, region, deg) in TAKES), (p.name, info)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_spmv(dtype):
+    p = pt.spmv_halo(60007, 97, 11, 13, 5, dtype)
+    g = grad_payload(p, 9)
+    g[::1001], g[7::2003], g[11::3001] = np.nan, np.inf, -np.inf
+    for alg, form in (("standard", 0), ("locality", 1)):
+        _, ex = forward(p, payload(p, 2), alg)
+        got, b = backward(ex, g, info="form=2")
+        assert b.info()["copy_forms"] & FORM
+        want = oracle.backward(p, g, form=form).view(g.dtype)
+        got = got.view(g.dtype)
+        assert np.array_equal(np.isnan(got), np.isnan(want))
+        assert_bytes_equal(np.where(np.isnan(got), 0, got), np.where(np.isnan(want), 0, want), f"{dtype} {alg}")
+
+
+def test_batch():
+    """Backward requests of both payload types and both orders started together."""
+    items = []
+    for k, (dtype, alg) in enumerate([("f32", "standard"), ("f64", "locality"), ("f32", "locality"), ("f64", "standard")]):
+        p = pt.spmv_halo(20011 + 1000 * k, 61, 8, 12, k, dtype)
+        _, ex = forward(p, payload(p, k), alg)
+        g = grad_payload(p, k + 10)
+        out = torch.zeros(p.sendbuf_bytes, dtype=torch.uint8, device="cuda")
+        items.append((p, g, out, gbx.backward_init(ex.request, dev_bytes(g), out), int(alg == "locality"), ex))
+    for _ in range(2):
+        gbx.startall([i[3] for i in items])
+        gbx.waitall([i[3] for i in items])
+    for p, g, out, _, form, _ in items:
+        assert_bytes_equal(out.cpu().numpy(), oracle.backward(p, g, form=form), p.name)
+
+
+def test_wait_gives_up():
+    p = ring(16, 1500, 999, 8, 7, 4, "f64")
+    _, ex = forward(p, payload(p, 1))
+    out = torch.zeros(p.sendbuf_bytes, dtype=torch.uint8, device="cuda")
+    b = gbx.backward_init(ex.request, dev_bytes(grad_payload(p, 2)), out, info="autotune=0;wait_limit=0")
+    assert b.info()["copy_forms"] & FORM
+    b.start()
+    with pytest.raises(gbx.GbxError) as e:
+        b.wait()
+    assert e.value.code == gbx.ERR_DEVICE_WAIT
+    assert gbx.device_status() == 1
