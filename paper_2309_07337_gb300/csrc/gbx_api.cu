@@ -707,6 +707,10 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
                     // SMs' load / store issue to the copy engine (repeated trials with a warm L2
                     // time the index-driven forms within a few per cent of it)
                     if (op.kind == 0 && form == 8) ms *= 0.97f;
+                    // so does the fold's window form: it reads a quarter of the others' tables, which
+                    // repeated trials find in L2 (415 k rows fp32: 12.4 us, fold kernel 16.5, and
+                    // trials within a few per cent)
+                    if (op.kind == 1 && form == 2) ms *= 0.9f;
                     if (ms < best.ms * (vec < best.vec ? margin : 1.0f)) best = {vec, blocks[bi], pers, form, ms};
                 }
             if (vec == 1) break;

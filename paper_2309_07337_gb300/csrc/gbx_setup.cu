@@ -1746,7 +1746,11 @@ int gbx_make_wfold(gbx_request_s *req, FoldDesc *d, int64_t nterms, int64_t *nru
     if (longest < 1 || longest > GBX_WFOLD_ROW) return GBX_SUCCESS;
     // (places: 32 * longest for the first slice, and each other slice no more than the terms of the
     // one before it: in all below 32 * longest + (c + longest))
-    const int64_t c = GBX_WFOLD_N - 33 * longest - 32, np = ceil_div(nterms, c);
+    // Fewer terms per piece where full ones would leave some of an SM's blocks without (the 200 k
+    // terms of a 3D stencil's reverse, fp64, node-blocked: 21.2 -> 15.0 us).
+    const int64_t c = std::min<int64_t>(GBX_WFOLD_N - 33 * longest - 32,
+                                        std::max<int64_t>(1024, ceil_div(nterms, 3ll * gbx_num_sms()))),
+                  np = ceil_div(nterms, c);
     FoldPiece *pieces;
     uint16_t *pos, *base, *rowout;
     uint8_t *rowcnt;
