@@ -413,7 +413,10 @@ __global__ void __launch_bounds__(32) gbx_bulk_kernel(const __grid_constant__ L 
         dst_of[q] = nullptr;
         len_of[q] = 0;
     }
-    auto load = [&](int q, int64_t t) {
+    // pieces from the last to the first: what the step before wrote last is still in L2 (2^20-row SpMV
+    // halo, locality form, 53.0 -> 52.2 us; 256^3 stencil 105.8 -> 105.0)
+    auto load = [&](int q, int64_t task) {
+        const int64_t t = ntasks - 1 - task;
         int64_t lt;
         const CopyDesc *d = list.at(t, lt);
         const BulkTask k = d->bulk[lt];
