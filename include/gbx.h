@@ -197,7 +197,7 @@ int gbx_graph_free(gbx_graph_t *graph);
  *       algorithm=standard|locality|auto   (default standard; auto times both and keeps
  *                                          the faster)
  *       graph=0|1          1 (default): a start of several launches replays a CUDA graph
- *                          captured at init (until a rebind; then, and for a single launch,
+ *                          captured at init (on other buffers, and for a single launch,
  *                          the kernels are launched with their descriptors as arguments);
  *                          such a start cannot be captured by the caller (GBX_ERR_CUDA).
  *                          0: plain launches that read descriptors in device memory
@@ -466,6 +466,15 @@ int gbx_waitall(int count, gbx_request_t *requests);
  * rewritten, on the request's stream, and a request that belongs to a cached batch (which may
  * run on another request's stream) synchronises that stream. */
 int gbx_request_bind(gbx_request_t request, const void *src, void *dst);
+
+/* One exchange from `src` into `dst`, in stream order: binds the two for this exchange only (as
+ * gbx_request_bind, with its requirements), sets dst to zero bytes first when zero_dst is set,
+ * starts the exchange after the work already on `stream` and completes it for `stream` (as
+ * gbx_start and gbx_wait_stream); the request's own binding is unchanged (a captured exchange,
+ * graph=0 only, leaves src and dst bound).  One call where a program with new buffers at every step
+ * (autograd) would make four.  The caller keeps src and dst alive until the work on `stream`
+ * after the call has run. */
+int gbx_exchange_stream(gbx_request_t request, const void *src, void *dst, int zero_dst, void *stream);
 
 /* One exchange on HOST buffers: copies host_src (the whole bound source buffer, pinned
  * host memory recommended) to the bound device source buffer, starts the exchange, and

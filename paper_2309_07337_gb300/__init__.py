@@ -85,6 +85,7 @@ def lib():
         "gbx_startall": [ctypes.c_int, _pvp],
         "gbx_waitall": [ctypes.c_int, _pvp],
         "gbx_request_bind": [_vp, _vp, _vp],
+        "gbx_exchange_stream": [_vp, _vp, _vp, ctypes.c_int, _vp],
         "gbx_start_host": [_vp, _vp, _vp],
         "gbx_start_host_async": [_vp, _vp, _vp],
         "gbx_request_get_info": [_vp, ctypes.POINTER(RequestInfo)],
@@ -225,6 +226,12 @@ class Request:
             self._bound_src = src
         if dst is not None:
             self._bound_dst = dst
+
+    def exchange_stream(self, src, dst, zero_dst: bool = False, stream=None):
+        """One stream-ordered exchange from src into dst (zeroed first when asked), without
+        changing the request's own binding; the caller keeps both alive on the stream."""
+        _check(lib().gbx_exchange_stream(self.handle, _buf(src), _buf(dst), int(zero_dst), _stream_handle(stream)),
+               "exchange_stream")
 
     def start_host(self, host_src, host_dst):
         """One exchange on host tensors (copied in, exchanged, copied out)."""

@@ -975,7 +975,10 @@ static int finalize(gbx_request_s *req) {
     for (HostOp &op : req->ops) { ptrs.push_back(&op); dts.push_back(req->dtype); }
     const int what = req->kind == 1 ? 2 : req->algorithm == GBX_ALG_LOCALITY ? 1 : 0;
     GBX_TRY(build_levels(req->mem, ptrs, dts, req->launches, 0, req->stream, 0, req->max_ctas, what));
-    // a single launch goes out directly; several are replayed as one graph until a rebind
+    // a single launch goes out directly; several are replayed as one graph while the buffers bound
+    // now are the request's
+    req->exec_src = req->src;
+    req->exec_dst = req->dst;
     if (req->use_graph && req->launches.size() > 1) GBX_TRY(capture(req->launches, &req->ops, &req->exec));
     fill_info(req);
     return GBX_SUCCESS;
@@ -1293,13 +1296,13 @@ extern "C" int gbx_partitioned_init(gbx_request_t forward, int npart, const int6
 }
 
 // The request's kernels on `st`.  graph=1: one launch with its descriptor by value, or the graph
-// captured at init, or after a rebind the launches one by one; none of these may be captured
+// captured at init, or on other buffers the launches one by one; none of these may be captured
 // into a caller's graph, whose replays would keep the buffers bound now.  graph=0: launches that
 // read the descriptors in device memory, which a rebind rewrites, so that they can be.
 static int launch_program(gbx_request_s *req, cudaStream_t st) {
     if (!req->use_graph) {
         GBX_CUDA_TRY(enqueue_levels(req->launches, nullptr, st));
-    } else if (req->exec) {
+    } else if (req->exec && req->src == req->exec_src && req->dst == req->exec_dst) {
         GBX_CUDA_TRY(cudaGraphLaunch(req->exec, st));
     } else if (!req->launches.empty()) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1670,10 +1673,6 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
     } else {
         req->desc_stale = 1;
     }
-    if (req->exec && (ns != req->src || nd != req->dst)) {   // (a running replay keeps it until it ends)
-        cudaGraphExecDestroy(req->exec);
-        req->exec = nullptr;
-    }
     req->src = ns;
     req->dst = nd;
     // cached batches hold their own widened copies of some of these ops: they follow the new
@@ -1700,6 +1699,38 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
     for (Batch *b : stale) destroy_batch(b);
     if (batched) GBX_CUDA_TRY(cudaStreamSynchronize(req->stream));
     return GBX_SUCCESS;
+}
+
+extern "C" int gbx_exchange_stream(gbx_request_t req, const void *src, void *dst, int zero_dst, void *stream) {
+    if (!req) return GBX_ERR_ARG;
+    if (req->kind == 2) return GBX_ERR_UNSUPPORTED;
+    if (req->active) return GBX_ERR_ACTIVE;
+    const char *const own_src = req->src;
+    char *const own_dst = req->dst;
+    if ((cudaStream_t)stream != req->stream || (cudaStream_t)stream == cudaStreamPerThread) {
+        cudaEvent_t ev;
+        GBX_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        cudaError_t e = cudaEventRecord(ev, (cudaStream_t)stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(req->stream, ev, 0);
+        cudaEventDestroy(ev);
+        GBX_CUDA_TRY(e);
+    }
+    GBX_TRY(gbx_request_bind(req, src, dst));
+    auto run = [&]() -> int {
+        if (zero_dst && req->dst_bytes > 0) {
+            if (req->host_down_pending) GBX_CUDA_TRY(cudaStreamWaitEvent(req->stream, req->host_down_ev, 0));
+            GBX_CUDA_TRY(cudaMemsetAsync(req->dst, 0, (size_t)req->dst_bytes, req->stream));
+        }
+        GBX_TRY(enqueue_start(req));
+        return gbx_wait_stream(req, stream);
+    };
+    const int rc = run();
+    // (a replay of a capture reads the descriptors as they are then: they keep these buffers)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    GBX_CUDA_TRY(cudaStreamIsCapturing(req->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return rc;
+    const int rb = gbx_request_bind(req, own_src, own_dst);
+    return rc != GBX_SUCCESS ? rc : rb;
 }
 
 static int host_streams(gbx_request_s *req) {

@@ -240,6 +240,8 @@ struct gbx_request_s {
     std::vector<HostOp> ops;
     std::vector<LevelLaunch> launches;
     cudaGraphExec_t exec;    // several launches: the start sequence over the buffers bound at init
+    const char *exec_src;    // (these)
+    char *exec_dst;
     int desc_stale;          // the device descriptors lack the last rebind (no launch reads them)
     gbx_request_info_t info;
     // maps kept for building the backward of this (forward) request

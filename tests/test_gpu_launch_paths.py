@@ -68,6 +68,33 @@ def test_rebinds_between_starts(alg, info, how):
         assert_bytes_equal(outs[k].cpu().numpy(), want[k], f"{alg} {info} {how} batch, buffers {k}")
 
 
+@pytest.mark.parametrize("alg", ["standard", "locality"])
+@pytest.mark.parametrize("info", ["", "graph=0"])
+@pytest.mark.parametrize("other_stream", [False, True])
+def test_exchange_stream(alg, info, other_stream):
+    """One call on buffers of its own: the same bytes, the gaps zero or as they were, the request's own
+    binding (and its graph) unchanged, errors as from the calls it stands for."""
+    p = pt.random_pattern(91, P=24, dtype="f64", max_count=60)
+    xs = [payload(p, k) for k in range(3)]
+    own, out = (torch.full((p.recvbuf_bytes,), 0xA5, dtype=torch.uint8, device="cuda") for _ in range(2))
+    ex = gbx.Exchange(p, dev_bytes(xs[0]), own, alg, info=info)
+    side = torch.cuda.Stream()
+    init = np.full(p.recvbuf_bytes, 0xA5, np.uint8)
+    for k, zero in ((1, False), (2, True), (1, True)):
+        send = dev_bytes(xs[k])
+        out.fill_(0xA5)
+        ex.request.exchange_stream(send, out, zero_dst=zero, stream=side if other_stream else None)
+        with torch.cuda.stream(side if other_stream else torch.cuda.current_stream()):
+            got = out.cpu().numpy()
+        assert_bytes_equal(got, oracle.standard(p, xs[k], None if zero else init), f"{alg} {info} {k} {zero}")
+    ex.start()
+    with pytest.raises(gbx.GbxError) as e:
+        ex.request.exchange_stream(send, out)
+    assert e.value.code == gbx.ERR_ACTIVE
+    ex.wait()
+    assert_bytes_equal(own.cpu().numpy(), oracle.standard(p, xs[0], init), "own binding")
+
+
 def test_start_under_capture_is_refused():
     """A graph=1 start launches with the buffers bound now, which a caller's graph would keep: it
     returns ERR_CUDA inside a stream capture and works again after it."""
