@@ -476,7 +476,7 @@ static void set_geometry(D &d, int vec, int cpe) {
     d.vec = vec;
     d.cpe = cpe;
     d.cpe_shift = shift;
-    d.cpe_magic = shift >= 0 ? 0u : (uint32_t)(((1ull << 32) + (uint64_t)cpe - 1) / (uint64_t)cpe);
+    d.cpe_magic = cpe > GBX_TILE ? 0u : (uint32_t)(((1 << GBX_MAGIC_SHIFT) + cpe - 1) / cpe);
     d.cpe_magic64 = shift >= 0 ? 0u : ~0ull / (uint64_t)cpe + 1;
 }
 

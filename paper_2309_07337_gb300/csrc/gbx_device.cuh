@@ -8,6 +8,7 @@
 #include <cstdint>
 
 #define GBX_TILE 1024                    // chunks per tile (block * unroll)
+#define GBX_MAGIC_SHIFT 21               // (2 * GBX_TILE) * GBX_TILE: see unit_of
 #define GBX_TERM_GROUP (1ull << 63)      // fold term: first term of a group
 #define GBX_TERM_BUFB (1ull << 62)       // fold term: reads buffer B (else A)
 #define GBX_TERM_MASK ((1ull << 62) - 1)
@@ -36,8 +37,8 @@ struct CopyDesc {
     const int64_t *tile_seg;  // ntiles + 1: segment holding each tile's first element
     int64_t nseg, nelem, nchunks, ntiles, elem_size;
     int32_t vec, cpe, cpe_shift;  // chunks per element; log2 of it, or -1
-    uint32_t cpe_magic;           // ceil(2^32 / cpe) when cpe is not a power of two
-    uint64_t cpe_magic64;         // likewise 2^64 / cpe
+    uint32_t cpe_magic;           // ceil(2^GBX_MAGIC_SHIFT / cpe), for cpe <= GBX_TILE
+    uint64_t cpe_magic64;         // ceil(2^64 / cpe) when cpe is not a power of two
     int32_t src_role, dst_role;
     // flat form (when set): destinations are one contiguous run from dst_flat0 and element
     // e reads source element flat_idx[e]; no segment search

@@ -117,12 +117,14 @@ static cudaError_t launch(void (*f)(const L), int grid, int block, size_t smem, 
     return cudaLaunchKernelEx(&c, f, l);
 }
 
-// Unit (element or row) and chunk-in-unit of local chunk x of a tile whose first chunk
-// is chunk r0 of unit e0.  x < GBX_TILE + cpe, so the 32-bit magic multiply is exact.
-__device__ __forceinline__ uint32_t unit_of(uint32_t x, int cpe, int sh, uint32_t magic) {
-    if (sh >= 0) return x >> sh;
-    if (cpe < 32768) return __umulhi(x, magic);
-    return x / (uint32_t)cpe;
+// Unit (element or row) that holds local chunk x of a tile whose first chunk is a chunk of unit 0:
+// x < GBX_TILE + cpe - 1.  Units of at most a tile: magic = ceil(2^21 / cpe), exact for x < 2048;
+// of a longer one a tile holds parts of two at most.  No branch: three ways by kind of cpe (shift,
+// multiply, divide) cost the 512^3 stencil halo 557 us where this takes 548, 606 and 580 with the
+// descriptor in device memory, where the compiler cannot know the branches to be uniform (2.6 M
+// 24-byte records: 34.3 and 33.0).
+__device__ __forceinline__ uint32_t unit_of(uint32_t x, int cpe, uint32_t magic) {
+    return cpe > GBX_TILE ? (uint32_t)(x >= (uint32_t)cpe) : (x * magic) >> GBX_MAGIC_SHIFT;
 }
 
 // First unit of the tile (or part of one) whose first chunk is c0: computed, so that no load of a
@@ -141,7 +143,7 @@ template <int VEC, int U>
 __device__ __forceinline__ void copy_tile_flat(const CopyDesc *__restrict__ d, int64_t t) {
     typedef typename VecT<VEC>::T V;
     constexpr int B = GBX_TILE / U;
-    const int cpe = d->cpe, sh = d->cpe_shift;
+    const int cpe = d->cpe;
     const uint32_t magic = d->cpe_magic;
     const int64_t e0 = first_unit(d, t * GBX_TILE);
     const uint32_t r0 = (uint32_t)(t * GBX_TILE - e0 * cpe);
@@ -152,7 +154,7 @@ __device__ __forceinline__ void copy_tile_flat(const CopyDesc *__restrict__ d, i
 #pragma unroll
     for (int u = 0; u < U; u++) {
         const uint32_t x = r0 + (uint32_t)(u * B) + threadIdx.x;
-        const uint32_t el = unit_of(x, cpe, sh, magic);
+        const uint32_t el = unit_of(x, cpe, magic);
         const int64_t j = (int64_t)(x - el * (uint32_t)cpe) * VEC;
         const int64_t e = e0 + el;
         const bool ok = (int64_t)(u * B + threadIdx.x) < left;
@@ -179,7 +181,7 @@ template <int VEC, int U>
 __device__ __forceinline__ void copy_tile_flat2(const CopyDesc *__restrict__ d, int64_t t) {
     typedef typename VecT<VEC>::T V;
     constexpr int B = GBX_TILE / U;
-    const int cpe = d->cpe, sh = d->cpe_shift;
+    const int cpe = d->cpe;
     const uint32_t magic = d->cpe_magic;
     const int64_t e0 = first_unit(d, t * GBX_TILE);
     const uint32_t r0 = (uint32_t)(t * GBX_TILE - e0 * cpe);
@@ -189,7 +191,7 @@ __device__ __forceinline__ void copy_tile_flat2(const CopyDesc *__restrict__ d, 
 #pragma unroll
     for (int u = 0; u < U; u++) {
         const uint32_t x = r0 + (uint32_t)(u * B) + threadIdx.x;
-        const uint32_t el = unit_of(x, cpe, sh, magic);
+        const uint32_t el = unit_of(x, cpe, magic);
         const int64_t j = (int64_t)(x - el * (uint32_t)cpe) * VEC;
         const int64_t e = e0 + el;
         const bool ok = (int64_t)(u * B + threadIdx.x) < left;
@@ -217,7 +219,7 @@ template <int VEC, int U, int FORM>
 __device__ __forceinline__ void flat_indices(const CopyDesc *__restrict__ d, int64_t t, uint32_t (&gi)[U],
                                              int32_t (&gd)[U], int64_t (&e)[U], int64_t (&j)[U], bool (&ok)[U]) {
     constexpr int B = GBX_TILE / U;
-    const int cpe = d->cpe, sh = d->cpe_shift;
+    const int cpe = d->cpe;
     const uint32_t magic = d->cpe_magic;
     const int64_t e0 = first_unit(d, t * GBX_TILE);
     const uint32_t r0 = (uint32_t)(t * GBX_TILE - e0 * cpe);
@@ -225,7 +227,7 @@ __device__ __forceinline__ void flat_indices(const CopyDesc *__restrict__ d, int
 #pragma unroll
     for (int u = 0; u < U; u++) {
         const uint32_t x = r0 + (uint32_t)(u * B) + threadIdx.x;
-        const uint32_t el = unit_of(x, cpe, sh, magic);
+        const uint32_t el = unit_of(x, cpe, magic);
         j[u] = (int64_t)(x - el * (uint32_t)cpe) * VEC;
         e[u] = e0 + el;
         ok[u] = (int64_t)(u * B + threadIdx.x) < left;
@@ -275,7 +277,7 @@ __device__ __forceinline__ void copy_tile(const CopyDesc *__restrict__ d, int64_
     typedef typename VecT<VEC>::T V;
     constexpr int B = GBX_TILE / U;
     const Seg *__restrict__ segs = d->segs;
-    const int cpe = d->cpe, sh = d->cpe_shift;
+    const int cpe = d->cpe;
     const uint32_t magic = d->cpe_magic;
     const int64_t e0 = first_unit(d, t * GBX_TILE);
     const uint32_t r0 = (uint32_t)(t * GBX_TILE - e0 * cpe);
@@ -288,7 +290,7 @@ __device__ __forceinline__ void copy_tile(const CopyDesc *__restrict__ d, int64_
 #pragma unroll
     for (int u = 0; u < U; u++) {
         const uint32_t x = r0 + (uint32_t)(u * B) + threadIdx.x;
-        const uint32_t el = unit_of(x, cpe, sh, magic);
+        const uint32_t el = unit_of(x, cpe, magic);
         j[u] = x - el * (uint32_t)cpe;
         e[u] = e0 + el;
         pos[u] = slo;
@@ -832,7 +834,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const __grid_constan
             }
         } else if (!ONE && e_al >= 0) {
             const CopyDesc *d = L::single ? list.first() : desc_s[q];
-            const int cpe = d->cpe, sh = d->cpe_shift;
+            const int cpe = d->cpe;
             const uint32_t magic = d->cpe_magic;
             const int64_t s = d->elem_size, e0 = efirst_s[q], c0 = tile_s[q] * GBX_TILE;
             const int left = (int)min((int64_t)GBX_TILE, d->nchunks - c0);
@@ -849,7 +851,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_stream_kernel(const __grid_constan
                     const int x = base + u * NC + ct;
                     if (x < left) {
                         const uint32_t xx = r0 + (uint32_t)x;
-                        const uint32_t el = unit_of(xx, cpe, sh, magic);
+                        const uint32_t el = unit_of(xx, cpe, magic);
                         const int64_t j = (int64_t)(xx - el * (uint32_t)cpe) * VEC;
                         const int64_t e = e0 + el;
                         const int w = (int)(e - e_al);   // < GBX_TILE + 8: inside the stage's copy
@@ -1000,7 +1002,7 @@ __global__ void __launch_bounds__(NW * 32, PS) gbx_agather_kernel(const __grid_c
 #pragma unroll
         for (int k = 0; k < K; k++) {
             const int x0 = k * 32 + lane;
-            gi[k] = x0 < left ? (uint32_t)__ldg(g + unit_of(r0 + (uint32_t)x0, d->cpe, d->cpe_shift, d->cpe_magic)) : 0u;
+            gi[k] = x0 < left ? (uint32_t)__ldg(g + unit_of(r0 + (uint32_t)x0, d->cpe, d->cpe_magic)) : 0u;
         }
     };
     if (u < nunits) indices(u);
@@ -1021,7 +1023,7 @@ __global__ void __launch_bounds__(NW * 32, PS) gbx_agather_kernel(const __grid_c
                 const int x0 = k * 32 + lane;
                 if (x0 < left) {
                     const uint32_t xx = r0 + (uint32_t)x0;
-                    const uint32_t j = xx - unit_of(xx, d->cpe, d->cpe_shift, d->cpe_magic) * (uint32_t)d->cpe;
+                    const uint32_t j = xx - unit_of(xx, d->cpe, d->cpe_magic) * (uint32_t)d->cpe;
                     const char *b = (gi[k] & GBX_FLAT_SRC2) ? d->src2 : d->src;
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
                                  ::"r"(sring + (uint32_t)((q * UNIT + x0) * 16)),
@@ -1324,7 +1326,7 @@ template <typename T, int VEC, int U>
 __device__ __forceinline__ void fold_tile(const FoldDesc *__restrict__ d, int64_t t) {
     typedef typename PackT<T, VEC>::T PK;
     constexpr int B = GBX_TILE / U;
-    const int cpe = d->cpe, sh = d->cpe_shift;
+    const int cpe = d->cpe;
     const uint32_t magic = d->cpe_magic;
     const int64_t e0 = first_unit(d, t * GBX_TILE);
     const uint32_t r0 = (uint32_t)(t * GBX_TILE - e0 * cpe);
@@ -1336,7 +1338,7 @@ __device__ __forceinline__ void fold_tile(const FoldDesc *__restrict__ d, int64_
 #pragma unroll
     for (int u = 0; u < U; u++) {
         const uint32_t x = r0 + (uint32_t)(u * B) + threadIdx.x;
-        const uint32_t el = unit_of(x, cpe, sh, magic);
+        const uint32_t el = unit_of(x, cpe, magic);
         jv[u] = (x - el * (uint32_t)cpe) * VEC;
         const bool ok = (int64_t)(u * B + threadIdx.x) < left;
         if (ok) {
@@ -1508,7 +1510,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const __grid_constant
         const int64_t r_first = rfirst_s[q];
         if (r_first >= 0) {
             const FoldDesc *d = L::single ? list.first() : desc_s[q];
-            const int cpe = d->cpe, sh = d->cpe_shift;
+            const int cpe = d->cpe;
             const uint32_t magic = d->cpe_magic;
             const int64_t c0 = tile_s[q] * GBX_TILE, tb_al = tbase_s[q];
             const int left = (int)min((int64_t)GBX_TILE, d->nchunks - c0);
@@ -1518,7 +1520,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_sfold_kernel(const __grid_constant
             const char *bufA = d->bufA, *bufB = d->bufB;
             for (int x = ct; x < left; x += NC) {
                 const uint32_t xx = r0 + (uint32_t)x;
-                const uint32_t el = unit_of(xx, cpe, sh, magic);
+                const uint32_t el = unit_of(xx, cpe, magic);
                 const int64_t jv = (int64_t)(xx - el * (uint32_t)cpe) * VEC;
                 const longlong2 rec = rs[el];
                 const uint64_t oa = (uint64_t)rec.x, ob = (uint64_t)rec.y;

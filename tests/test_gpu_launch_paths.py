@@ -68,6 +68,20 @@ def test_rebinds_between_starts(alg, info, how):
         assert_bytes_equal(outs[k].cpu().numpy(), want[k], f"{alg} {info} {how} batch, buffers {k}")
 
 
+@pytest.mark.parametrize("comps", [1, 5, 2046, 2048, 2050, 6144])
+@pytest.mark.parametrize("info", ["form=1", "form=5", "form=10", "form=14", "flat=0", "graph=0", "vec=8;form=5"])
+def test_chunks_per_element(comps, info):
+    """Elements of less, exactly and more than a tile (1024 chunks of 16 bytes; of 8 with vec=8)."""
+    p = pt.stencil((8, 6, 4), (2, 2, 2), ppn=3, comps=comps)
+    x = payload(p, 9)
+    recv = torch.full((p.recvbuf_bytes,), 0xA5, dtype=torch.uint8, device="cuda")
+    ex = gbx.Exchange(p, dev_bytes(x), recv, "standard", info=info)
+    ex.start()
+    ex.wait()
+    want = oracle.standard(p, x, np.full(p.recvbuf_bytes, 0xA5, np.uint8))
+    assert_bytes_equal(recv.cpu().numpy(), want, f"{comps} {info}")
+
+
 @pytest.mark.parametrize("alg", ["standard", "locality"])
 @pytest.mark.parametrize("info", ["", "graph=0"])
 @pytest.mark.parametrize("other_stream", [False, True])
