@@ -24,6 +24,13 @@ struct Batch {
     cudaStream_t on = nullptr;
     int done_timed = 0, other_streams = 0;   // see done_event_for_other_streams
     int finished = 0;             // the last start's end has been seen: its members need not ask again
+    // the members' buffers at capture: on other buffers the launches go out one by one
+    std::vector<std::pair<const char *, char *>> bound;
+    bool as_captured() const {
+        for (size_t k = 0; k < members.size(); k++)
+            if (members[k]->src != bound[k].first || members[k]->dst != bound[k].second) return false;
+        return true;
+    }
 };
 
 extern "C" const char *gbx_error_string(int code) {
@@ -533,16 +540,17 @@ static cudaError_t launch_op_alone(gbx_request_s *req, HostOp &op, int block, in
     const int vec = op_vec(op), flat = op.kind == 0 && op_flat(op) == 15 ? window_code(op.cd) : op_flat(op);
     const int grid = grid_for(op.kind, req->dtype, vec, flat, block, persistent, tiles, req->max_ctas);
     if (op.kind == 0)
-        return gbx_launch_copy({&op.cd, nullptr, nullptr, 1, tiles}, vec, launch_code(flat, op.cd.cpe == 1), block, grid,
-                               req->stream, false);
-    return gbx_launch_fold({&op.fd, nullptr, nullptr, 1, tiles}, req->dtype, vec, block, grid, req->stream, flat, false);
+        return gbx_launch_copy({op.d_self ? nullptr : &op.cd, (const CopyDesc *const *)op.d_self, nullptr, 1, tiles}, vec,
+                               launch_code(flat, op.cd.cpe == 1), block, grid, req->stream, false);
+    return gbx_launch_fold({op.d_self ? nullptr : &op.fd, (const FoldDesc *const *)op.d_self, nullptr, 1, tiles},
+                           req->dtype, vec, block, grid, req->stream, flat, false);
 }
 
 // A level's launch in form `flat`, `block` and `grid`; ops: the request's ops, for launches of one
 // op passed by value (null: every launch reads its device descriptor list).
-static cudaError_t launch_level(const LevelLaunch &L, const std::vector<HostOp> *ops, int flat, int block, int grid,
+static cudaError_t launch_level(const LevelLaunch &L, bool by_value, int flat, int block, int grid,
                                 cudaStream_t st, bool dep) {
-    const HostOp *op = ops && L.one_op >= 0 ? &(*ops)[L.one_op] : nullptr;
+    const HostOp *op = by_value ? L.only : nullptr;
     if (L.kind == 0)
         return gbx_launch_copy({op ? &op->cd : nullptr, (const CopyDesc *const *)L.d_ops, L.d_prefix, L.nops, L.total_tiles},
                                L.vec, launch_code(flat, L.one), block, grid, st, dep);
@@ -556,7 +564,7 @@ static cudaError_t launch_level(const LevelLaunch &L, const std::vector<HostOp> 
 // the shape: every candidate moves the same bytes to the same places.  Chosen shapes are
 // cached by a signature of the op, so identical patterns are tuned once per process.
 struct TuneKey {
-    int kind, max_vec, min_vec, dtype, flat_ok;
+    int kind, max_vec, min_vec, dtype, flat_ok, list;
     int64_t units, nseg, elem_size, nterms;
     bool operator<(const TuneKey &o) const {
         return memcmp(this, &o, sizeof(TuneKey)) < 0;
@@ -616,6 +624,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
                                      128 * (req->allow_stream == 2) + 256 * (req->forced_form + 1) +   // forced forms tune apart
                                      8192 * op.ag_ok + 16384 * op.win_ok
                 : 0;
+    key.list = op.list = !req->use_graph;
     int blocks[4] = {128, 256, 512, 1024};
     if (!req->autotune || req->forced_block) {
         op.block = req->forced_block ? req->forced_block : 256;
@@ -653,6 +662,14 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
             set_form_bytes(op);
             return set_vec(req, op, it->second.vec);
         }
+    }
+    // timed as it will be launched: graph=0 through its descriptor in device memory (512^3 stencil
+    // halo, by value / so: async gather 548 / 580 us, pipelined 617 / 551, stream 569 / 686)
+    if (op.list) {
+        GBX_TRY(req->mem.get(&op.d_self, 1));
+        const void *desc = op.d_desc;
+        GBX_CUDA_TRY(cudaMemcpyAsync(op.d_self, &desc, sizeof(desc), cudaMemcpyHostToDevice, req->stream));
+        GBX_CUDA_TRY(cudaStreamSynchronize(req->stream));
     }
     TuneVal best = {op.max_vec, 256, 1, 0, 1e30f};
     // candidate forms: segments, flat (gather or two-index), and the pipelined flat form
@@ -754,11 +771,11 @@ static int tune_launch(LevelLaunch &L, cudaStream_t st) {
             for (int pers = 1; pers >= (strm ? 1 : 0) && e == cudaSuccess; pers--) {
                 const int blk = blocks[bi];
                 const int grid = grid_for(L.kind, L.dtype, L.vec, fl, blk, pers, L.total_tiles, L.max_ctas);
-                e = launch_level(L, nullptr, fl, blk, grid, st, false);
+                e = launch_level(L, false, fl, blk, grid, st, false);
                 float t = 1e30f;
                 for (int r = 0; r < 3 && e == cudaSuccess; r++) {
                     cudaEventRecord(a, st);
-                    e = launch_level(L, nullptr, fl, blk, grid, st, false);
+                    e = launch_level(L, false, fl, blk, grid, st, false);
                     cudaEventRecord(b, st);
                     if (e == cudaSuccess) e = cudaEventSynchronize(b);
                     float x = 0;
@@ -861,7 +878,8 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
                 L.flat = kind ? ops[groups[g][0]]->fold_form
                               : (groups[g].size() == 1 && (keys[g].first & 15) != 15 && op_flat(*ops[groups[g][0]]) != 15
                                      ? op_flat(*ops[groups[g][0]]) : keys[g].first & 63);
-                L.one_op = !batch && groups[g].size() == 1 ? (int)groups[g][0] : -1;
+                // (a batch launches an op as it was tuned)
+                L.only = groups[g].size() == 1 && !(batch && ops[groups[g][0]]->list) ? ops[groups[g][0]] : nullptr;
                 L.one = 1;
                 for (size_t i : groups[g])
                     if (kind != 0 || ops[i]->cd.cpe != 1) L.one = 0;
@@ -895,8 +913,7 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
     return GBX_SUCCESS;
 }
 
-static cudaError_t enqueue_levels(const std::vector<LevelLaunch> &levels, const std::vector<HostOp> *ops,
-                                  cudaStream_t st) {
+static cudaError_t enqueue_levels(const std::vector<LevelLaunch> &levels, bool by_value, cudaStream_t st) {
     // The first launch follows the stream's earlier work, the others their predecessor.  A launch of
     // at most one block per SM may start beside its predecessor (dependent launch); a larger grid,
     // sized to what an SM holds, may not: the shared-memory / L1 split of an SM cannot change
@@ -906,20 +923,23 @@ static cudaError_t enqueue_levels(const std::vector<LevelLaunch> &levels, const 
     bool first = true;
     for (const LevelLaunch &L : levels) {
         GbxRange r(L.phase);
-        cudaError_t e = launch_level(L, ops, L.flat, L.block, L.grid, st, !first && L.grid <= gbx_num_sms());
+        // (the pipelined forms of a list read payload through the non-coherent path: never dependent)
+        const bool pipe_list = L.kind == 0 && (L.flat == 5 || L.flat == 7) && !(by_value && L.only);
+        const bool dep = !first && L.grid <= gbx_num_sms() && !pipe_list;
+        cudaError_t e = launch_level(L, by_value, L.flat, L.block, L.grid, st, dep);
         if (e != cudaSuccess) return e;
         first = false;
     }
     return cudaSuccess;
 }
 
-static int capture(const std::vector<LevelLaunch> &levels, const std::vector<HostOp> *ops, cudaGraphExec_t *exec) {
+static int capture(const std::vector<LevelLaunch> &levels, cudaGraphExec_t *exec) {
     cudaStream_t cs;
     GBX_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t e2 = enqueue_levels(levels, ops, cs);
+        cudaError_t e2 = enqueue_levels(levels, true, cs);
         e = cudaStreamEndCapture(cs, &graph);
         if (e == cudaSuccess) e = e2;
     }
@@ -979,7 +999,7 @@ static int finalize(gbx_request_s *req) {
     // now are the request's
     req->exec_src = req->src;
     req->exec_dst = req->dst;
-    if (req->use_graph && req->launches.size() > 1) GBX_TRY(capture(req->launches, &req->ops, &req->exec));
+    if (req->use_graph && req->launches.size() > 1) GBX_TRY(capture(req->launches, &req->exec));
     fill_info(req);
     return GBX_SUCCESS;
 }
@@ -1095,11 +1115,11 @@ static float program_ms(gbx_request_s *req) {
     // time of one eager pass over the levels (used by algorithm=auto)
     cudaEvent_t a, b;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return 1e30f;
-    enqueue_levels(req->launches, &req->ops, req->stream);
+    enqueue_levels(req->launches, req->use_graph, req->stream);
     float best = 1e30f;
     for (int r = 0; r < 3; r++) {
         cudaEventRecord(a, req->stream);
-        enqueue_levels(req->launches, &req->ops, req->stream);
+        enqueue_levels(req->launches, req->use_graph, req->stream);
         cudaEventRecord(b, req->stream);
         cudaEventSynchronize(b);
         float t = 0;
@@ -1301,14 +1321,14 @@ extern "C" int gbx_partitioned_init(gbx_request_t forward, int npart, const int6
 // read the descriptors in device memory, which a rebind rewrites, so that they can be.
 static int launch_program(gbx_request_s *req, cudaStream_t st) {
     if (!req->use_graph) {
-        GBX_CUDA_TRY(enqueue_levels(req->launches, nullptr, st));
+        GBX_CUDA_TRY(enqueue_levels(req->launches, false, st));
     } else if (req->exec && req->src == req->exec_src && req->dst == req->exec_dst) {
         GBX_CUDA_TRY(cudaGraphLaunch(req->exec, st));
     } else if (!req->launches.empty()) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         GBX_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
         if (cap != cudaStreamCaptureStatusNone) return GBX_ERR_CUDA;
-        GBX_CUDA_TRY(enqueue_levels(req->launches, &req->ops, st));
+        GBX_CUDA_TRY(enqueue_levels(req->launches, true, st));
     }
     return GBX_SUCCESS;
 }
@@ -1606,17 +1626,27 @@ extern "C" int gbx_startall(int count, gbx_request_t *reqs) {
         int rc = build_levels(b->mem, ops, dts, b->launches, 1, st, tune, cap);
         if (rc == GBX_SUCCESS && done_event_create(&b->done) != cudaSuccess)
             rc = GBX_ERR_CUDA;
-        if (rc == GBX_SUCCESS && !b->launches.empty()) rc = capture(b->launches, nullptr, &b->exec);
+        if (rc == GBX_SUCCESS && !b->launches.empty()) rc = capture(b->launches, &b->exec);
         if (rc != GBX_SUCCESS) {
             if (b->exec) cudaGraphExecDestroy(b->exec);
             if (b->done) cudaEventDestroy(b->done);
             delete b;
             return rc;
         }
-        for (gbx_request_s *r : key) r->batches.push_back(b);
+        for (gbx_request_s *r : key) {
+            r->batches.push_back(b);
+            b->bound.emplace_back(r->src, r->dst);
+        }
     }
     cudaStream_t st = reqs[0]->stream;
-    if (b->exec) GBX_CUDA_TRY(cudaGraphLaunch(b->exec, st));
+    if (b->exec && b->as_captured()) {
+        GBX_CUDA_TRY(cudaGraphLaunch(b->exec, st));
+    } else if (b->exec) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        GBX_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return GBX_ERR_CUDA;
+        GBX_CUDA_TRY(enqueue_levels(b->launches, true, st));
+    }
     if (b->other_streams) GBX_TRY(done_event_for_other_streams(&b->done, &b->done_timed));
     GBX_CUDA_TRY(cudaEventRecord(b->done, st));
     b->on = st;
@@ -1666,7 +1696,7 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
     // launches of one op take the new descriptor with their next start; the device descriptors
     // are rewritten only where a launch reads them
     bool lists = !req->use_graph || !req->batches.empty();
-    for (const LevelLaunch &L : req->launches) lists |= L.one_op < 0;
+    for (const LevelLaunch &L : req->launches) lists |= !L.only;
     if (lists) {
         for (HostOp &op : req->ops) GBX_TRY(upload_desc(req, op));
         req->desc_stale = 0;

@@ -143,6 +143,8 @@ struct HostOp {
     CopyDesc cd;     // host copies of the descriptor
     FoldDesc fd;
     void *d_desc;           // device descriptor
+    int list;               // its request's launches read d_desc (graph=0), and so do the tuner's,
+    void **d_self;          // through a list of this one op
     longlong2 *d_rec;       // fold: packed row records
     int64_t *d_tile_seg;    // copy: tile_seg storage sized for min_vec
     int32_t *d_flat_idx;    // copy: source element of every element when the flat form applies
@@ -185,8 +187,8 @@ struct LevelLaunch {
     int max_ctas;           // grid cap (0: none)
     const char *phase;      // NVTX name of the launch (a string literal)
     int one;                // copies: every op has one chunk per element (stream kernels specialise)
-    int one_op;             // index of the launch's only op in its request, whose descriptor is passed by
-                            // value; -1: pooled ops (and batches), read from d_ops
+    const HostOp *only;     // the launch's only op, whose descriptor may be passed by value; null: pooled
+                            // ops, read from d_ops
     void **d_ops;           // device array of descriptor pointers
     int64_t *d_prefix;      // device tile prefix (nops + 1)
 };

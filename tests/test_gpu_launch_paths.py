@@ -1,7 +1,7 @@
 """GPU: the ways a start reaches the device.  A launch of one op carries its descriptor by value,
-a start of several launches replays a graph until the first rebind and launches them one by one
-afterwards, graph=0 and batches read descriptors in device memory (rewritten by a rebind, or by
-the first batch after one).  Every way writes the oracle's bytes into the buffers bound at that
+a start of several launches replays a graph on the buffers bound at init and launches them one by one
+on others, graph=0 and pooled launches read descriptors in device memory (rewritten by a rebind, or
+by the first batch after one).  Every way writes the oracle's bytes into the buffers bound at that
 moment, whether the start is completed by the host, on the request's own stream or on another."""
 import numpy as np
 import pytest
@@ -66,6 +66,30 @@ def test_rebinds_between_starts(alg, info, how):
         other.request.wait()
         torch.cuda.synchronize()
         assert_bytes_equal(outs[k].cpu().numpy(), want[k], f"{alg} {info} {how} batch, buffers {k}")
+
+
+@pytest.mark.parametrize("info", ["", "graph=0"])
+def test_rebinds_between_batch_starts(info):
+    """A batch of a forward and its backward exchange: launches of one op each, by value."""
+    p = pt.stencil((24, 20, 16), (3, 2, 2), ppn=4, comps=8)
+    xs = [payload(p, 70 + k) for k in range(2)]
+    rng = np.random.default_rng(7)
+    ws = [rng.standard_normal(p.recvbuf_bytes // 8) for _ in range(2)]
+    sends, grads = [dev_bytes(x) for x in xs], [torch.from_numpy(w).cuda() for w in ws]
+    halo = [torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    gx = [torch.zeros(p.sendbuf_bytes // 8, dtype=torch.float64, device="cuda") for _ in range(2)]
+    ex = gbx.Exchange(p, sends[0], halo[0], "standard", info=info)
+    bwd = gbx.backward_init(ex.request, grads[0], gx[0], info=info)
+    for k, rebind in ((0, 0), (0, 0), (1, 1), (1, 0), (0, 1)):
+        if rebind:
+            ex.request.bind(sends[k], halo[k])
+            bwd.bind(grads[k], gx[k])
+        halo[k].fill_(0xA5)
+        gx[k].zero_()
+        gbx.startall([ex.request, bwd])
+        gbx.waitall([ex.request, bwd])
+        assert_bytes_equal(halo[k].cpu().numpy(), oracle.standard(p, xs[k], np.full(p.recvbuf_bytes, 0xA5, np.uint8)), "forward")
+        assert_bytes_equal(gx[k].cpu().numpy(), oracle.backward(p, ws[k], form=0), "backward")
 
 
 @pytest.mark.parametrize("comps", [1, 5, 2046, 2048, 2050, 6144])
