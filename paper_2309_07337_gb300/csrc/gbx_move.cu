@@ -39,8 +39,9 @@ template <> struct VecT<1> { typedef unsigned char T; };
 
 // Payload loads are plain ld.global: within a chain of dependent launches the payload may be
 // written (by the launch before) after this kernel has started, which the non-coherent path does
-// not allow for.  Indices and descriptors, fixed at init, use it.  (The two run equally fast
-// here, and so did L1::no_allocate, L2 prefetch hints and evict-first stores.)
+// not allow for.  Indices and descriptors, fixed at init, use it.  (With the descriptor in the
+// constant bank the two run equally fast, and so did L1::no_allocate, L2 prefetch hints and
+// evict-first stores.)
 template <int VEC>
 __device__ __forceinline__ typename VecT<VEC>::T ldv(const char *p) {
     return *reinterpret_cast<const typename VecT<VEC>::T *>(p);
@@ -1004,8 +1005,10 @@ int gbx_stream_prepare(void) {
 // so the bytes in flight per SM are set by the ring (192 KB) and not by the register file
 // (32 KB with one chunk per thread at full occupancy).  A warp waits only for copies it has
 // issued itself (cp.async.wait_group), never on a flag.  Bound by HBM: 512^3 stencil halo (64-byte
-// points, 3.57 GB of whole 128-byte lines) 558 us = 6.4 TB/s of line traffic; register-pipelined
-// form 561-576 us, stream form 569 us.  Chunks of 4 and 8 bytes gain nothing (2^20-row SpMV halo
+// points, 3.57 GB of whole 128-byte lines) 549 us = 6.5 TB/s of line traffic; flat form 543-589 us,
+// stream form 573, register-pipelined form 590-617.  More bytes in flight are not better: the shapes
+// of 64 KB per CTA are fastest at 2-2.5 CTAs per SM (548-551 us), with 3 they take 605 and 624.
+// Chunks of 4 and 8 bytes gain nothing (2^20-row SpMV halo
 // 45 us, stream form 38: a request per line and element bounds them, not bytes in flight).
 // Destinations in host memory (bulk_dst = 0) are stored by the lanes.
 template <int K, int S, int NW, int PS, typename L>
