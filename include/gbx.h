@@ -470,8 +470,9 @@ int gbx_request_bind(gbx_request_t request, const void *src, void *dst);
 /* One exchange from `src` into `dst`, in stream order: binds the two for this exchange only (as
  * gbx_request_bind, with its requirements), sets dst to zero bytes first when zero_dst is set,
  * starts the exchange after the work already on `stream` and completes it for `stream` (as
- * gbx_start and gbx_wait_stream); the request's own binding is unchanged (a captured exchange,
- * graph=0 only, leaves src and dst bound).  One call where a program with new buffers at every step
+ * gbx_start and gbx_wait_stream); the request's own binding is unchanged, whatever the call returns
+ * (except by a captured exchange, graph=0 only, which leaves src and dst bound; with graph=1 a call
+ * under a capture gives GBX_ERR_CUDA before anything is bound or enqueued).  One call where a program with new buffers at every step
  * (autograd) would make four.  The caller keeps src and dst alive until the work on `stream`
  * after the call has run. */
 int gbx_exchange_stream(gbx_request_t request, const void *src, void *dst, int zero_dst, void *stream);

@@ -1735,12 +1735,20 @@ extern "C" int gbx_exchange_stream(gbx_request_t req, const void *src, void *dst
     if (!req) return GBX_ERR_ARG;
     if (req->kind == 2) return GBX_ERR_UNSUPPORTED;
     if (req->active) return GBX_ERR_ACTIVE;
+    const cudaStream_t user = (cudaStream_t)stream;
+    // graph=1 launches cannot be captured (launch_program): refused here, while nothing is bound and
+    // nothing is in the caller's graph
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone, own_cap = cudaStreamCaptureStatusNone;
+    GBX_CUDA_TRY(cudaStreamIsCapturing(user, &cap));
+    GBX_CUDA_TRY(cudaStreamIsCapturing(req->stream, &own_cap));
+    const bool capturing = cap != cudaStreamCaptureStatusNone || own_cap != cudaStreamCaptureStatusNone;
+    if (capturing && req->use_graph && !req->launches.empty()) return GBX_ERR_CUDA;
     const char *const own_src = req->src;
     char *const own_dst = req->dst;
-    if ((cudaStream_t)stream != req->stream || (cudaStream_t)stream == cudaStreamPerThread) {
+    if (user != req->stream || user == cudaStreamPerThread) {
         cudaEvent_t ev;
         GBX_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-        cudaError_t e = cudaEventRecord(ev, (cudaStream_t)stream);
+        cudaError_t e = cudaEventRecord(ev, user);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(req->stream, ev, 0);
         cudaEventDestroy(ev);
         GBX_CUDA_TRY(e);
@@ -1752,13 +1760,16 @@ extern "C" int gbx_exchange_stream(gbx_request_t req, const void *src, void *dst
             GBX_CUDA_TRY(cudaMemsetAsync(req->dst, 0, (size_t)req->dst_bytes, req->stream));
         }
         GBX_TRY(enqueue_start(req));
-        return gbx_wait_stream(req, stream);
+        const int rc = gbx_wait_stream(req, stream);
+        if (rc != GBX_SUCCESS) {   // (a started exchange that `stream` could not be made to wait for: the host waits)
+            cudaStreamSynchronize(req->stream);
+            req->active = 0;
+        }
+        return rc;
     };
     const int rc = run();
     // (a replay of a capture reads the descriptors as they are then: they keep these buffers)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    GBX_CUDA_TRY(cudaStreamIsCapturing(req->stream, &cap));
-    if (cap != cudaStreamCaptureStatusNone) return rc;
+    if (rc == GBX_SUCCESS && capturing && !req->use_graph) return rc;
     const int rb = gbx_request_bind(req, own_src, own_dst);
     return rc != GBX_SUCCESS ? rc : rb;
 }

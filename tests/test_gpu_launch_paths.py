@@ -153,3 +153,34 @@ def test_start_under_capture_is_refused():
     ex.start()
     ex.wait()
     assert_bytes_equal(recv.cpu().numpy(), oracle.standard(p, x), "after the capture")
+
+
+@pytest.mark.parametrize("alg", ["standard", "locality"])
+@pytest.mark.parametrize("zero", [False, True])
+@pytest.mark.parametrize("joins", [False, True])
+def test_exchange_stream_under_capture_is_refused(alg, zero, joins):
+    """graph=1, on the capturing stream or with the request's own stream outside the capture: nothing
+    stays bound, nothing enters the caller's graph, the request's own stream joins no capture."""
+    p = pt.random_pattern(92, P=24, dtype="f64", max_count=60)
+    xs = [payload(p, k) for k in range(2)]
+    init = np.full(p.recvbuf_bytes, 0xA5, np.uint8)
+    own, other = (torch.full((p.recvbuf_bytes,), 0xA5, dtype=torch.uint8, device="cuda") for _ in range(2))
+    s, own_stream = torch.cuda.Stream(), torch.cuda.Stream()
+    send = dev_bytes(xs[1])
+    ex = gbx.Exchange(p, dev_bytes(xs[0]), own, alg, stream=own_stream if joins else s)
+    own.fill_(0xA5)
+    torch.cuda.synchronize()
+    probe = torch.zeros(4, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        probe.add_(1)
+        with pytest.raises(gbx.GbxError) as e:
+            ex.request.exchange_stream(send, other, zero_dst=zero, stream=s)
+    assert e.value.code == gbx.ERR_CUDA
+    g.replay()
+    ex.start()
+    ex.wait()
+    torch.cuda.synchronize()
+    assert probe.tolist() == [1.0] * 4
+    assert_bytes_equal(other.cpu().numpy(), init, "the refused call's destination")
+    assert_bytes_equal(own.cpu().numpy(), oracle.standard(p, xs[0], init), "the request's own buffers")
