@@ -920,12 +920,19 @@ static cudaError_t enqueue_levels(const std::vector<LevelLaunch> &levels, bool b
     // while the predecessor's blocks run on it, so it would get too little of either (2^20-row
     // SpMV halo, locality form in the stream form: 107 us as dependent launches, 68 without;
     // small grids are launch bound: three launches of 100-230 blocks 17.1 -> 13.4 us).
+    // Under a cap the launches together must stay within it, as the blocks of a dependent launch
+    // are resident beside its predecessor's.  A grid that a cap cut short is never dependent by this, so a
+    // dependent launch of the stream kernels has one tile per block, and their producers, which do
+    // not wait for the predecessor, never poll for a stage while it still runs.
+    int64_t blocks = 0;
+    for (const LevelLaunch &L : levels) blocks += L.grid;
     bool first = true;
     for (const LevelLaunch &L : levels) {
         GbxRange r(L.phase);
         // (the pipelined forms of a list read payload through the non-coherent path: never dependent)
         const bool pipe_list = L.kind == 0 && (L.flat == 5 || L.flat == 7) && !(by_value && L.only);
-        const bool dep = !first && L.grid <= gbx_num_sms() && !pipe_list;
+        const bool capped = L.max_ctas > 0 && blocks > L.max_ctas;
+        const bool dep = !first && L.grid <= gbx_num_sms() && !capped && !pipe_list;
         cudaError_t e = launch_level(L, by_value, L.flat, L.block, L.grid, st, dep);
         if (e != cudaSuccess) return e;
         first = false;

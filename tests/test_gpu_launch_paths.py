@@ -184,3 +184,50 @@ def test_exchange_stream_under_capture_is_refused(alg, zero, joins):
     assert probe.tolist() == [1.0] * 4
     assert_bytes_equal(other.cpu().numpy(), init, "the refused call's destination")
     assert_bytes_equal(own.cpu().numpy(), oracle.standard(p, xs[0], init), "the request's own buffers")
+
+
+def _smallest_limit(make):
+    """The smallest power of two as wait_limit with which five starts of a request succeed."""
+    for k in range(23):
+        r = make(1 << k)
+        try:
+            for _ in range(5):
+                r.start()
+                r.wait()
+            return 1 << k
+        except gbx.GbxError as e:
+            assert e.code == gbx.ERR_DEVICE_WAIT
+    raise AssertionError("no limit is enough")
+
+
+def test_capped_launches_do_not_wait_for_each_other():
+    """Two blocks per launch walk hundreds of tiles each: a launch that started beside its predecessor
+    would fill its stages and then spend its bounded wait on the predecessor's whole run.  A
+    limit well above what one launch needs by itself is enough for a chain of three."""
+    p = pt.spmv_halo(200003, 64, 8, 12, 5, "f64")
+    x, g = payload(p, 1), np.random.default_rng(2).standard_normal(p.recvbuf_bytes // 8)
+    send, grad = dev_bytes(x), torch.from_numpy(g).cuda()
+    recv = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+    gx = torch.zeros(p.sendbuf_bytes // 8, dtype=torch.float64, device="cuda")
+    dp, keep = gbx.DevicePattern(p), []
+
+    def forward(alg, limit):
+        keep.append(gbx.Exchange(p, send, recv, alg, info=f"stream=2;autotune=0;max_ctas=2;wait_limit={limit}", dp=dp))
+        assert keep[-1].info()["copy_forms"] == 1 << 10
+        return keep[-1].request
+
+    def backward(alg, limit):
+        r = gbx.backward_init(forward(alg, 1 << 22), grad, gx, info=f"stream=2;autotune=0;max_ctas=2;wait_limit={limit};"
+                                                                    "single_split=0")
+        assert r.info()["copy_forms"] & 1 << 12
+        return r
+
+    for make, out, want in ((forward, recv, oracle.standard(p, x)), (backward, gx, oracle.backward(p, g, form=1))):
+        limit = 16 * _smallest_limit(lambda n: make("standard", n))
+        r = make("locality", limit)
+        for _ in range(5):
+            out.zero_()
+            r.start()
+            r.wait()
+            assert_bytes_equal(out.cpu().numpy(), want, f"{make.__name__} {limit}")
+    gbx.device_status()
