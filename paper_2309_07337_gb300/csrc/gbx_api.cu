@@ -565,7 +565,7 @@ static cudaError_t launch_level(const LevelLaunch &L, bool by_value, int flat, i
 // cached by a signature of the op, so identical patterns are tuned once per process.
 struct TuneKey {
     int kind, max_vec, min_vec, dtype, flat_ok, list;
-    int64_t units, nseg, elem_size, nterms;
+    int64_t units, nseg, elem_size, nterms, max_ctas;
     bool operator<(const TuneKey &o) const {
         return memcmp(this, &o, sizeof(TuneKey)) < 0;
     }
@@ -625,6 +625,9 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
                                      8192 * op.ag_ok + 16384 * op.win_ok
                 : 0;
     key.list = op.list = !req->use_graph;
+    // few blocks want shapes with more threads and bytes in flight each (256^3 locality halo, 64 blocks:
+    // 375 us with the shapes of the whole GPU, 214 with its own)
+    key.max_ctas = req->max_ctas;
     int blocks[4] = {128, 256, 512, 1024};
     if (!req->autotune || req->forced_block) {
         op.block = req->forced_block ? req->forced_block : 256;

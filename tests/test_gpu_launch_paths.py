@@ -231,3 +231,31 @@ def test_capped_launches_do_not_wait_for_each_other():
             r.wait()
             assert_bytes_equal(out.cpu().numpy(), want, f"{make.__name__} {limit}")
     gbx.device_status()
+
+
+def _us(r, n=9):
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    t = []
+    for _ in range(n + 2):
+        ev[0].record()
+        r.start()
+        r.wait_stream()
+        ev[1].record()
+        ev[1].synchronize()
+        t.append(ev[0].elapsed_time(ev[1]) * 1e3)
+    return sorted(t[2:])[n // 2]
+
+
+def test_capped_requests_have_shapes_of_their_own():
+    """Shapes are tuned once per process and kind of op: the whole GPU's shapes of a form take up to
+    twice the time of its best one on a few blocks, so a capped request is tuned under its cap."""
+    p = pt.stencil((256,) * 3, (8,) * 3, 64, comps=8)
+    x = torch.zeros(p.sendbuf_bytes, dtype=torch.uint8, device="cuda")
+    y = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+    ex = gbx.Exchange(p, x, y)
+    dp, graph = ex.dp, ex.graph
+    us = {}
+    for form in ("", "form=1", "form=5", "form=14"):
+        gbx.Exchange(p, x, y, info=form, dp=dp, graph=graph)
+        us[form] = _us(gbx.Exchange(p, x, y, info="max_ctas=16;" + form, dp=dp, graph=graph).request)
+    assert max(us[""], us["form=5"], us["form=14"]) <= 1.45 * min(us.values()), us
