@@ -395,10 +395,17 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
     HostOp op;
     memset(&op, 0, sizeof(op));
     int64_t nruns = 0;
-    op.fd.row_ptr = row_ptr; op.fd.row_out = row_out; op.fd.terms = terms; op.fd.nrows = nrows;
-    GBX_TRY(gbx_make_wfold(req, &op.fd, nterms, &nruns, &op.wfold_ok));
+    auto window = [&]() -> int {
+        op.fd.row_ptr = row_ptr; op.fd.row_out = row_out; op.fd.terms = terms; op.fd.nrows = nrows;
+        return gbx_make_wfold(req, &op.fd, nterms, &nruns, &op.wfold_ok);
+    };
     // The window form takes single-term rows with the others, at the same cost per term: no split
-    // (3 of 10 rows single, 415 k rows fp32 in node-blocked order: 27.3 us, split copy and folds 34.9).
+    // (all terms in one launch against split copy and window fold of the rest, single values, 11 to 95 %
+    // of the rows single, both orders: 0.5 to 1.02 of the time on the whole GPU, once 1.08, and 0.72 to
+    // 1.25 at 152 blocks).  On a few blocks the copy kernels have more bytes in flight per block and the
+    // split is kept (up to 48 blocks: 0.96 to 2.5, with 64 down to 0.86).
+    const bool few = req->max_ctas > 0 && req->max_ctas <= 48;
+    if (!few) GBX_TRY(window());
     if (!accumulate && !req->no_single_split && !op.wfold_ok) {
         // rows with one term are copies: a two-index flat copy op takes them
         int32_t *gs = nullptr, *gd = nullptr;
@@ -419,6 +426,7 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
             nterms = nt;
         }
     }
+    if (few) GBX_TRY(window());
     op.kind = 1;
     op.level = level;
     op.units = nrows;

@@ -99,3 +99,19 @@ def test_wait_gives_up():
         b.wait()
     assert e.value.code == gbx.ERR_DEVICE_WAIT
     assert gbx.device_status() == 1
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("nb", ["faces", "all"])
+def test_single_rows_on_few_blocks(dtype, nb):
+    """Up to 48 blocks, rows of one term go through a copy of their own and the window form takes the
+    rest, where it is large enough; with more blocks, and when accumulating, it takes all rows."""
+    p = pt.stencil((96, 96, 96), (8, 8, 8), 16, 1, dtype, nb)
+    _, ex = forward(p, payload(p, 1))
+    g, old = grad_payload(p, 3), payload(p, 4)
+    for cap, acc in ((1, False), (48, False), (48, True), (49, False), (0, False)):
+        got, b = backward(ex, g, grad_send_init=old, accumulate=acc, info=f"form=2;max_ctas={cap}")
+        assert_bytes_equal(got, oracle.backward(p, g, grad_send=old, form=0, accumulate=acc), f"cap {cap} {acc}")
+        copies = b.info()["copy_forms"] & ~(FORM | 1 << 12)
+        assert bool(copies) == (0 < cap <= 48 and not acc), (cap, acc, b.info()["copy_forms"])
+        assert b.info()["copy_forms"] & FORM, (cap, acc, b.info()["copy_forms"])
