@@ -3,6 +3,8 @@ a start of several launches replays a graph on the buffers bound at init and lau
 on others, graph=0 and pooled launches read descriptors in device memory (rewritten by a rebind, or
 by the first batch after one).  Every way writes the oracle's bytes into the buffers bound at that
 moment, whether the start is completed by the host, on the request's own stream or on another."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -22,6 +24,15 @@ from gpu_util import assert_bytes_equal, dev_bytes, payload  # noqa: E402
 def built():
     import __graft_entry__
     __graft_entry__.build()
+
+
+@pytest.fixture(autouse=True)
+def no_collection():
+    """Requests of earlier tests that a collection frees inside a capture would invalidate it."""
+    gc.collect()
+    gc.disable()
+    yield
+    gc.enable()
 
 
 def _complete(how, r, side):
