@@ -235,11 +235,11 @@ static int agather_ok_for(const gbx_request_s *req, int max_vec) {
 // every offset of a 16-byte vector op and every buffer bound to it).
 static void set_bulk_dst(CopyDesc &d) { d.bulk_dst = !host_mem(d.dst); }
 
-// The window form reads its windows with the bulk-copy engine from 16-byte aligned device memory
-// (every window starts at a multiple of 16 bytes), with plain loads otherwise.
-static void set_win_bulk(CopyDesc &d) {
-    d.win_bulk = d.src && !((uintptr_t)d.src & 15) && !host_mem(d.src);
-    d.win_bulk2 = d.src2 && !((uintptr_t)d.src2 & 15) && !host_mem(d.src2);
+// The window form reads its windows with the bulk-copy engine from device memory (every window starts
+// a multiple of 16 bytes into its buffer), with plain loads from host memory.
+static void set_win_lead(CopyDesc &d) {
+    d.win_lead = host_mem(d.src) ? -1 : (int)((uintptr_t)d.src & 15);
+    d.win_lead2 = host_mem(d.src2) ? -1 : (int)((uintptr_t)d.src2 & 15);
 }
 
 // Elements of the buffer an op's pointer of this role reads.
@@ -261,7 +261,7 @@ static int add_window(gbx_request_s *req, HostOp &op) {
     d.win_elems = t.elems;
     d.nwin = op.nwin = t.npieces;
     op.algo_bytes_win = d.nelem * (2 * req->elem_size + 2) + d.nelem / 4 + 4 * t.nruns + 32 * t.npieces;
-    set_win_bulk(d);
+    set_win_lead(d);
     return GBX_SUCCESS;
 }
 
@@ -1705,7 +1705,7 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
             if (op.cd.src_role == ROLE_SRC) op.cd.src = ns;
             if (op.cd.dst_role == ROLE_DST) op.cd.dst = nd;
             set_bulk_dst(op.cd);
-            if (op.win_ok) set_win_bulk(op.cd);
+            if (op.win_ok) set_win_lead(op.cd);
         } else {
             if (op.fd.out_role == ROLE_DST) op.fd.out = nd;
             if (op.fd.a_role == ROLE_SRC) op.fd.bufA = ns;
@@ -1735,7 +1735,7 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
             c.cd.src = o.cd.src;
             c.cd.dst = o.cd.dst;
             c.cd.bulk_dst = o.cd.bulk_dst;
-            c.cd.win_bulk = o.cd.win_bulk;
+            c.cd.win_lead = o.cd.win_lead;
             if (((uintptr_t)c.cd.src | (uintptr_t)c.cd.dst) & (uintptr_t)(c.cd.vec - 1)) {
                 stale.push_back(b);
                 break;

@@ -70,8 +70,8 @@ def test_edges(P, n, region, deg, s):
 
 @pytest.mark.parametrize("s", [4, 8])
 def test_rebind_and_batch(s):
-    """Sources one element past a 16-byte boundary and in host memory (lane copies instead of the
-    bulk engine), destinations in host memory, then a batch of two patterns in one launch."""
+    """Sources one element past a 16-byte boundary and in host memory (lane copies for ends or all of
+    the windows), destinations in host memory, then a batch of two patterns in one launch."""
     p, q = ring(16, 1500, 999, s, 3), ring(5, 4097, 1025, s, 4)
     xs = [pt.random_bytes(p.sendbuf_bytes, k) for k in range(3)]
     y = pt.random_bytes(q.sendbuf_bytes, 9)
@@ -100,6 +100,57 @@ def test_rebind_and_batch(s):
                 ex.start()
                 ex.wait()
             assert_bytes_equal(out.cpu().numpy(), oracle.standard(p, x), f"batch={batch}")
+
+
+@pytest.mark.parametrize("s,off", [(4, 4), (4, 8), (4, 12), (8, 8)])
+def test_sources_off_a_16_byte_boundary(s, off):
+    """At init and after a bind: windows whose first and last 16-byte units are partly theirs, down to
+    single elements, in the first and last window of the buffer, in both window sizes and a batch."""
+    for P, n, region, deg in CASES:
+        p = ring(P, n, region, s, n + s, deg)
+        x = pt.random_bytes(p.sendbuf_bytes, n)
+        want = oracle.standard(p, x)
+        room = torch.zeros(p.sendbuf_bytes + 16, dtype=torch.uint8, device="cuda")
+        src = room[off:off + p.sendbuf_bytes]
+        src.copy_(dev_bytes(x))
+        recv = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+        late = torch.zeros_like(recv)
+        ex = gbx.Exchange(p, src, recv, info="form=15")
+        assert ex.info()["copy_forms"] & FORM
+        other = gbx.Exchange(p, dev_bytes(x), late, info="form=15;block=128", dp=ex.dp, graph=ex.graph)
+        other.request.bind(src, late)
+        for start in (lambda: (ex.start(), other.start()), lambda: gbx.startall([ex.request, other.request])):
+            recv.zero_()
+            late.zero_()
+            start()
+            gbx.waitall([ex.request, other.request])
+            assert_bytes_equal(recv.cpu().numpy(), want, f"{p.name} +{off}")
+            assert_bytes_equal(late.cpu().numpy(), want, f"{p.name} +{off} bound later")
+
+
+def test_time_off_a_16_byte_boundary():
+    """Windows copied by the lanes alone took three times as long."""
+    p = pt.spmv_halo_torch(1 << 19, 512, 32, 20, 5, "f64")
+    n = p.sendbuf_bytes // 8
+    x = torch.zeros(n + 1, dtype=torch.float64, device="cuda")
+    y = torch.zeros(p.recvbuf_bytes // 8, dtype=torch.float64, device="cuda")
+    ex = gbx.Exchange(p, x[:n], y, info="form=15")
+    assert ex.info()["copy_forms"] & FORM
+    us = []
+    for src in (x[:n], x[1:]):
+        ex.request.bind(src, y)
+        t = []
+        for _ in range(12):
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            ev[0].record()
+            for _ in range(10):
+                ex.start()
+                ex.request.wait_stream()
+            ev[1].record()
+            ev[1].synchronize()
+            t.append(ev[0].elapsed_time(ev[1]) * 100)
+        us.append(sorted(t)[6])
+    assert us[1] <= 1.5 * us[0], us
 
 
 def test_wait_gives_up():
