@@ -233,7 +233,10 @@ static int agather_ok_for(const gbx_request_s *req, int max_vec) {
 
 // The async gather's bulk stores write device memory only (their run is 16-byte aligned, as
 // every offset of a 16-byte vector op and every buffer bound to it).
-static void set_bulk_dst(CopyDesc &d) { d.bulk_dst = !host_mem(d.dst); }
+static void set_bulk_dst(HostOp &op) {
+    op.host_dst = host_mem(op.cd.dst);
+    op.cd.bulk_dst = !op.host_dst;
+}
 
 // The window form reads its windows with the bulk-copy engine from device memory (every window starts
 // a multiple of 16 bytes into its buffer), with plain loads from host memory.
@@ -315,7 +318,7 @@ int gbx_make_copy_op(gbx_request_s *req, int level, const char *src, int src_rol
         op.algo_bytes_flat = 2 * nelem * req->elem_size + 4 * nelem;
         op.stream_ok = op.flat_ok && stream_ok_for(req, op.d_flat_idx, nullptr, op.max_vec);
         op.ag_ok = op.flat_ok && agather_ok_for(req, op.max_vec);
-        set_bulk_dst(d);
+        set_bulk_dst(op);
         if (op.flat_ok && idx) GBX_TRY(add_window(req, op));
     }
     if (req->allow_bulk && !host_mem(src) && !host_mem(dst)) {
@@ -356,7 +359,7 @@ int gbx_make_flat_op(gbx_request_s *req, int level, const char *src, int src_rol
     d.status = req->status_dev; d.wait_limit = req->wait_limit;
     op.stream_ok = stream_ok_for(req, g, nullptr, op.max_vec);
     op.ag_ok = agather_ok_for(req, op.max_vec);
-    set_bulk_dst(d);
+    set_bulk_dst(op);
     if (windows) GBX_TRY(add_window(req, op));
     GBX_TRY(req->mem.alloc(&op.d_desc, sizeof(CopyDesc)));
     req->ops.push_back(op);
@@ -395,7 +398,9 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
     HostOp op;
     memset(&op, 0, sizeof(op));
     int64_t nruns = 0;
+    op.host_dst = host_mem(out);
     auto window = [&]() -> int {
+        if (op.host_dst) return GBX_SUCCESS;   // (see launch_alone)
         op.fd.row_ptr = row_ptr; op.fd.row_out = row_out; op.fd.terms = terms; op.fd.nrows = nrows;
         return gbx_make_wfold(req, &op.fd, nterms, &nruns, &op.wfold_ok);
     };
@@ -566,6 +571,29 @@ static cudaError_t launch_level(const LevelLaunch &L, bool by_value, int flat, i
                            L.dtype, L.vec, block, grid, st, flat, dep);
 }
 
+// One op of a launch in a window form, by itself.  Window forms store in the order of their source:
+// runs, or single values, which L2 gathers into lines for device memory, but which go to host memory piece by
+// piece.  An op bound to host memory after it was tuned on device memory runs here in the stream form, a
+// fold in the fold kernel (2^20-row SpMV halo into host memory, fp64 728 -> 455 us, fp32 of a fifth of the
+// entries 238 -> 78; its reverse fp64 232 -> 85, in the stream fold 105).
+static cudaError_t launch_alone(const LevelLaunch &L, size_t i, bool by_value, cudaStream_t st) {
+    const HostOp &op = *L.ops[i];
+    int flat = L.flat, block = L.block, persistent = 1;
+    int64_t tiles = L.kind ? op.fd.nwpiece : form_tiles(op, L.flat);
+    if (op.host_dst) {
+        flat = L.kind ? 0 : op.stream_ok && L.vec >= 4 ? 10 : 1;
+        block = L.kind ? 1024 : 256;
+        persistent = !L.kind;
+        tiles = ceil_div(L.kind ? op.fd.nchunks : op.cd.nchunks, GBX_TILE);
+    }
+    const int grid = grid_for(L.kind, L.dtype, L.vec, flat, block, persistent, tiles, L.max_ctas);
+    if (L.kind == 0)
+        return gbx_launch_copy({by_value ? &op.cd : nullptr, (const CopyDesc *const *)L.d_ops + i, nullptr, 1, tiles}, L.vec,
+                               launch_code(flat, op.cd.cpe == 1), block, grid, st, false);
+    return gbx_launch_fold({by_value ? &op.fd : nullptr, (const FoldDesc *const *)L.d_ops + i, nullptr, 1, tiles}, L.dtype,
+                           L.vec, block, grid, st, flat, false);
+}
+
 // ------------------------------------------------------------------ autotuner
 // Times every candidate shape of an op (vector width, block size, grid mode) with
 // CUDA events on the request's stream and keeps the fastest.  Results never depend on
@@ -573,7 +601,7 @@ static cudaError_t launch_level(const LevelLaunch &L, bool by_value, int flat, i
 // cached by a signature of the op, so identical patterns are tuned once per process.
 struct TuneKey {
     int kind, max_vec, min_vec, dtype, flat_ok, list;
-    int64_t units, nseg, elem_size, nterms, max_ctas;
+    int64_t units, nseg, elem_size, nterms, max_ctas, host;
     bool operator<(const TuneKey &o) const {
         return memcmp(this, &o, sizeof(TuneKey)) < 0;
     }
@@ -636,6 +664,7 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
     // few blocks want shapes with more threads and bytes in flight each (256^3 locality halo, 64 blocks:
     // 375 us with the shapes of the whole GPU, 214 with its own)
     key.max_ctas = req->max_ctas;
+    key.host = host_mem(req->src) + 2 * host_mem(req->dst);
     int blocks[4] = {128, 256, 512, 1024};
     if (!req->autotune || req->forced_block) {
         op.block = req->forced_block ? req->forced_block : 256;
@@ -898,6 +927,7 @@ static int build_levels(DevPool &mem, const std::vector<HostOp *> &ops, const st
                 std::vector<int64_t> pre(1, 0);
                 const HostOp *big = ops[groups[g][0]];
                 for (size_t i : groups[g]) {
+                    L.ops.push_back(ops[i]);
                     ptrs.push_back(ops[i]->d_desc);
                     pre.push_back(pre.back() + (kind ? op_tiles(*ops[i]) : form_tiles(*ops[i], L.flat)));
                     if (op_tiles(*ops[i]) > op_tiles(*big)) big = ops[i];
@@ -944,7 +974,12 @@ static cudaError_t enqueue_levels(const std::vector<LevelLaunch> &levels, bool b
         const bool pipe_list = L.kind == 0 && (L.flat == 5 || L.flat == 7) && !(by_value && L.only);
         const bool capped = L.max_ctas > 0 && blocks > L.max_ctas;
         const bool dep = !first && L.grid <= gbx_num_sms() && !capped && !pipe_list;
-        cudaError_t e = launch_level(L, by_value, L.flat, L.block, L.grid, st, dep);
+        bool alone = false;   // some op of a window form has a host destination
+        if (L.kind ? L.flat == 2 : (L.flat & 31) == 15)
+            for (const HostOp *op : L.ops) alone |= op->host_dst != 0;
+        cudaError_t e = cudaSuccess;
+        if (!alone) e = launch_level(L, by_value, L.flat, L.block, L.grid, st, dep);
+        for (size_t i = 0; alone && e == cudaSuccess && i < L.ops.size(); i++) e = launch_alone(L, i, by_value, st);
         if (e != cudaSuccess) return e;
         first = false;
     }
@@ -1704,10 +1739,11 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
         if (op.kind == 0) {
             if (op.cd.src_role == ROLE_SRC) op.cd.src = ns;
             if (op.cd.dst_role == ROLE_DST) op.cd.dst = nd;
-            set_bulk_dst(op.cd);
+            set_bulk_dst(op);
             if (op.win_ok) set_win_lead(op.cd);
         } else {
             if (op.fd.out_role == ROLE_DST) op.fd.out = nd;
+            op.host_dst = host_mem(op.fd.out);
             if (op.fd.a_role == ROLE_SRC) op.fd.bufA = ns;
         }
     }
@@ -1735,6 +1771,7 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
             c.cd.src = o.cd.src;
             c.cd.dst = o.cd.dst;
             c.cd.bulk_dst = o.cd.bulk_dst;
+            c.host_dst = o.host_dst;
             c.cd.win_lead = o.cd.win_lead;
             if (((uintptr_t)c.cd.src | (uintptr_t)c.cd.dst) & (uintptr_t)(c.cd.vec - 1)) {
                 stale.push_back(b);

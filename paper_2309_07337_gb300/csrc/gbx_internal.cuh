@@ -165,6 +165,7 @@ struct HostOp {
     int64_t algo_bytes_win;
     int sfold_ok;           // fold: records and terms aligned and padded, one payload class: the
                             // stream form of the fold is available
+    int host_dst;           // the destination bound now is host memory
     int wfold_ok;           // fold: the window form is available
     int64_t algo_bytes_fold, algo_bytes_wfold;
     int fold_form;          // fold: 0 the fold kernel, 1 its stream form, 2 its window form (tuned)
@@ -187,6 +188,7 @@ struct LevelLaunch {
     int max_ctas;           // grid cap (0: none)
     const char *phase;      // NVTX name of the launch (a string literal)
     int one;                // copies: every op has one chunk per element (stream kernels specialise)
+    std::vector<const HostOp *> ops;
     const HostOp *only;     // the launch's only op, whose descriptor may be passed by value; null: pooled
                             // ops, read from d_ops
     void **d_ops;           // device array of descriptor pointers
