@@ -70,6 +70,7 @@ struct Opts {
     int graph = 1, autotune = 1, vec = 0, block = 0, timeout_ms = 60000, min_run = 4, piece = 0, flat = -1;
     int split = 1, split_order = 2;   // 2: source order where the scatter form can run, else dest
     int check_dup = 0, bulk = 1, max_ctas = 0, wait_limit = GBX_WAIT_LIMIT, stream = 1, form = -1;
+    bool windows = true;   // build the tables of the window forms (no key: see init_request)
     bool ok = true;
 };
 
@@ -252,7 +253,7 @@ static int64_t role_elems(const gbx_request_s *req, int role) {
 
 static int add_window(gbx_request_s *req, HostOp &op) {
     CopyDesc &d = op.cd;
-    if (!req->allow_stream || op.max_vec != req->elem_size) return GBX_SUCCESS;   // one chunk per element
+    if (!req->allow_stream || req->no_windows || op.max_vec != req->elem_size) return GBX_SUCCESS;   // one chunk per element
     WinTables t;
     GBX_TRY(gbx_make_window(req, d.flat_idx, d.nelem, role_elems(req, d.src_role),
                             d.src2 ? role_elems(req, d.src2_role) : 0, &t, &op.win_ok));
@@ -400,7 +401,7 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
     int64_t nruns = 0;
     op.host_dst = host_mem(out);
     auto window = [&]() -> int {
-        if (op.host_dst) return GBX_SUCCESS;   // (see launch_alone)
+        if (op.host_dst || req->no_windows) return GBX_SUCCESS;   // (host_dst: see launch_alone)
         op.fd.row_ptr = row_ptr; op.fd.row_out = row_out; op.fd.terms = terms; op.fd.nrows = nrows;
         return gbx_make_wfold(req, &op.fd, nterms, &nruns, &op.wfold_ok);
     };
@@ -1145,6 +1146,7 @@ static gbx_request_s *new_request(const Opts &o, void *stream) {
     req->wait_limit = o.wait_limit;
     req->allow_stream = o.stream;
     req->forced_form = o.form;
+    req->no_windows = !o.windows;
     if (done_event_create(&req->done) != cudaSuccess) {
         cudaGetLastError();
         req->done = nullptr;
@@ -1162,6 +1164,20 @@ static gbx_request_s *new_request(const Opts &o, void *stream) {
         req->status_dev = (int *)d;
     }
     return req;
+}
+
+// Builds a request by `build`; when the device memory does not suffice, once more without the tables
+// and workspaces of the window forms, which an exchange can do without (a gather's: up to 17 and 32
+// bytes per element).
+template <typename Build>
+static int init_request(Opts &o, const Build &build) {
+    int rc = build();
+    if (rc == GBX_ERR_NOMEM && o.stream) {
+        cudaGetLastError();
+        o.windows = false;
+        rc = build();
+    }
+    return rc;
 }
 
 static float program_ms(gbx_request_s *req) {
@@ -1205,7 +1221,7 @@ extern "C" int gbx_neighbor_alltoallv_init(const void *sendbuf, int64_t sendbuf_
     Opts o = parse_info(info);
     if (!o.ok) return GBX_ERR_ARG;
 
-    auto build = [&](int locality, gbx_request_s **out) -> int {
+    auto build_once = [&](int locality, gbx_request_s **out) -> int {
         GbxRange range(locality ? "gbx.setup.forward_locality" : "gbx.setup.forward_standard");
         gbx_request_s *req = new_request(o, stream);
         if (!req->done) { destroy_request(req); return GBX_ERR_CUDA; }
@@ -1224,6 +1240,7 @@ extern "C" int gbx_neighbor_alltoallv_init(const void *sendbuf, int64_t sendbuf_
         *out = req;
         return GBX_SUCCESS;
     };
+    auto build = [&](int locality, gbx_request_s **out) { return init_request(o, [&] { return build_once(locality, out); }); };
 
     gbx_request_s *req = nullptr;
     if (o.algorithm_auto) {
@@ -1261,21 +1278,23 @@ extern "C" int gbx_neighbor_alltoallw_init(const void *sendbuf, int64_t sendbuf_
     if (!o.ok) return GBX_ERR_ARG;
     if (o.algorithm != GBX_ALG_STANDARD || o.algorithm_auto) return GBX_ERR_UNSUPPORTED;
     GbxRange range("gbx.setup.alltoallw");
-    gbx_request_s *req = new_request(o, stream);
-    if (!req->done) { destroy_request(req); return GBX_ERR_CUDA; }
-    req->kind = 0;
-    req->graph = graph;
-    req->src = (const char *)sendbuf;
-    req->dst = (char *)recvbuf;
-    req->src_bytes = sendbuf_bytes;
-    req->dst_bytes = recvbuf_bytes;
-    req->dtype = dtype;
-    int rc = gbx_setup_alltoallw(req, send_base, sendcounts, sdispls, sendtypes, recv_base, recvcounts, rdispls,
-                                 recvtypes, types, ntypes);
-    if (rc == GBX_SUCCESS) rc = finalize(req);
-    if (rc != GBX_SUCCESS) { destroy_request(req); return rc; }
-    *request = req;
-    return GBX_SUCCESS;
+    return init_request(o, [&]() -> int {
+        gbx_request_s *req = new_request(o, stream);
+        if (!req->done) { destroy_request(req); return GBX_ERR_CUDA; }
+        req->kind = 0;
+        req->graph = graph;
+        req->src = (const char *)sendbuf;
+        req->dst = (char *)recvbuf;
+        req->src_bytes = sendbuf_bytes;
+        req->dst_bytes = recvbuf_bytes;
+        req->dtype = dtype;
+        int rc = gbx_setup_alltoallw(req, send_base, sendcounts, sdispls, sendtypes, recv_base, recvcounts, rdispls,
+                                     recvtypes, types, ntypes);
+        if (rc == GBX_SUCCESS) rc = finalize(req);
+        if (rc != GBX_SUCCESS) { destroy_request(req); return rc; }
+        *request = req;
+        return GBX_SUCCESS;
+    });
 }
 
 // ------------------------------------------------------------ partitioned
@@ -1286,18 +1305,8 @@ static int check_part_ptr(int n, const int64_t *ptr, int64_t bytes) {
     return GBX_SUCCESS;
 }
 
-extern "C" int gbx_partitioned_init(gbx_request_t forward, int npart, const int64_t *part_ptr, int nrpart,
-                                    const int64_t *rpart_ptr, const char *info, void *stream,
-                                    gbx_request_t *request) {
-    if (!request) return GBX_ERR_ARG;
-    *request = nullptr;
-    if (!forward || forward->kind != 0) return GBX_ERR_ARG;
-    if (forward->algorithm != GBX_ALG_STANDARD) return GBX_ERR_UNSUPPORTED;
-    GBX_TRY(check_part_ptr(npart, part_ptr, forward->src_bytes));
-    GBX_TRY(check_part_ptr(nrpart, rpart_ptr, forward->dst_bytes));
-    Opts o = parse_info(info);
-    if (!o.ok) return GBX_ERR_ARG;
-    GbxRange range("gbx.setup.partitioned");
+static int build_partitioned(gbx_request_t forward, int npart, const int64_t *part_ptr, int nrpart,
+                             const int64_t *rpart_ptr, const Opts &o, void *stream, gbx_request_t *request) {
     gbx_request_s *req = new_request(o, stream);
     if (!req->done) { destroy_request(req); return GBX_ERR_CUDA; }
     req->kind = 2;
@@ -1366,6 +1375,21 @@ extern "C" int gbx_partitioned_init(gbx_request_t forward, int npart, const int6
     I.algo_bytes = algo;
     *request = req;
     return GBX_SUCCESS;
+}
+
+extern "C" int gbx_partitioned_init(gbx_request_t forward, int npart, const int64_t *part_ptr, int nrpart,
+                                    const int64_t *rpart_ptr, const char *info, void *stream,
+                                    gbx_request_t *request) {
+    if (!request) return GBX_ERR_ARG;
+    *request = nullptr;
+    if (!forward || forward->kind != 0) return GBX_ERR_ARG;
+    if (forward->algorithm != GBX_ALG_STANDARD) return GBX_ERR_UNSUPPORTED;
+    GBX_TRY(check_part_ptr(npart, part_ptr, forward->src_bytes));
+    GBX_TRY(check_part_ptr(nrpart, rpart_ptr, forward->dst_bytes));
+    Opts o = parse_info(info);
+    if (!o.ok) return GBX_ERR_ARG;
+    GbxRange range("gbx.setup.partitioned");
+    return init_request(o, [&] { return build_partitioned(forward, npart, part_ptr, nrpart, rpart_ptr, o, stream, request); });
 }
 
 // The request's kernels on `st`.  graph=1: one launch with its descriptor by value, or the graph
@@ -1445,24 +1469,26 @@ extern "C" int gbx_backward_init(gbx_request_t forward, const void *grad_recv, v
     Opts o = parse_info(info);
     if (!o.ok) return GBX_ERR_ARG;
     GbxRange range("gbx.setup.backward");
-    gbx_request_s *req = new_request(o, stream);
-    if (!req->done) { destroy_request(req); return GBX_ERR_CUDA; }
-    req->kind = 1;
-    req->forward = forward;
-    req->graph = forward->graph;
-    req->src = (const char *)grad_recv;
-    req->dst = (char *)grad_send;
-    req->src_bytes = forward->dst_bytes;
-    req->dst_bytes = forward->src_bytes;
-    req->elem_size = forward->elem_size;
-    req->dtype = forward->dtype;
-    req->algorithm = forward->algorithm;
-    req->align = forward->align | (uint64_t)(uintptr_t)grad_recv | (uint64_t)(uintptr_t)grad_send;
-    int rc = gbx_setup_backward(req, accumulate ? 1 : 0);
-    if (rc == GBX_SUCCESS) rc = finalize(req);
-    if (rc != GBX_SUCCESS) { destroy_request(req); return rc; }
-    *request = req;
-    return GBX_SUCCESS;
+    return init_request(o, [&]() -> int {
+        gbx_request_s *req = new_request(o, stream);
+        if (!req->done) { destroy_request(req); return GBX_ERR_CUDA; }
+        req->kind = 1;
+        req->forward = forward;
+        req->graph = forward->graph;
+        req->src = (const char *)grad_recv;
+        req->dst = (char *)grad_send;
+        req->src_bytes = forward->dst_bytes;
+        req->dst_bytes = forward->src_bytes;
+        req->elem_size = forward->elem_size;
+        req->dtype = forward->dtype;
+        req->algorithm = forward->algorithm;
+        req->align = forward->align | (uint64_t)(uintptr_t)grad_recv | (uint64_t)(uintptr_t)grad_send;
+        int rc = gbx_setup_backward(req, accumulate ? 1 : 0);
+        if (rc == GBX_SUCCESS) rc = finalize(req);
+        if (rc != GBX_SUCCESS) { destroy_request(req); return rc; }
+        *request = req;
+        return GBX_SUCCESS;
+    });
 }
 
 // ------------------------------------------------------------- start / wait

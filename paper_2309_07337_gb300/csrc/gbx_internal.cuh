@@ -207,6 +207,7 @@ struct gbx_request_s {
     int forced_flat;         // -1: the tuner chooses the flat form or segments; 0 / 1: forced
     int allow_flat;
     int no_combine;          // locality form: keep direct copies and redistribution apart
+    int no_windows;          // no tables of the window forms
     int no_single_split;     // keep single-term fold rows in the fold
     int split_order;         // single-term rows as copies: 0 in row (destination) order, 1 in source order
     int check_dup;           // locality form: compare every deduplicated value's bytes with its representative's at init

@@ -218,6 +218,58 @@ def test_time_into_host_memory():
     assert max(us[:2]) <= 1.3 * us[2] and max(us[3:5]) <= 1.3 * us[5], us
 
 
+@pytest.mark.parametrize("what", ["forward", "backward"])
+def test_too_little_memory_for_the_tables(what):
+    """With just the memory that a request needs without window forms it is built without them."""
+    p = ring(1000, 2000, 1900, 8, 3, 4, "f64")
+    x, g = pt.random_bytes(p.sendbuf_bytes, 1), np.random.default_rng(2).standard_normal(p.recvbuf_bytes // 8)
+    send, grad = dev_bytes(x), torch.from_numpy(g).cuda()
+    recv = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+    gx = torch.zeros(p.sendbuf_bytes // 8, dtype=torch.float64, device="cuda")
+    fwd = gbx.Exchange(p, send, recv, info="stream=0;min_run=0")
+
+    def make(info):
+        if what == "forward":
+            return gbx.Exchange(p, send, recv, info="min_run=0;" + info, dp=fwd.dp, graph=fwd.graph).request
+        return gbx.backward_init(fwd.request, grad, gx, accumulate=True, info=info)
+
+    bit = 1 << (15 if what == "forward" else 13)
+    for info in ("stream=0", "form=15" if what == "forward" else "form=2"):   # (loads the kernels)
+        r = make(info)
+        assert bool(r.info()["copy_forms"] & bit) == (info != "stream=0")
+        r.free()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    block, keep = 16 << 20, []
+    try:
+        free = torch.cuda.mem_get_info()[0]
+        keep = [torch.empty(free - (4 << 30), dtype=torch.uint8, device="cuda")]
+        while torch.cuda.mem_get_info()[0] > 5 * block:
+            keep.append(torch.empty(block, dtype=torch.uint8, device="cuda"))
+        r = None
+        while r is None:
+            assert len(keep) > 1
+            keep.pop()
+            torch.cuda.empty_cache()
+            try:
+                r = make("stream=0")
+            except gbx.GbxError as e:
+                assert e.code == gbx.ERR_NOMEM
+        r.free()
+        r = make("")
+    finally:
+        del keep
+        torch.cuda.empty_cache()
+    assert not r.info()["copy_forms"] & bit
+    gx.zero_()
+    r.start()
+    r.wait()
+    if what == "forward":
+        assert_bytes_equal(recv.cpu().numpy(), oracle.standard(p, x), what)
+    else:
+        assert_bytes_equal(gx.cpu().numpy(), oracle.backward(p, g, form=0), what)
+
+
 def test_wait_gives_up():
     p = ring(16, 1500, 999, 8, 7)
     x = pt.random_bytes(p.sendbuf_bytes, 7)
