@@ -1041,7 +1041,16 @@ static int finalize(gbx_request_s *req) {
     }
     {
         GbxRange r("gbx.setup.tune");
-        for (HostOp &op : req->ops) GBX_TRY(tune_op(req, op));
+        for (HostOp &op : req->ops) {
+            GBX_TRY(tune_op(req, op));
+            // (a fold's form is final; a gather's window tables also serve batches, which run it in the
+            // window form when most of their elements do)
+            if (op.kind == 1 && op.wfold_ok && op.fold_form != 2) {
+                gbx_drop_wfold(req, &op.fd);
+                op.wfold_ok = 0;
+                GBX_TRY(upload_desc(req, op));
+            }
+        }
     }
     GbxRange r("gbx.setup.capture");
     std::vector<HostOp *> ptrs;

@@ -21,6 +21,7 @@
 
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/gbx.h"
@@ -60,12 +61,13 @@ static inline int bitlen_u64(uint64_t x) { int n = 0; while (x) { n++; x >>= 1; 
 
 // Device allocations owned by one object; freed together.
 struct DevPool {
-    std::vector<void *> ptrs;
+    std::vector<std::pair<void *, size_t>> ptrs;
     int64_t bytes = 0;
     int alloc(void **p, size_t n);   // GBX_SUCCESS / GBX_ERR_NOMEM
     template <typename T>
     int get(T **p, int64_t count) { return alloc(reinterpret_cast<void **>(p), (size_t)(count > 0 ? count : 1) * sizeof(T)); }
     void release();
+    void drop(const void *p);   // frees one of its allocations (waits for the device)
     void give_to(DevPool &other) {   // its allocations become the other pool's
         other.ptrs.insert(other.ptrs.end(), ptrs.begin(), ptrs.end());
         other.bytes += bytes;
@@ -335,6 +337,7 @@ int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t
 int gbx_window_prepare(void);
 // Window-form tables of a fold's rows into `d`; *ok = 0 where the form does not apply.
 int gbx_make_wfold(gbx_request_s *req, FoldDesc *d, int64_t nterms, int64_t *nruns, int *ok);
+void gbx_drop_wfold(gbx_request_s *req, FoldDesc *d);
 int gbx_wfold_prepare(void);
 int gbx_stream_prepare(void);
 int gbx_agather_prepare(void);

@@ -19,15 +19,25 @@ int DevPool::alloc(void **p, size_t n) {
         *p = nullptr;
         return GBX_ERR_NOMEM;
     }
-    ptrs.push_back(*p);
+    ptrs.emplace_back(*p, n);
     bytes += (int64_t)n;
     return GBX_SUCCESS;
 }
 
 void DevPool::release() {
-    for (void *p : ptrs) cudaFree(p);
+    for (const auto &p : ptrs) cudaFree(p.first);
     ptrs.clear();
     bytes = 0;
+}
+
+void DevPool::drop(const void *p) {
+    for (size_t i = 0; i < ptrs.size(); i++)
+        if (ptrs[i].first == p) {
+            cudaFree(ptrs[i].first);
+            bytes -= (int64_t)ptrs[i].second;
+            ptrs.erase(ptrs.begin() + (ptrdiff_t)i);
+            return;
+        }
 }
 
 // --------------------------------------------------------------------------- scan

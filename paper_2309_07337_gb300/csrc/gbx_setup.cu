@@ -1501,18 +1501,20 @@ int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t
     GBX_TRY(gbx_read_i64(first + nw, &np, st));
     t->npieces = np;
     if (np * we > 2 * nelem) return GBX_SUCCESS;
-    GBX_TRY(req->mem.get(&t->pieces, np));
-    GBX_TRY(req->mem.get(&t->idx, np * GBX_WIN_N));
-    GBX_TRY(req->mem.get(&t->grp, np * (GBX_WIN_N / 32)));
-    GBX_TRY(req->mem.get(&t->run, np * GBX_WIN_RUNS));
+    DevPool tp;
+    GBX_TRY(tp.get(&t->pieces, np));
+    GBX_TRY(tp.get(&t->idx, np * GBX_WIN_N));
+    GBX_TRY(tp.get(&t->grp, np * (GBX_WIN_N / 32)));
+    GBX_TRY(tp.get(&t->run, np * GBX_WIN_RUNS));
     win_fill_kernel<<<(unsigned)np, WIN_FILL_T, 0, st>>>(g, key, elem, start, first, nw, nelem, s, we, nw1, src_elems,
                                                          src2_elems, t->pieces, t->idx, t->grp, t->run, bad);
     GBX_CUDA_TRY(cudaGetLastError());
     int hb = 0;
     GBX_CUDA_TRY(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
     GBX_CUDA_TRY(cudaStreamSynchronize(st));
-    if (hb) return GBX_SUCCESS;   // (the tables stay allocated with the request, unused)
+    if (hb) return GBX_SUCCESS;
     GBX_TRY(gbx_window_prepare());
+    tp.give_to(req->mem);
     *ok = 1;
     return GBX_SUCCESS;
 }
@@ -1777,6 +1779,15 @@ int gbx_make_wfold(gbx_request_s *req, FoldDesc *d, int64_t nterms, int64_t *nru
     tp.give_to(req->mem);
     *ok = 1;
     return GBX_SUCCESS;
+}
+
+void gbx_drop_wfold(gbx_request_s *req, FoldDesc *d) {
+    for (const void *p : {(const void *)d->wpiece, (const void *)d->wpos, (const void *)d->wbase, (const void *)d->wrowcnt,
+                          (const void *)d->wrowout, (const void *)d->wgrp, (const void *)d->wrun, (const void *)d->wgroup})
+        req->mem.drop(p);
+    d->wpiece = nullptr; d->wpos = nullptr; d->wbase = nullptr; d->wrowcnt = nullptr; d->wrowout = nullptr;
+    d->wgrp = nullptr; d->wrun = nullptr; d->wgroup = nullptr;
+    d->nwpiece = 0;
 }
 
 __global__ void check_bulk_kernel(const BulkTask *tasks, int64_t n, int64_t src_bytes, int64_t dst_bytes, int *err) {

@@ -115,3 +115,16 @@ def test_single_rows_on_few_blocks(dtype, nb):
         copies = b.info()["copy_forms"] & ~(FORM | 1 << 12)
         assert bool(copies) == (0 < cap <= 48 and not acc), (cap, acc, b.info()["copy_forms"])
         assert b.info()["copy_forms"] & FORM, (cap, acc, b.info()["copy_forms"])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_tables_of_a_form_not_chosen_are_freed(dtype):
+    """A request in another fold form holds as much memory as one that had no window tables."""
+    p = pt.spmv_halo(60007, 97, 11, 13, 5, dtype)
+    _, ex = forward(p, payload(p, 1))
+    g, old = grad_payload(p, 3), payload(p, 4)
+    _, plain = backward(ex, g, grad_send_init=old, info="stream=0;single_split=0")   # builds no window tables
+    got, b = backward(ex, g, grad_send_init=old, info="form=1;single_split=0")
+    assert b.info()["copy_forms"] == 1 << 12 and plain.info()["copy_forms"] == 0
+    assert b.info()["device_bytes"] <= plain.info()["device_bytes"] + 64
+    assert_bytes_equal(got, oracle.backward(p, g, grad_send=old, form=0), dtype)
