@@ -138,8 +138,10 @@ def _nbytes(t) -> int:
 
 def _stream_handle(stream) -> Optional[int]:
     import torch
-    if stream is None:   # the current stream's handle, without building a Stream object (2.7 us)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if stream is None:
+        # the current stream's handle, without building a Stream object (2.7 us) where torch has a call for it
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
     return stream.cuda_stream
 
 

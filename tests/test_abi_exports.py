@@ -67,3 +67,17 @@ def test_oracle_and_library_error_codes_agree():
     hdr = open(os.path.join(ROOT, "include", "gbx.h")).read()
     for name, val in re.findall(r"#define GBX_(ERR_\w+)\s+(\d+)", hdr):
         assert getattr(g, name) == int(val), name
+
+
+def test_stream_handle_without_torch_internals(monkeypatch):
+    """The current stream's handle comes from torch's raw call where there is one, else from the Stream."""
+    import types
+    import torch
+    import paper_2309_07337_gb300 as g
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=17))
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda d: 100 + d, raising=False)
+    assert g._stream_handle(None) == 103
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    assert g._stream_handle(None) == 17
+    assert g._stream_handle(types.SimpleNamespace(cuda_stream=5)) == 5
