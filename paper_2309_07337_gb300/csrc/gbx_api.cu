@@ -219,17 +219,12 @@ static int stream_ok_for(const gbx_request_s *req, const int32_t *g, const int32
 }
 
 // The async gather takes flat gathers of 16-byte chunks, where it was measured ahead of the
-// register-pipelined and stream forms (512^3 stencil halo 558 us against 561-576 and 569); with
+// register-pipelined and stream forms (512^3 stencil halo 549 us against 590-617 and 573); with
 // narrower chunks it was behind (2^20-row SpMV halo, 8 bytes: 45 us against 38).  Info stream=0
 // leaves it out with the other forms that stage in shared memory.
 static int agather_ok_for(const gbx_request_s *req, int max_vec) {
-    static int prepared = 0;
-    if (!req->allow_stream || max_vec < 16) return 0;
-    if (!prepared) {
-        if (gbx_agather_prepare() != GBX_SUCCESS) return 0;
-        prepared = 1;
-    }
-    return 1;
+    // (prepared for the device that is current now, whichever requests came before)
+    return req->allow_stream && max_vec >= 16 && gbx_agather_prepare() == GBX_SUCCESS;
 }
 
 // The async gather's bulk stores write device memory only (their run is 16-byte aligned, as
