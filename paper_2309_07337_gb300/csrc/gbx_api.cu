@@ -259,7 +259,8 @@ static int add_window(gbx_request_s *req, HostOp &op) {
     d.win_run = t.run;
     d.win_elems = t.elems;
     d.nwin = op.nwin = t.npieces;
-    op.algo_bytes_win = d.nelem * (2 * req->elem_size + 2) + d.nelem / 4 + 4 * t.nruns + 32 * t.npieces;
+    // every window read once, and per element its value written and 2 bytes of index; the tables' other parts
+    op.algo_bytes_win = t.window_bytes + d.nelem * (req->elem_size + 2) + d.nelem / 4 + 4 * t.nruns + 32 * t.npieces;
     set_win_lead(d);
     return GBX_SUCCESS;
 }

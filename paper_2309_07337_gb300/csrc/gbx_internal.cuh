@@ -330,7 +330,8 @@ struct WinTables {
     uint2 *grp;
     int32_t *run;
     int64_t npieces, nruns;
-    int elems;   // source elements per window
+    int64_t window_bytes;   // of all windows read
+    int elems;              // source elements per window
 };
 int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t src_elems, int64_t src2_elems,
                     WinTables *t, int *ok);

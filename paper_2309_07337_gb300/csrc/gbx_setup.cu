@@ -1500,6 +1500,7 @@ int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t
     GBX_TRY(gbx_scan_i64(cnt, first, nw, st, ws));
     GBX_TRY(gbx_read_i64(first + nw, &np, st));
     t->npieces = np;
+    t->window_bytes = nw * we * s;
     if (np * we > 2 * nelem) return GBX_SUCCESS;
     DevPool tp;
     GBX_TRY(tp.get(&t->pieces, np));

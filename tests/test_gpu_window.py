@@ -153,6 +153,19 @@ def test_time_off_a_16_byte_boundary():
     assert us[1] <= 1.5 * us[0], us
 
 
+@pytest.mark.parametrize("s", [4, 8])
+def test_algorithmic_bytes(s):
+    """Every window counts once, however many elements and pieces read it."""
+    for (P, n, region, deg), we in ((CASES[4], 1024), (CASES[0], 2048)):
+        p = ring(P, n, region, s, n, deg)
+        _, ex = forward(p, pt.random_bytes(p.sendbuf_bytes, n), info="form=15")
+        rank = np.repeat(np.arange(p.P), np.diff(p.send_slot_ptr))
+        windows = len(np.unique((np.asarray(p.send_base)[rank] // s + p.send_idx) // we))
+        low = windows * we * s + p.volume * (s + 2)
+        assert ex.info()["copy_forms"] == FORM
+        assert low < ex.info()["algo_bytes"] < low + p.volume * 9 // 4 + 32 * (windows + p.volume // 2048 + 1)
+
+
 def _host(n, dtype=torch.uint8):
     return torch.zeros(n, dtype=dtype).pin_memory()
 
