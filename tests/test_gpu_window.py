@@ -102,6 +102,51 @@ def test_rebind_and_batch(s):
             assert_bytes_equal(out.cpu().numpy(), oracle.standard(p, x), f"batch={batch}")
 
 
+def _kernels(fn):
+    """Names of the kernels that run in fn ([] where the profiler records none)."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        fn()
+        torch.cuda.synchronize()
+    return [e.name for e in prof.events() if "gbx_" in e.name]
+
+
+@pytest.mark.parametrize("s", [4, 8])
+@pytest.mark.parametrize("sizes", [("wide",), ("narrow",), ("wide", "narrow"), ("narrow", "other"), ("wide", "narrow", "other"),
+                                   ("narrow", "other", "other")])
+def test_batch_of_both_window_sizes(s, sizes):
+    """One launch takes windows of 1024 and of 2048 elements, and an op tuned to another form where most
+    elements were tuned to windows; where they were not, none runs in windows."""
+    make = {"wide": (ring(130, 4, 200, s, 3, 129), 2048, "form=15"), "narrow": (ring(16, 1500, 999, s, 4), 1024, "form=15"),
+            "other": (ring(12, 1500, 999, s, 5), 1024, "form=1")}
+    items = []
+    for k, w in enumerate(sizes):
+        p, _, info = make[w]
+        x = pt.random_bytes(p.sendbuf_bytes, k)
+        out = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda")
+        ex = gbx.Exchange(p, dev_bytes(x), out, info=info)
+        assert ex.info()["copy_forms"] == (FORM if w != "other" else 2)
+        items.append((p, x, out, ex))
+    reqs = [i[3].request for i in items]
+
+    def start():
+        gbx.startall(reqs)
+        gbx.waitall(reqs)
+
+    start()                                          # (builds and tunes the batch)
+    for _, _, out, _ in items:
+        out.zero_()
+    names = _kernels(start)
+    for p, x, out, _ in items:
+        assert_bytes_equal(out.cpu().numpy(), oracle.standard(p, x), f"{p.name} {sizes}")
+    tuned = sum(p.volume if w != "other" else -p.volume for w, (p, _, _, _) in zip(sizes, items))
+    if names and tuned >= 0:
+        assert len(names) == 1 and "gbx_window_kernel" in names[0], names
+        assert f"<{s}, {2048 if 'wide' in sizes else 1024}," in names[0], names
+    elif names:
+        assert not any("gbx_window_kernel" in k for k in names), names
+
+
 @pytest.mark.parametrize("s,off", [(4, 4), (4, 8), (4, 12), (8, 8)])
 def test_sources_off_a_16_byte_boundary(s, off):
     """At init and after a bind: windows whose first and last 16-byte units are partly theirs, down to
