@@ -542,12 +542,14 @@ static int op_flat(const HostOp &op) { return op.kind == 0 ? op.cd.flat : op.fol
 // every op of the launch has one chunk per element (one).
 static int launch_code(int flat, int one) { return (flat == 10 || flat == 11) && one ? flat + 2 : flat; }
 
-// The window form's launch code carries the window size (15: 1024 elements, 47: 2048).
+// The window form's launch code carries the window size (15: 1024 elements, 47: 2048) and, added when
+// it is launched, whether some source lies off a 16-byte boundary.
 static int window_code(const CopyDesc &d) { return d.win_elems > 1024 ? 47 : 15; }
+static int window_shift(const CopyDesc &d) { return d.win_lead > 0 || d.win_lead2 > 0 ? 128 : 0; }
 
 static cudaError_t launch_op_alone(gbx_request_s *req, HostOp &op, int block, int persistent) {
     const int64_t tiles = op_tiles(op);
-    const int vec = op_vec(op), flat = op.kind == 0 && op_flat(op) == 15 ? window_code(op.cd) : op_flat(op);
+    const int vec = op_vec(op), flat = op.kind == 0 && op_flat(op) == 15 ? window_code(op.cd) | window_shift(op.cd) : op_flat(op);
     const int grid = grid_for(op.kind, req->dtype, vec, flat, block, persistent, tiles, req->max_ctas);
     if (op.kind == 0)
         return gbx_launch_copy({op.d_self ? nullptr : &op.cd, (const CopyDesc *const *)op.d_self, nullptr, 1, tiles}, vec,
@@ -561,6 +563,8 @@ static cudaError_t launch_op_alone(gbx_request_s *req, HostOp &op, int block, in
 static cudaError_t launch_level(const LevelLaunch &L, bool by_value, int flat, int block, int grid,
                                 cudaStream_t st, bool dep) {
     const HostOp *op = by_value ? L.only : nullptr;
+    if (L.kind == 0 && (flat & 31) == 15)
+        for (const HostOp *o : L.ops) flat |= window_shift(o->cd);
     if (L.kind == 0)
         return gbx_launch_copy({op ? &op->cd : nullptr, (const CopyDesc *const *)L.d_ops, L.d_prefix, L.nops, L.total_tiles},
                                L.vec, launch_code(flat, L.one), block, grid, st, dep);
@@ -575,7 +579,7 @@ static cudaError_t launch_level(const LevelLaunch &L, bool by_value, int flat, i
 // entries 238 -> 78; its reverse fp64 232 -> 85, in the stream fold 105).
 static cudaError_t launch_alone(const LevelLaunch &L, size_t i, bool by_value, cudaStream_t st) {
     const HostOp &op = *L.ops[i];
-    int flat = L.flat, block = L.block, persistent = 1;
+    int flat = L.kind ? L.flat : L.flat | window_shift(op.cd), block = L.block, persistent = 1;
     int64_t tiles = L.kind ? op.fd.nwpiece : form_tiles(op, L.flat);
     if (op.host_dst) {
         flat = L.kind ? 0 : op.stream_ok && L.vec >= 4 ? 10 : 1;

@@ -1130,11 +1130,8 @@ int gbx_agather_prepare(void) {
 // ------------------------------------------------------------------ window
 // Window form of a flat gather of elements of VEC bytes (tables: WinPiece).  Warp 0 is the
 // producer: per piece it has the bulk-copy engine read the source window and the piece's tables
-// into one of S shared-memory stages, completing on the stage's "full" mbarrier.  A window lies in
-// its stage as far from a 16-byte boundary as in the source, so the engine reads all of it but the
-// parts of a 16-byte unit at its ends, which the lanes copy (an unaligned source copied by the lanes
-// alone: 2^20-row halo 99 us fp64, 89 fp32; now as aligned ones, 31 and 27).  Sources in host memory they
-// copy whole.  The consumer warps pick the elements out of the window and store them: 32 consecutive slots of a piece per
+// into one of S shared-memory stages, completing on the stage's "full" mbarrier.  The consumer
+// warps pick the elements out of the window and store them: 32 consecutive slots of a piece per
 // warp and step, whose destinations are runs of consecutive elements.  The element index costs 2
 // bytes and its share of a run instead of 4, every source line is read whole by the copy
 // engine, and no load of a single element goes through L1.  That is what bounds the other forms
@@ -1143,19 +1140,24 @@ int gbx_agather_prepare(void) {
 // best of them and takes 30.3 (fp32: 28.5 -> 21.0), its locality form 63.5 -> 52.5, a start of 16
 // uneven patterns 115 -> 78; now shared-memory and store wavefronts (54 %) and the 2-CTA ramp
 // weigh most.  Waits bounded as in the stream form.
-#define GBX_WIN_LEAD 16   // room for a window up to 15 bytes into a 16-byte unit
+// Sources off a 16-byte boundary (SHIFT): a window lies as far from a boundary in its stage as in the
+// source, so that the engine reads all of it but the partial 16-byte units at its ends, which the
+// producer's lanes copy.  2^20-row halo from such a source: 33 us fp64 and 28 fp32, 99 and 89 where
+// the lanes copy whole windows, as they do without SHIFT, and from host memory.  A kernel of its own, as the few
+// instructions more per piece cost the others time (fp32 halo in locality form 37.0 -> 37.7 us).
+#define GBX_WIN_LEAD(shift) ((shift) ? 16 : 0)   // room before a window
 #define GBX_WIN_TABLES (GBX_WIN_N * 2 + GBX_WIN_N / 32 * 8 + GBX_WIN_RUNS * 4)
 
-template <int VEC, int WE, int NT, int S, int PS, typename L>
+template <int VEC, int WE, int NT, int S, int PS, bool SHIFT, typename L>
 __global__ void __launch_bounds__(NT, PS) gbx_window_kernel(const __grid_constant__ L list) {
     typedef typename VecT<VEC>::T V;
     constexpr int NCW = NT / 32 - 1, U = 4;
-    constexpr int WB = WE * VEC, STAGE = WB + GBX_WIN_LEAD + GBX_WIN_TABLES;
-    constexpr int OFF_IDX = WB + GBX_WIN_LEAD, OFF_GRP = OFF_IDX + GBX_WIN_N * 2, OFF_RUN = OFF_GRP + GBX_WIN_N / 32 * 8;
+    constexpr int WB = WE * VEC, STAGE = WB + GBX_WIN_LEAD(SHIFT) + GBX_WIN_TABLES;
+    constexpr int OFF_IDX = WB + GBX_WIN_LEAD(SHIFT), OFF_GRP = OFF_IDX + GBX_WIN_N * 2, OFF_RUN = OFF_GRP + GBX_WIN_N / 32 * 8;
     extern __shared__ __align__(128) unsigned char gbx_window_smem[];
     __shared__ __align__(8) uint64_t full[S], empty[S];
     __shared__ char *dst_s[S];
-    __shared__ int n_s[S], lead_s[S];
+    __shared__ int n_s[S], lead_s[SHIFT ? S : 1];
     __shared__ volatile int abort_flag;
     pdl_trigger();
     const int64_t npieces = list.tiles();
@@ -1190,19 +1192,6 @@ __global__ void __launch_bounds__(NT, PS) gbx_window_kernel(const __grid_constan
         for (int64_t k = 0;; k++) {
             const int64_t t = blockIdx.x + k * gridDim.x;
             if (t >= npieces) break;
-            // all that the piece's copies need, read while its stage is still in use (16 uneven patterns: 80.6 us,
-            // 81.7 when read after the wait)
-            const char *src = (P.buf ? d->src2 : d->src) + P.src;
-            const bool good = P.n > 0 && P.n <= GBX_WIN_N && P.nrun > 0 && P.nrun <= GBX_WIN_RUNS && P.bytes > 0 && P.bytes <= WB;
-            // window byte o lies at lead + o of the stage; the engine reads [head, head + b16), the lanes the rest
-            const int wl = P.buf ? d->win_lead2 : d->win_lead;
-            const uint32_t lead = wl < 0 ? 0u : (uint32_t)wl, bytes = good ? (uint32_t)P.bytes : 0u;
-            const uint32_t head = min(bytes, (16u - lead) & 15u), b16 = wl < 0 ? 0u : (bytes - head) & ~15u;
-            const bool rest = b16 < bytes;
-            char *const dst = d->dst + d->dst_flat0;
-            const uint16_t *const g_idx = d->win_idx + lt * GBX_WIN_N;
-            const uint2 *const g_grp = d->win_grp + lt * (GBX_WIN_N / 32);
-            const int32_t *const g_run = d->win_run + lt * GBX_WIN_RUNS;
             const int q = (int)(k % S);
             bool go = k < S || bulk_wait(sempty + 8 * q, (uint32_t)((k / S - 1) & 1), limit);
             go = __all_sync(0xffffffffu, go && !abort_flag);
@@ -1212,49 +1201,45 @@ __global__ void __launch_bounds__(NT, PS) gbx_window_kernel(const __grid_constan
                 break;
             }
             const uint32_t fb = sfull + 8 * q, stage = sbuf + q * STAGE;
+            const char *src = (P.buf ? d->src2 : d->src) + P.src;
+            const bool good = P.n > 0 && P.n <= GBX_WIN_N && P.nrun > 0 && P.nrun <= GBX_WIN_RUNS && P.bytes > 0 && P.bytes <= WB;
+            // window byte o lies at lead + o of the stage; the engine reads [head, head + b16), the lanes the rest
+            const int wl = P.buf ? d->win_lead2 : d->win_lead;
+            const uint32_t lead = SHIFT && wl > 0 ? (uint32_t)wl : 0u, head = SHIFT ? min((uint32_t)P.bytes, (16u - lead) & 15u) : 0u;
+            const uint32_t b16 = (SHIFT ? wl >= 0 : wl == 0) ? ((uint32_t)P.bytes - head) & ~15u : 0u;
+            unsigned char *win = gbx_window_smem + q * STAGE + lead;
+            if (good) {
+                if (SHIFT && lane * VEC < head) *reinterpret_cast<V *>(win + lane * VEC) = ldv<VEC>(src + lane * VEC);
+                for (uint32_t o = head + b16 + lane * VEC; o < (uint32_t)P.bytes; o += 32 * VEC)
+                    *reinterpret_cast<V *>(win + o) = ldv<VEC>(src + o);
+            }
+            __syncwarp();
             if (lane == 0) {
-                dst_s[q] = dst;
+                dst_s[q] = d->dst + d->dst_flat0;
                 n_s[q] = good ? P.n : 0;
-                lead_s[q] = (int)lead;
+                if (SHIFT) lead_s[q] = (int)lead;
                 if (!good) {   // validated at init; recorded, skipped
                     gbx_raise(list, 2);
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fb) : "memory");
                 } else {
+                    const int64_t slot = lt * GBX_WIN_N;
                     const uint32_t ib = ((uint32_t)P.n * 2 + 15) & ~15u, gb = (((uint32_t)P.n + 31) / 32 * 8 + 15) & ~15u,
                                    rb = ((uint32_t)P.nrun * 4 + 15) & ~15u;
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // consumers' reads before the refill
-                    if (rest)
-                        asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;"
-                                     ::"r"(fb), "r"(b16 + ib + gb + rb) : "memory");
-                    else
-                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                                     ::"r"(fb), "r"(b16 + ib + gb + rb) : "memory");
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
+                                 "r"(b16 + ib + gb + rb)
+                                 : "memory");
                     if (b16)
                         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                                      ::"r"(stage + lead + head), "l"(src + head), "r"(b16), "r"(fb) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(stage + OFF_IDX), "l"(g_idx), "r"(ib), "r"(fb) : "memory");
+                                 ::"r"(stage + OFF_IDX), "l"(d->win_idx + slot), "r"(ib), "r"(fb) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(stage + OFF_GRP), "l"(g_grp), "r"(gb), "r"(fb) : "memory");
+                                 ::"r"(stage + OFF_GRP), "l"(d->win_grp + slot / 32), "r"(gb), "r"(fb) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(stage + OFF_RUN), "l"(g_run), "r"(rb), "r"(fb) : "memory");
+                                 ::"r"(stage + OFF_RUN), "l"(d->win_run + lt * GBX_WIN_RUNS), "r"(rb), "r"(fb) : "memory");
                     last[q] = k;
                 }
-            }
-            if (rest) {   // while those copies run
-                unsigned char *win = gbx_window_smem + q * STAGE + lead;
-                if (lane * VEC < head) *reinterpret_cast<V *>(win + lane * VEC) = ldv<VEC>(src + lane * VEC);
-                for (uint32_t o = head + b16 + lane * VEC; o < bytes; o += 32 * VEC * U) {
-                    V v[U];
-#pragma unroll
-                    for (int u = 0; u < U; u++)
-                        if (o + u * 32 * VEC < bytes) v[u] = ldv<VEC>(src + o + u * 32 * VEC);
-#pragma unroll
-                    for (int u = 0; u < U; u++)
-                        if (o + u * 32 * VEC < bytes) *reinterpret_cast<V *>(win + o + u * 32 * VEC) = v[u];
-                }
-                __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fb) : "memory");
             }
             const int64_t tn = t + gridDim.x;
             if (tn < npieces) {
@@ -1281,7 +1266,7 @@ __global__ void __launch_bounds__(NT, PS) gbx_window_kernel(const __grid_constan
             break;
         }
         const unsigned char *stage = gbx_window_smem + q * STAGE;
-        const V *win = reinterpret_cast<const V *>(stage + lead_s[q]);
+        const V *win = reinterpret_cast<const V *>(stage + (SHIFT ? lead_s[q] : 0));
         const uint16_t *idx = reinterpret_cast<const uint16_t *>(stage + OFF_IDX);
         const uint2 *grp = reinterpret_cast<const uint2 *>(stage + OFF_GRP);
         const int32_t *run = reinterpret_cast<const int32_t *>(stage + OFF_RUN);
@@ -1316,13 +1301,13 @@ template <> struct WinShape<4096> { static constexpr int S0 = 2, P0 = 8, S1 = 3,
 template <> struct WinShape<8192> { static constexpr int S0 = 2, P0 = 6, S1 = 3, P1 = 4, S2 = 6, P2 = 2; };
 template <> struct WinShape<16384> { static constexpr int S0 = 2, P0 = 4, S1 = 2, P1 = 4, S2 = 4, P2 = 2; };
 
-template <int VEC, int WE, typename L>
+template <int VEC, int WE, bool SHIFT, typename L>
 static cudaError_t window_launch_v(int block, int grid, cudaStream_t st, bool dep, const L &l) {
     typedef WinShape<VEC * WE> H;
-    constexpr size_t B = VEC * WE + GBX_WIN_LEAD + GBX_WIN_TABLES;
-    if (block <= 128) return launch(gbx_window_kernel<VEC, WE, 160, H::S0, H::P0, L>, grid, 160, H::S0 * B, st, dep, l);
-    if (block <= 256) return launch(gbx_window_kernel<VEC, WE, 288, H::S1, H::P1, L>, grid, 288, H::S1 * B, st, dep, l);
-    return launch(gbx_window_kernel<VEC, WE, 544, H::S2, H::P2, L>, grid, 544, H::S2 * B, st, dep, l);
+    constexpr size_t B = VEC * WE + GBX_WIN_LEAD(SHIFT) + GBX_WIN_TABLES;
+    if (block <= 128) return launch(gbx_window_kernel<VEC, WE, 160, H::S0, H::P0, SHIFT, L>, grid, 160, H::S0 * B, st, dep, l);
+    if (block <= 256) return launch(gbx_window_kernel<VEC, WE, 288, H::S1, H::P1, SHIFT, L>, grid, 288, H::S1 * B, st, dep, l);
+    return launch(gbx_window_kernel<VEC, WE, 544, H::S2, H::P2, SHIFT, L>, grid, 544, H::S2 * B, st, dep, l);
 }
 
 template <int WB> static int win_per_sm(int block) {
@@ -1333,25 +1318,40 @@ static int window_per_sm(int vec, int wide, int block) {
     return wb == 4096 ? win_per_sm<4096>(block) : wb == 8192 ? win_per_sm<8192>(block) : win_per_sm<16384>(block);
 }
 
+template <int VEC, int WE, typename L>
+static cudaError_t window_launch_s(int shift, int block, int grid, cudaStream_t st, bool dep, const L &l) {
+    return shift ? window_launch_v<VEC, WE, true>(block, grid, st, dep, l) : window_launch_v<VEC, WE, false>(block, grid, st, dep, l);
+}
+
+// code: the launch code (15, + 32 for the wide windows, + 128 for sources off a 16-byte boundary)
 template <typename L>
-static cudaError_t window_launch(int vec, int wide, int block, int grid, cudaStream_t st, bool dep, const L &l) {
-    if (vec == 8) return wide ? window_launch_v<8, 2048>(block, grid, st, dep, l) : window_launch_v<8, 1024>(block, grid, st, dep, l);
-    if (vec == 4) return wide ? window_launch_v<4, 2048>(block, grid, st, dep, l) : window_launch_v<4, 1024>(block, grid, st, dep, l);
+static cudaError_t window_launch(int vec, int code, int block, int grid, cudaStream_t st, bool dep, const L &l) {
+    const int wide = code >> 5 & 1, shift = code >> 7 & 1;
+    if (vec == 8)
+        return wide ? window_launch_s<8, 2048>(shift, block, grid, st, dep, l) : window_launch_s<8, 1024>(shift, block, grid, st, dep, l);
+    if (vec == 4)
+        return wide ? window_launch_s<4, 2048>(shift, block, grid, st, dep, l) : window_launch_s<4, 1024>(shift, block, grid, st, dep, l);
     return cudaErrorInvalidValue;   // offered for elements of 4 and 8 bytes
 }
 
-template <int VEC, int WE, int NT, int S, int PS>
+template <int VEC, int WE, int NT, int S, int PS, bool SHIFT>
 static cudaError_t window_attr_k() {
-    return smem_attr(gbx_window_kernel<VEC, WE, NT, S, PS, OneOp<CopyDesc>>,
-                     gbx_window_kernel<VEC, WE, NT, S, PS, OpList<CopyDesc>>, S * (VEC * WE + GBX_WIN_LEAD + GBX_WIN_TABLES));
+    return smem_attr(gbx_window_kernel<VEC, WE, NT, S, PS, SHIFT, OneOp<CopyDesc>>,
+                     gbx_window_kernel<VEC, WE, NT, S, PS, SHIFT, OpList<CopyDesc>>,
+                     S * (VEC * WE + GBX_WIN_LEAD(SHIFT) + GBX_WIN_TABLES));
+}
+template <int VEC, int WE, bool SHIFT>
+static cudaError_t window_attr_s() {
+    typedef WinShape<VEC * WE> H;
+    cudaError_t e = window_attr_k<VEC, WE, 160, H::S0, H::P0, SHIFT>();
+    if (e == cudaSuccess) e = window_attr_k<VEC, WE, 288, H::S1, H::P1, SHIFT>();
+    if (e == cudaSuccess) e = window_attr_k<VEC, WE, 544, H::S2, H::P2, SHIFT>();
+    return e;
 }
 template <int VEC, int WE>
 static cudaError_t window_attr() {
-    typedef WinShape<VEC * WE> H;
-    cudaError_t e = window_attr_k<VEC, WE, 160, H::S0, H::P0>();
-    if (e == cudaSuccess) e = window_attr_k<VEC, WE, 288, H::S1, H::P1>();
-    if (e == cudaSuccess) e = window_attr_k<VEC, WE, 544, H::S2, H::P2>();
-    return e;
+    const cudaError_t e = window_attr_s<VEC, WE, false>();
+    return e == cudaSuccess ? window_attr_s<VEC, WE, true>() : e;
 }
 
 int gbx_window_prepare(void) {
@@ -1973,7 +1973,7 @@ int gbx_occupancy(int kind, int dtype, int vec, int block, int flat) {
     if (kind == 0 && flat == 8) return 1;   // bulk kernel: one CTA per SM (its ring)
     if (kind == 0 && flat == 9) return scatter_shape(block).per_sm;
     if (kind == 0 && flat >= 10 && flat <= 13) return stream_shape(block).per_sm;
-    if (kind == 0 && (flat & 31) == 15) return window_per_sm(vec, flat >> 5, block);
+    if (kind == 0 && (flat & 31) == 15) return window_per_sm(vec, flat >> 5 & 1, block);
     if (kind == 0 && flat == 14) return agather_per_sm(block);
     if (kind == 0) block = pipe_block(flat, block);
     const void *f = kind == 0 ? (const void *)copy_fn<OneOp<CopyDesc>>(vec, block, flat)
@@ -2000,7 +2000,7 @@ static cudaError_t launch_copy(const L &l, int nops, int vec, int flat, int bloc
         return stream_launch(vec, flat, block, grid, st, dep, l);
     }
     if ((flat & 31) == 15)   // window form: a "tile" is one piece (code 47: the wide windows)
-        return window_launch(vec, flat >> 5, block, grid, st, dep, l);
+        return window_launch(vec, flat, block, grid, st, dep, l);
     if (flat == 14) return agather_launch(block, grid, st, dep, l);   // async gather (vec 16)
     if ((flat == 5 || flat == 7) && nops > 1) flat -= 4;   // the pipelined kernels take one op
     block = pipe_block(flat, block);
