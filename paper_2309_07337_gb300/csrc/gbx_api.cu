@@ -236,10 +236,7 @@ static void set_bulk_dst(HostOp &op) {
 
 // The window form reads its windows with the bulk-copy engine from device memory (every window starts
 // a multiple of 16 bytes into its buffer), with plain loads from host memory.
-static void set_win_lead(CopyDesc &d) {
-    d.win_lead = host_mem(d.src) ? -1 : (int)((uintptr_t)d.src & 15);
-    d.win_lead2 = host_mem(d.src2) ? -1 : (int)((uintptr_t)d.src2 & 15);
-}
+static int win_lead_of(const char *p, bool host) { return host ? -1 : (int)((uintptr_t)p & 15); }
 
 // Elements of the buffer an op's pointer of this role reads.
 static int64_t role_elems(const gbx_request_s *req, int role) {
@@ -261,7 +258,8 @@ static int add_window(gbx_request_s *req, HostOp &op) {
     d.nwin = op.nwin = t.npieces;
     // every window read once, and per element its value written and 2 bytes of index; the tables' other parts
     op.algo_bytes_win = t.window_bytes + d.nelem * (req->elem_size + 2) + d.nelem / 4 + 4 * t.nruns + 32 * t.npieces;
-    set_win_lead(d);
+    d.win_lead = win_lead_of(d.src, host_mem(d.src));
+    d.win_lead2 = win_lead_of(d.src2, host_mem(d.src2));
     return GBX_SUCCESS;
 }
 
@@ -1772,14 +1770,21 @@ extern "C" int gbx_request_bind(gbx_request_t req, const void *src, void *dst) {
     }
     for (HostOp &op : req->ops) {
         if (op.kind == 0) {
-            if (op.cd.src_role == ROLE_SRC) op.cd.src = ns;
-            if (op.cd.dst_role == ROLE_DST) op.cd.dst = nd;
-            set_bulk_dst(op);
-            if (op.win_ok) set_win_lead(op.cd);
+            if (src && op.cd.src_role == ROLE_SRC) {
+                op.cd.src = ns;
+                op.cd.win_lead = win_lead_of(ns, ns_host);
+            }
+            if (dst && op.cd.dst_role == ROLE_DST) {
+                op.cd.dst = nd;
+                op.host_dst = nd_host;
+                op.cd.bulk_dst = !nd_host;
+            }
         } else {
-            if (op.fd.out_role == ROLE_DST) op.fd.out = nd;
-            op.host_dst = host_mem(op.fd.out);
             if (op.fd.a_role == ROLE_SRC) op.fd.bufA = ns;
+            if (dst && op.fd.out_role == ROLE_DST) {
+                op.fd.out = nd;
+                op.host_dst = nd_host;
+            }
         }
     }
     // launches of one op take the new descriptor with their next start; the device descriptors
