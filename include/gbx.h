@@ -219,21 +219,23 @@ int gbx_graph_free(gbx_graph_t *graph);
  *                          bulk-copy engine, scattered to their destinations by the threads
  *       stream=0|1|2       offer the stream form of the flat copies (the per-element index
  *                          arrays copied into shared memory ahead of the payload loads by the
- *                          bulk-copy engine) to the autotuner (default 1; 0 leaves it out, 2
- *                          forces it where it applies: index arrays the library built, vectors
- *                          of at least 4 bytes)
+ *                          bulk-copy engine) to the autotuner (default 1; 0 leaves it out, and the
+ *                          async and window forms with it; 2 forces it where it applies: index
+ *                          arrays the library built, vectors of at least 4 bytes)
  *       form=F             the autotuner times only copy form F (a bit number of copy_forms
  *                          below) in every copy that offers it, the others as usual (default
  *                          -1); for reproducing one program shape, e.g. under a profiler
  *       max_ctas=N         at most N thread blocks in any launch (default 0: no cap), leaving
  *                          the rest of the GPU to other requests' kernels on other streams;
- *                          every move kernel covers its work with any grid
+ *                          every move kernel covers its work with any grid, shapes are tuned
+ *                          under the cap, and a step starts beside the one before it only
+ *                          where all steps' blocks together stay within the cap
  *       check_dup=0|1      locality form: at init, compare the bytes of every element that
  *                          shares a (node pair, global index) value with the value's
  *                          representative in the send buffer as bound then (default 0)
  *       wait_limit=N       polls (N >= 0, default 4194304) of each main wait of the kernels
- *                          that wait on their own asynchronous copies (the bulk-copy and
- *                          scatter forms) before the wait gives up and the start reports
+ *                          that wait on their own asynchronous copies (the bulk, scatter,
+ *                          stream and window forms) before the wait gives up and the start reports
  *                          GBX_ERR_DEVICE_WAIT; waits that drain copies already in flight
  *                          keep the default.  In a batch the first request's limit applies
  * Errors: GBX_ERR_ARG, _TRUNCATE, _INDEX, _GIDX, _OVERLAP (receive blocks must not
@@ -286,8 +288,8 @@ int gbx_neighbor_allgatherv_init(const void *sendbuf, int64_t sendbuf_bytes, con
                                  const char *info, void *stream, gbx_request_t *request);
 
 /* Reads and clears the process-wide status word of the move kernels, the aggregate of every
- * request's own word: 1 when a bounded wait of the bulk or scatter kernel gave up since the
- * last call (the launch then left its pieces unfinished), 2 when one of their pieces failed
+ * request's own word: 1 when a bounded wait of a bulk, scatter, stream or window kernel gave up since
+ * the last call (the launch then left its pieces unfinished), 2 when one of their pieces failed
  * its in-kernel check and was skipped, else 0.  Each request also has its own word, which
  * gbx_wait / gbx_test read (GBX_ERR_DEVICE_WAIT).  No counterpart in the paper. */
 int gbx_device_status(int *status);
@@ -420,8 +422,8 @@ int gbx_backward_init(gbx_request_t forward, const void *grad_recv, void *grad_s
                       gbx_request_t *request);
 
 /* MPIX_Start (section 2.2, Listing 4): enqueues one exchange on the request's stream
- * (one CUDA graph launch, or eager kernel launches when graph=0).  GBX_ERR_ACTIVE if
- * the request was started and not yet completed by wait/test. */
+ * (one launch, or several as one CUDA graph; see the graph key for rebound buffers and graph=0).
+ * GBX_ERR_ACTIVE if the request was started and not yet completed by wait/test. */
 int gbx_start(gbx_request_t request);
 
 /* MPIX_Wait (section 2.2, Listing 4): blocks the host until the started exchange has
@@ -448,7 +450,8 @@ int gbx_wait_stream(gbx_request_t request, void *stream);
 /* Starts `count` inactive requests as one batch: all their move phases run as fused
  * multi-pattern kernels (one launch per dependent phase, every pattern's tiles in the
  * same grid), replayed from one CUDA graph built and cached on the first call for this
- * exact request list (that first call allocates and blocks once).  The batch runs on
+ * exact request list (that first call allocates and blocks once; while some request is bound
+ * to other buffers than then, the launches go out one by one).  The batch runs on
  * requests[0]'s stream; each request completes through gbx_wait/gbx_waitall.  The
  * requests must write disjoint memory. */
 int gbx_startall(int count, gbx_request_t *requests);
@@ -470,11 +473,11 @@ int gbx_request_bind(gbx_request_t request, const void *src, void *dst);
 /* One exchange from `src` into `dst`, in stream order: binds the two for this exchange only (as
  * gbx_request_bind, with its requirements), sets dst to zero bytes first when zero_dst is set,
  * starts the exchange after the work already on `stream` and completes it for `stream` (as
- * gbx_start and gbx_wait_stream); the request's own binding is unchanged, whatever the call returns
- * (except by a captured exchange, graph=0 only, which leaves src and dst bound; with graph=1 a call
- * under a capture gives GBX_ERR_CUDA before anything is bound or enqueued).  One call where a program with new buffers at every step
- * (autograd) would make four.  The caller keeps src and dst alive until the work on `stream`
- * after the call has run. */
+ * gbx_start and gbx_wait_stream); the request's own binding is unchanged, whatever the call
+ * returns (except by a captured exchange, graph=0 only, which leaves src and dst bound; with
+ * graph=1 a call under a capture gives GBX_ERR_CUDA before anything is bound or enqueued).  One
+ * call where a program with new buffers at every step (autograd) would make four.  The caller
+ * keeps src and dst alive until the work on `stream` after the call has run. */
 int gbx_exchange_stream(gbx_request_t request, const void *src, void *dst, int zero_dst, void *stream);
 
 /* One exchange on HOST buffers: copies host_src (the whole bound source buffer, pinned

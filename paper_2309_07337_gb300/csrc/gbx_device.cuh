@@ -69,7 +69,7 @@ struct CopyDesc {
     int64_t nwin;
     int32_t win_elems;            // source elements per window: 1024 or 2048
     int32_t win_lead, win_lead2;  // address of src / src2 modulo 16, or -1: host memory
-    // the waiting kernels (bulk, scatter): the request's status word (host-mapped memory,
+    // the waiting kernels (bulk, scatter, stream, window): the request's status word (host-mapped memory,
     // read by gbx_wait / gbx_test), set to 1 when a bounded wait gave up and 2 when a piece
     // failed its in-kernel check; and the spin limit of their main waits (the waits that
     // drain copies already in flight keep GBX_WAIT_LIMIT)

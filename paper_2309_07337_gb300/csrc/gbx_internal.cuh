@@ -182,7 +182,7 @@ struct LevelLaunch {
     int kind;
     int dtype;              // fold: payload type
     int vec;                // vector width of every op
-    int flat;               // copy: the form of every op; fold: 0, or 1 for the stream form
+    int flat;               // copy: the form of every op; fold: 0, 1 for the stream form, 2 for the window form
     int block;
     int grid;
     int nops;

@@ -1006,8 +1006,10 @@ int gbx_stream_prepare(void) {
 // (32 KB with one chunk per thread at full occupancy).  A warp waits only for copies it has
 // issued itself (cp.async.wait_group), never on a flag.  Bound by HBM: 512^3 stencil halo (64-byte
 // points, 3.57 GB of whole 128-byte lines) 549 us = 6.5 TB/s of line traffic; flat form 543-589 us,
-// stream form 573, register-pipelined form 590-617.  More bytes in flight are not better: the shapes
-// of 64 KB per CTA are fastest at 2-2.5 CTAs per SM (548-551 us), with 3 they take 605 and 624.
+// stream form 573, register-pipelined form 590-617.  More bytes in flight are not better: of the
+// shapes the one of 48 KB per CTA takes 549 us, those of 64 KB 574 and 597 at the 3 CTAs per SM that they
+// are launched with (548 and 550 at 2.4 and 2).  They stay for smaller exchanges, where they are level with it
+// or ahead (256^3 halo 70 us in all three, its locality form 109 and 110, 113 with 48 KB).
 // Chunks of 4 and 8 bytes gain nothing (2^20-row SpMV halo
 // 45 us, stream form 38: a request per line and element bounds them, not bytes in flight).
 // Destinations in host memory (bulk_dst = 0) are stored by the lanes.
@@ -1136,10 +1138,10 @@ int gbx_agather_prepare(void) {
 // bytes and its share of a run instead of 4, every source line is read whole by the copy
 // engine, and no load of a single element goes through L1.  That is what bounds the other forms
 // here: a request to L2 and an L1 line for every scattered element (2^20-row SpMV halo, 10.8 M
-// elements of 8 bytes: L1-to-L2 requests 55 %, DRAM 27 % of peak).  The halo took 39.0 us in the
-// best of them and takes 30.3 (fp32: 28.5 -> 21.0), its locality form 63.5 -> 52.5, a start of 16
-// uneven patterns 115 -> 78; now shared-memory and store wavefronts (54 %) and the 2-CTA ramp
-// weigh most.  Waits bounded as in the stream form.
+// elements of 8 bytes: L1-to-L2 requests 55 %, DRAM 27 % of peak).  Start and wait of the halo took 39.0 us
+// in the best of them and takes 30.3 (fp32, repeated on the same buffers: 30.9 -> 18.6), its locality form
+// 63.5 -> 52.3, a start of 16 uneven patterns 115 -> 80.  Now the requests of short destination runs weigh
+// most, then the producer's work per piece.  Waits bounded as in the stream form.
 // Sources off a 16-byte boundary (SHIFT): a window lies as far from a boundary in its stage as in the
 // source, so that the engine reads all of it but the partial 16-byte units at its ends, which the
 // producer's lanes copy.  2^20-row halo from such a source: 33 us fp64 and 28 fp32, 99 and 89 where
@@ -1676,9 +1678,10 @@ int gbx_sfold_prepare(void) {
 // and end together.  A term costs 2 bytes of place and its share of a run (8 bytes per term in
 // the other forms) and no dependent load.  The other forms are bound by the latency of the chain
 // record -> term -> gradient and by scattered 4- and 8-byte reads; here the phases of 3 or 4
-// blocks per SM overlap, and the longest row's chain of sums weighs most.  Reverse halo of 2^20
-// rows, 10.8 M terms: fp32 41.0 -> 37.0 us, fp64 in node-blocked order 117 -> 87; of 415 k rows
-// fp32 20.5 -> 12.4; of 300 k rows fp64, node-blocked, accumulating 59 -> 42.
+// blocks per SM overlap, and the longest row's chain of sums weighs most.  Starts repeated on the
+// same buffers, before and after: reverse halo of 2^20 rows, 10.8 M terms, fp32 53.4 -> 29.2 us, fp64 in
+// node-blocked order 128 -> 86; of 415 k rows fp32 20.7 -> 12.4; of 300 k rows fp64, node-blocked,
+// accumulating 50.9 -> 27.9 (on changing buffers 59 -> 38).
 // The wait for the tables is bounded as in the other forms.
 #define GBX_WFOLD_TABLES \
     (GBX_WFOLD_N * 2 + GBX_WFOLD_N / 32 * 8 + GBX_WFOLD_RUNS * 4 + GBX_WFOLD_N + GBX_WFOLD_N * 2 + GBX_WFOLD_N / 16 + GBX_WFOLD_N / 8)

@@ -1522,9 +1522,9 @@ int gbx_make_window(gbx_request_s *req, const int32_t *g, int64_t nelem, int64_t
 
 // ------------------------------------------------------------ window form of a fold
 // The rows of a fold of one-chunk elements, cut into pieces: piece p takes the rows whose first
-// term lies in [p * c, (p + 1) * c), c = GBX_WFOLD_N minus 32 times the longest row, so that its
-// rows, sorted by length and laid out in slices of 32, fill at most GBX_WFOLD_N places (a slice
-// is as wide as its longest row, which the shortest row of the slice before it covers).
+// term lies in [p * c, (p + 1) * c).  Sorted by length and laid out in slices of 32, they fill at most
+// GBX_WFOLD_N places as long as c <= GBX_WFOLD_N - 33 * longest row - 32 (a slice is as wide as its longest
+// row, which the shortest row of the slice before it covers); c is less where that leaves blocks idle.
 __global__ void wfold_max_row_kernel(const int64_t *row_ptr, int64_t nrows, unsigned long long *mx) {
     unsigned long long m = 0;
     FOR_EACH(r, nrows) {
@@ -1749,8 +1749,10 @@ int gbx_make_wfold(gbx_request_s *req, FoldDesc *d, int64_t nterms, int64_t *nru
     if (longest < 1 || longest > GBX_WFOLD_ROW) return GBX_SUCCESS;
     // (places: 32 * longest for the first slice, and each other slice no more than the terms of the
     // one before it: in all below 32 * longest + (c + longest))
-    // Fewer terms per piece where full ones would leave some of an SM's blocks without (the 200 k
-    // terms of a 3D stencil's reverse, fp64, node-blocked: 21.2 -> 15.0 us).
+    // Fewer terms per piece, 1024 at least, where full ones would leave some SM with less than three (the
+    // 200 k terms of a 3D stencil's reverse, fp64, node-blocked: 21.2 -> 15.0 us).  Three are what an SM holds
+    // of the fp64 kernel; sized for the four of the fp32 one, fp32 reverse halos of 30 k to 2^20 rows took
+    // 0.97 to 1.03 of the time, with either sign at neighbouring sizes.
     const int64_t c = std::min<int64_t>(GBX_WFOLD_N - 33 * longest - 32,
                                         std::max<int64_t>(1024, ceil_div(nterms, 3ll * gbx_num_sms()))),
                   np = ceil_div(nterms, c);
