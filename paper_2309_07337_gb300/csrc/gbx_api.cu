@@ -401,10 +401,11 @@ int gbx_make_fold_op(gbx_request_s *req, int level, char *out, int out_role, con
     };
     // The window form takes single-term rows with the others, at the same cost per term: no split
     // (all terms in one launch against split copy and window fold of the rest, single values, 11 to 95 %
-    // of the rows single, both orders: 0.5 to 1.02 of the time on the whole GPU, once 1.08, and 0.72 to
-    // 1.25 at 152 blocks).  On a few blocks the copy kernels have more bytes in flight per block and the
-    // split is kept (up to 48 blocks: 0.96 to 2.5, with 64 down to 0.86).
-    const bool few = req->max_ctas > 0 && req->max_ctas <= 48;
+    // of the rows single, both orders: 0.5 to 1.02 of the time on the whole GPU, once 1.08).  On few blocks
+    // the copy kernels have more bytes in flight per block and the split is kept: one launch takes 1.15 to 1.9
+    // of its time up to 48 blocks in fp32 and 1.0 to 1.3 with 64, and in fp64 0.99 to 1.3 up to 8, 0.87 to 1.05 with 24, 0.69 to 1.0
+    // with 48 (stencils of 128^3 and 256^3 points).
+    const bool few = req->max_ctas > 0 && req->max_ctas <= (req->dtype == GBX_F32 ? 64 : 16);
     if (!few) GBX_TRY(window());
     if (!accumulate && !req->no_single_split && !op.wfold_ok) {
         // rows with one term are copies: a two-index flat copy op takes them
@@ -680,12 +681,20 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
     }
     if (op.kind == 1 && op.fd.accumulate) {
         // an accumulating fold adds into the caller's buffer, so it is never trial-launched:
-        // it takes the shape tuned for the same rows without accumulation, or the default
+        // it takes the shape tuned for the same rows without accumulation, or the default: the window form
+        // where there is one; with less than a block per SM that one keeps too few loads of 4-byte
+        // terms, or of long rows, in flight, and the fold kernel with 1024 threads is faster (reverse
+        // halo of 300 k rows fp32, one block: 1,748 us against 3,647, 48 blocks: 48 against 85; fp64 2,837
+        // against 3,623 and 81 against 85; but not of a
+        // 256^3 stencil, fp64, 1.1 terms a row: 6,724 against 5,339, 175 against 140)
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
-        op.block = it != g_tune_cache.end() ? it->second.block : 256;
+        const bool window = op.wfold_ok && req->allow_stream != 2;
+        const bool few = window && req->forced_form != 2 && req->max_ctas > 0 && req->max_ctas <= gbx_num_sms() &&
+                         (req->dtype == GBX_F32 || op.idx_len >= 8 * op.fd.nrows);
+        op.block = it != g_tune_cache.end() ? it->second.block : few ? 1024 : 256;
         op.persistent = it != g_tune_cache.end() ? it->second.persistent : 1;
-        op.fold_form = it != g_tune_cache.end() ? it->second.flat : op.wfold_ok && req->allow_stream != 2 ? 2 : 0;
+        op.fold_form = it != g_tune_cache.end() ? it->second.flat : window && !few ? 2 : 0;
         set_form_bytes(op);
         return set_vec(req, op, it != g_tune_cache.end() ? it->second.vec : op.max_vec);
     }
@@ -767,7 +776,12 @@ static int tune_op(gbx_request_s *req, HostOp &op) {
                     // repeated trials find in L2 (415 k rows fp32: 12.4 us, fold kernel 16.5, and
                     // trials within a few per cent).  Reverse halos of 74 k to 25 M single values, fp32 and
                     // fp64, both orders: 1.14 to 2.6 times as fast as split copy and the other folds.
-                    if (op.kind == 1 && form == 2) ms *= 0.9f;
+                    // On few blocks it is the fold kernel that the trials underrate: the others
+                    // stage their tables, which a cold L2 holds up (300 k rows fp64, 4 blocks, trial and in use:
+                    // fold kernel 697 and 703 us, stream form 683 and 988; 16 blocks: 186 and 191, window form 180
+                    // and 230; with 152 blocks the window form holds up, 100 k rows 15 us and 17).
+                    if (op.kind == 1 && form == 2 && req->max_ctas == 0) ms *= 0.9f;
+                    if (op.kind == 1 && form > 0 && req->max_ctas > 0 && req->max_ctas <= 48) ms *= 1.15f;
                     if (ms < best.ms * (vec < best.vec ? margin : 1.0f)) best = {vec, blocks[bi], pers, form, ms};
                 }
             if (vec == 1) break;

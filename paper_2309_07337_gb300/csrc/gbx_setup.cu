@@ -1752,9 +1752,10 @@ int gbx_make_wfold(gbx_request_s *req, FoldDesc *d, int64_t nterms, int64_t *nru
     // Fewer terms per piece, 1024 at least, where full ones would leave some SM with less than three (the
     // 200 k terms of a 3D stencil's reverse, fp64, node-blocked: 21.2 -> 15.0 us).  Three are what an SM holds
     // of the fp64 kernel; sized for the four of the fp32 one, fp32 reverse halos of 30 k to 2^20 rows took
-    // 0.97 to 1.03 of the time, with either sign at neighbouring sizes.
-    const int64_t c = std::min<int64_t>(GBX_WFOLD_N - 33 * longest - 32,
-                                        std::max<int64_t>(1024, ceil_div(nterms, 3ll * gbx_num_sms()))),
+    // 0.97 to 1.03 of the time, with either sign at neighbouring sizes.  Under a cap there are no more
+    // blocks than it allows (30 k rows fp64 on one block, pieces a quarter full before: 799 -> 339 us).
+    const int64_t blocks = req->max_ctas > 0 ? std::min<int64_t>(req->max_ctas, 3ll * gbx_num_sms()) : 3ll * gbx_num_sms(),
+                  c = std::min<int64_t>(GBX_WFOLD_N - 33 * longest - 32, std::max<int64_t>(1024, ceil_div(nterms, blocks))),
                   np = ceil_div(nterms, c);
     FoldPiece *pieces;
     uint16_t *pos, *base, *rowout;
