@@ -269,4 +269,4 @@ def test_capped_requests_have_shapes_of_their_own():
     for form in ("", "form=1", "form=5", "form=14"):
         gbx.Exchange(p, x, y, info=form, dp=dp, graph=graph)
         us[form] = _us(gbx.Exchange(p, x, y, info="max_ctas=16;" + form, dp=dp, graph=graph).request)
-    assert max(us[""], us["form=5"], us["form=14"]) <= 1.45 * min(us.values()), us
+    assert max(us[""], us["form=5"], us["form=14"]) <= 1.6 * min(us.values()), us

@@ -105,9 +105,15 @@ def test_rebind_and_batch(s):
 def _kernels(fn):
     """Names of the kernels that run in fn ([] where the profiler records none)."""
     from torch.profiler import ProfilerActivity, profile
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+    prof = profile(activities=[ProfilerActivity.CUDA])
+    try:
+        prof.start()
+    except RuntimeError:     # (another profiler holds the device)
         fn()
-        torch.cuda.synchronize()
+        return []
+    fn()
+    torch.cuda.synchronize()
+    prof.stop()
     return [e.name for e in prof.events() if "gbx_" in e.name]
 
 
@@ -292,9 +298,9 @@ def test_too_little_memory_for_the_tables(what):
         return gbx.backward_init(fwd.request, grad, gx, accumulate=True, info=info)
 
     bit = 1 << (15 if what == "forward" else 13)
-    for info in ("stream=0", "form=15" if what == "forward" else "form=2"):   # (loads the kernels)
+    for info in ("", "stream=0", "form=15" if what == "forward" else "form=2"):   # (loads the kernels)
         r = make(info)
-        assert bool(r.info()["copy_forms"] & bit) == (info != "stream=0")
+        assert info == "" or bool(r.info()["copy_forms"] & bit) == (info != "stream=0")
         r.free()
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
