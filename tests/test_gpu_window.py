@@ -282,6 +282,40 @@ def test_time_into_host_memory():
     assert max(us[:2]) <= 1.3 * us[2] and max(us[3:5]) <= 1.3 * us[5], us
 
 
+@pytest.mark.parametrize("captured", ["aligned", "off", "host"])
+def test_replays_after_a_rebind(captured):
+    """graph=0: a caller's graph keeps the kernel that suited the buffers bound when it was captured, and
+    reads the descriptors of those bound now: aligned, off a 16-byte boundary, into host memory."""
+    import gc
+    gc.collect()
+    p = ring(16, 1500, 999, 8, 3)
+    x = pt.random_bytes(p.sendbuf_bytes, 5)
+    want = oracle.standard(p, x)
+    room = torch.zeros(p.sendbuf_bytes + 8, dtype=torch.uint8, device="cuda")
+    room[8:].copy_(dev_bytes(x))
+    dev, host = torch.zeros(p.recvbuf_bytes, dtype=torch.uint8, device="cuda"), _host(p.recvbuf_bytes)
+    bound = {"aligned": (dev_bytes(x), dev), "off": (room[8:], dev), "host": (room[8:], host)}
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ex = gbx.Exchange(p, dev_bytes(x), dev, info="form=15;graph=0", stream=s)
+    assert ex.info()["copy_forms"] & FORM
+    ex.request.bind(*bound[captured])
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        ex.start()
+        ex.request.wait_stream(s)
+    for now in ("aligned", "off", "host", captured):
+        ex.request.bind(*bound[now])
+        out = bound[now][1]
+        out.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s):
+            g.replay()
+        torch.cuda.synchronize()
+        assert_bytes_equal(out.cpu().numpy(), want, f"captured {captured}, bound {now}")
+
+
 @pytest.mark.parametrize("what", ["forward", "backward"])
 def test_too_little_memory_for_the_tables(what):
     """With just the memory that a request needs without window forms it is built without them."""
